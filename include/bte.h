@@ -160,7 +160,15 @@ typedef struct {
                             232,448 bytes, or the G clusters do not fit the
                             GPU at once (small grids: 31 x 201 FP64 runs
                             5.5 instead of 16.1 us per step on a GB300).
-                            0: one fused step kernel launch per step.      */
+                            0: with every field of this struct zero, a
+                            grid that fits the shared memory of the SMs
+                            together runs there in calls of four steps or
+                            more, cut into one block per SM, one
+                            cooperative launch per up to 4096 steps whose
+                            CTAs exchange their blocks' edges through
+                            global memory (bounded waits: BTE_ETIMEOUT);
+                            otherwise one fused step kernel launch per
+                            step.  Both give the same bits.                */
     int32_t walk;        /* order in which one-step launches walk the
                             harmonic rows of a work item: 0 automatic
                             (alternate when the ping-pong state exceeds 96

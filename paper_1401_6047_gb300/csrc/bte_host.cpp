@@ -192,7 +192,79 @@ struct Layout {
     size_t wide_smem;
     size_t off_wx, off_wpart;  /* tagged edge-column words, per-cluster sums */
     size_t wide_words;         /* bytes of the tagged words */
+    /* on chip, one block per SM (blkGR = 0: the grid does not fit): blkGR x
+     * blkGC blocks of blkR rows x blkW columns, blkV columns per thread */
+    int blkGR, blkGC, blkR, blkW, blkV, blk_threads;
+    size_t blk_smem, blk_words; /* shared memory per CTA; bytes of exchange words */
+    int blk_steps, blk_mpad;    /* steps per launch at most; pitch of the kept rows */
+    size_t off_blkx, off_blkq, off_blkrows;
 };
+
+/* On chip, one block per SM: CTAs (the SMs of a GB300), bytes of kept rows
+ * per launch (half the state's, within these limits: launches of 240 steps
+ * or more, so that the 12 to 25 us a launch costs beyond its steps stay near
+ * one per cent), and the fewest steps of a call for which the launch, the
+ * load of the blocks and the fold are worth it. */
+constexpr int kBlkCtas = 152;
+constexpr size_t kBlkSmemMax = 232448;
+constexpr size_t kBlkRowBytesMin = 2u << 20, kBlkRowBytesMax = 16u << 20;
+constexpr int kBlkMaxSteps = 4096;
+constexpr int kBlkMinSteps = 4;
+
+/* Blocks of the on-chip mode of one block per SM: of all row splits GR and
+ * the two column-group widths V, the one with the least estimated time of a
+ * half-step in cycles.  The interior cells run while the neighbours' edges
+ * are under way (about 1100 cycles from a store to its poll), the boundary
+ * cells after them.  FP32: a pass over one group per thread takes about 700
+ * cycles, and 166 (V = 4) or 100 (V = 2) issue slots per warp and row.  FP64:
+ * a warp's pass takes about 3300 cycles per column, however many of its
+ * lanes hold a cell, and one of four warps runs at a time on each quarter of
+ * an SM.  Measured on a GB300 (us per step, this choice / best of a sweep of
+ * 13 row splits, both widths and 64 to 512 threads): 31 x 201 FP64 4.5 /
+ * 4.4, FP32 2.0 / 1.9; 138 x 1533 FP32 3.6 / 3.6; 120 x 4000 FP32 4.5 / 4.5;
+ * 401 x 4001 FP32 7.5 / 7.5; 65 x 1000 FP64 11.9 / 11.9.  False when no
+ * split fits the shared memory. */
+bool pick_blocks(int N1, int M1, size_t elem, Layout& L) {
+    double best = 1e30;
+    for (int V = elem == 8 ? 1 : 2; V <= (elem == 8 ? 2 : 4); V *= 2)
+        for (int gr = 1; gr <= std::min(N1, kBlkCtas); ++gr) {
+            const int R = (N1 + gr - 1) / gr, GR = (N1 + R - 1) / R;
+            if (GR != gr) continue;
+            const int gc = kBlkCtas / GR;
+            const int W = ((M1 + gc - 1) / gc + V - 1) / V * V, GC = (M1 + W - 1) / W;
+            const size_t smem = elem == 8 ? bte::grid_smem_bytes<double>(R, W, V) : bte::grid_smem_bytes<float>(R, W, V);
+            if (smem > kBlkSmemMax) continue;
+            const int ncg = W / V, nci = std::max(ncg - 2, 0), nri = std::max(R - 2, 0);
+            const int ni = nci * nri, nb = (R >= 2 ? 2 : 1) * ncg + (ncg >= 2 ? 2 : 1) * nri;
+            const int nq = 2 * (W + 2) + 2 * R;
+            int thr = std::max((ni / 3 + 127) / 128 * 128, (std::max(nb, nq / 2) + 31) / 32 * 32);
+            thr = std::min(std::max(thr, 64), bte::kGridThreads);
+            double t_int = 0.0, t_bnd;
+            if (elem == 8) {
+                t_int = ni ? 3300.0 * V * std::max(1.0, ni / 128.0) : 0.0;
+                t_bnd = 3300.0 * V * std::max(1.0, nb / 128.0);
+            } else {
+                if (ni) {
+                    const int cpp = std::min(nci, thr), split = thr / cpp;
+                    const int rows = (nri + split - 1) / split, passes = (nci + cpp - 1) / cpp;
+                    t_int = std::max(330.0 * passes * (rows + 2), ni * (V == 4 ? 1.3 : 0.8));
+                }
+                t_bnd = (nb + thr - 1) / thr * 700.0 + 2.0 * nb;
+            }
+            const double t = std::max(t_int, 1100.0) + t_bnd + 0.5 * nq;
+            if (t < best) {
+                best = t;
+                L.blkGR = GR;
+                L.blkGC = GC;
+                L.blkR = R;
+                L.blkW = W;
+                L.blkV = V;
+                L.blk_smem = smem;
+                L.blk_threads = thr;
+            }
+        }
+    return best < 1e30;
+}
 
 /* steps of one persistent launch at most (a bte_step/bte_run call of more
  * steps queues several launches) */
@@ -358,6 +430,24 @@ int plan(const bte_params* p, const bte_tuning* t, const TimeGrid& tg, Layout& L
         L.off_wpart = o;
         o += align_up((size_t)kPersistMaxSteps * L.wideG * 2 * sizeof(double), 256);
     }
+    /* one block per SM, where the launch shape is left to the library */
+    L.blkGR = 0;
+    const bool shaped = t && (t->tile_m || t->chunk_n || t->graph_steps || t->vec || t->walk);
+    if (!shaped && pick_blocks(N1, M1, L.elem, L)) {
+        L.blk_mpad = (int)align_up(M1, 32);
+        const size_t row_bytes = 2 * (size_t)L.blk_mpad * L.elem;
+        const size_t keep = std::min(std::max(4 * arr, kBlkRowBytesMin), kBlkRowBytesMax);
+        const long long steps = std::min<long long>(keep / row_bytes, kBlkMaxSteps);
+        L.blk_steps = (int)std::max<long long>(std::min(steps, tg.K), 1);
+        /* 2 buffers x 2 grids x 2 sides, 16 bytes per FP32 cell, 32 per FP64 */
+        L.blk_words = (size_t)8 * ((size_t)L.blkGR * M1 + (size_t)L.blkGC * N1) * 4 * L.elem;
+        L.off_blkx = o;
+        o += align_up(L.blk_words, 256);
+        L.off_blkq = o; /* cleared together with the words */
+        o += 256;
+        L.off_blkrows = o;
+        o += align_up((size_t)L.blk_steps * row_bytes, 256);
+    }
     L.total = o;
     return BTE_OK;
 }
@@ -379,6 +469,7 @@ struct bte_handle {
     int graph_len; /* steps per captured graph (a multiple of the fused step count) */
     int grid[3];   /* persistent CTAs of the step kernel fusing 1 / 2 steps */
     int grid_persist; /* CTAs of a persistent (multi-step) launch, all co-resident */
+    bool blk;      /* calls of kBlkMinSteps steps or more run on chip, one block per SM */
     int set;       /* ping-pong set holding the current state (flips per launch) */
     cudaGraphExec_t graph[2]; /* one graph per starting set */
     double r1;     /* I_1/I_0 */
@@ -743,8 +834,64 @@ int enqueue_persist(bte_handle* h, long long n) {
     return BTE_OK;
 }
 
+/* On chip, one block per SM: launches of at most blk_steps steps, each one
+ * cooperative launch that advances the current ping-pong set in place (its
+ * exchange words and quit word zeroed before it), then the sums of the rows
+ * it kept. */
+template <typename T>
+int enqueue_blocks(bte_handle* h, long long n) {
+    const Layout& L = h->L;
+    const int set = h->set;
+    const bte::StepArgs<T> sa = step_args<T>(h);
+    bte::GridArgs<T> g{};
+    g.a_w = sa.a_w[set];
+    g.b_w = sa.b_w[set];
+    g.a_f = sa.a_f[set];
+    g.b_f = sa.b_f[set];
+    g.row_a0 = sa.row_a0;
+    g.col_g = sa.col_g;
+    g.col_phi = sa.col_phi;
+    g.e_whole = sa.e_whole;
+    g.e_frac = sa.e_frac;
+    g.rowx = h->mem + L.off_blkx;
+    g.colx = h->mem + L.off_blkx + (size_t)8 * L.blkGR * h->p.m_points * 4 * L.elem;
+    g.rows = h->ptr<T>(L.off_blkrows);
+    g.err = sa.err;
+    g.quit = h->ptr<int>(L.off_blkq);
+    g.base = sa.base;
+    g.N = sa.N;
+    g.M = sa.M;
+    g.pitch = sa.pitch;
+    g.P = sa.P;
+    g.dstride = sa.dstride;
+    g.GR = L.blkGR;
+    g.GC = L.blkGC;
+    g.R = L.blkR;
+    g.W = L.blkW;
+    g.mpad = L.blk_mpad;
+    g.h = sa.h;
+    g.hh = sa.hh;
+    g.nu = sa.nu;
+    g.xi = sa.xi;
+    while (n > 0) {
+        const int c = (int)std::min<long long>(n, L.blk_steps);
+        g.K = c;
+        CU(cudaMemsetAsync(g.rowx, 0, L.off_blkq + 256 - L.off_blkx, h->stream));
+        int rc = bte::launch_grid<T>(g, L.blkV, L.blk_threads, L.blk_smem, h->stream);
+        if (!rc)
+            rc = bte::launch_fold_rows<T>(g.rows, g.mpad, g.M, L.tile_m, L.vec, c, sa.vscale, sa.nscale, g.base,
+                                          sa.trace_v, sa.trace_n, h->stream);
+        if (!rc) rc = bte::launch_advance_base(h->ptr<long long>(L.off_base), c, h->stream);
+        if (rc) return fail(BTE_ECUDA, "on-chip step kernel: %s", cudaGetErrorString((cudaError_t)rc));
+        h->k += c;
+        n -= c;
+    }
+    return BTE_OK;
+}
+
 template <typename T>
 int enqueue_steps(bte_handle* h, long long n) {
+    if (h->blk && n >= kBlkMinSteps) return enqueue_blocks<T>(h, n);
     if (h->L.resC) return n > 0 ? enqueue_resident<T>(h, n) : BTE_OK;
     if (h->L.wideG) return n > 0 ? enqueue_wide<T>(h, n) : BTE_OK;
     if (h->L.persist) return enqueue_persist<T>(h, n);
@@ -1616,6 +1763,18 @@ int bte_create_ex(const bte_params* p, void* stream, const bte_tuning* tune, voi
                                  items, cap));
             h->grid_persist = (int)items;
         }
+    }
+    h->blk = false;
+    if (h->L.blkGR && !h->L.resC && !h->L.wideG && !h->L.persist) {
+        /* every block must be resident at once */
+        int bps = 0, dev = 0, sms = 0, coop = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+        rc = h->fp64 ? bte::grid_configure<double>(h->L.blkV, h->L.blk_smem, h->L.blk_threads, &bps)
+                     : bte::grid_configure<float>(h->L.blkV, h->L.blk_smem, h->L.blk_threads, &bps);
+        if (rc) return bail(fail(BTE_ECUDA, "on-chip kernel configure: %s", cudaGetErrorString((cudaError_t)rc)));
+        h->blk = coop && (long long)bps * sms >= (long long)h->L.blkGR * h->L.blkGC;
     }
     if (h->L.resC) {
         /* sets the on-chip kernel's shared-memory (and cluster-size) attributes */

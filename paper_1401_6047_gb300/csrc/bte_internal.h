@@ -164,6 +164,31 @@ struct WideArgs {
     T h, hh, nu, xi;
 };
 
+/* threads per CTA of the on-chip kernel of one block per SM, at most */
+constexpr int kGridThreads = 512;
+
+/* Arguments of the single-instance on-chip kernel of one block per SM
+ * (bte_grid.cu): GR x GC blocks of R rows x W columns, advanced in place
+ * (one ping-pong set). */
+template <typename T>
+struct GridArgs {
+    T* a_w; T* b_w; T* a_f; T* b_f;    /* state, rows `pitch` elements apart     */
+    const T* row_a0; const T* col_g; const T* col_phi;
+    const T* e_whole; const T* e_frac; /* drive tables as in StepArgs           */
+    void* rowx;       /* exchange words [2 buffers][2 grids][GR][first, last row][M+1],
+                         zeroed by the caller before the launch; an entry is a
+                         and b as 32-bit parts, each under its half-step's number */
+    void* colx;       /* the same, [2][2][GC][first, last column][N+1]          */
+    T* rows;          /* [K][2][mpad] rows 0 (a) and 1 (b) of each new whole grid */
+    int* err;         /* error word: kErrTimeout when a wait gave up           */
+    int* quit;        /* set when a wait of this launch gave up (zeroed before it) */
+    const long long* base; /* step counter: the launch advances steps base ..   */
+    int K;            /* steps of this launch                                  */
+    int N, M, pitch, P, dstride;
+    int GR, GC, R, W, mpad;
+    T h, hh, nu, xi;
+};
+
 /* One plain application of T (start-up half step), unfused. */
 template <typename T>
 struct ApplyArgs {
@@ -247,6 +272,19 @@ template <typename T>
 int launch_wide(const WideArgs<T>& a, int threads, size_t smem, void* stream);
 int launch_wide_fold(const double* part, int G, long long K, long long k0, double vscale,
                      double nscale, double* trace_v, double* trace_n, void* stream);
+/* On-chip kernel of one block per SM: shared memory of one CTA, CTAs that
+ * fit an SM (sets the kernel's attributes), launch, and the sums of the
+ * rows it kept of K steps, written to trace[*base + 1 ..]. */
+template <typename T>
+size_t grid_smem_bytes(int R, int W, int vec);
+template <typename T>
+int grid_configure(int vec, size_t smem, int threads, int* blocks_per_sm);
+template <typename T>
+int launch_grid(const GridArgs<T>& a, int vec, int threads, size_t smem, void* stream);
+template <typename T>
+int launch_fold_rows(const T* rows, int mpad, int M, int tile_m, int vec, int K, double vscale,
+                     double nscale, const long long* base, double* trace_v, double* trace_n,
+                     void* stream);
 /* Sets the calling thread's bte_last_error() message; returns code. */
 int report_error(int code, const char* msg);
 template <typename T>
