@@ -99,10 +99,13 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-/* 1/x for the Crank-Nicolson denominator D = nu^2 + theta'^2 >= 1: the
- * hardware approximate reciprocal in FP32 (PTX rcp.approx.ftz.f32, about one
- * ulp; D is never subnormal, zero or infinite), the correctly rounded
- * division in FP64. */
+/* 1/x for the Crank-Nicolson denominator D >= 1 (never subnormal or zero):
+ * in FP32 the hardware approximate reciprocal (PTX rcp.approx.ftz.f32, about
+ * one ulp); in FP64 the hardware seed (rcp.approx.ftz.f64, 2^-23) and one
+ * third-order Newton step x (1 + e + e^2), e = 1 - D x, which leaves e^3 <
+ * 2^-68 and the roundings (the whole update stays as near the 64-bit
+ * oracle as with the division).  It
+ * takes 3 of the FP64 pipe's slots where the division takes about 7. */
 template <typename T>
 __device__ __forceinline__ T recip(T x);
 template <>
@@ -113,7 +116,10 @@ __device__ __forceinline__ float recip<float>(float x) {
 }
 template <>
 __device__ __forceinline__ double recip<double>(double x) {
-    return 1.0 / x;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = __fma_rn(-x, r, 1.0);
+    return __fma_rn(r, __fma_rn(e, e, e), r);
 }
 
 /* Arithmetic with exactly one rounding per operation and no contraction
@@ -139,7 +145,9 @@ struct Rn<double> {
 };
 
 /* Constants of the Crank-Nicolson operator T_h (Sec. 3): nu = 1 + h/2,
- * xi = 1 - h/2 and the products nu^2, nu h. */
+ * xi = 1 - h/2 and the products nu^2, nu h.  FP64 kernels work with the
+ * equations divided by nu: h here is h/nu, as the rotation factors (hh) and
+ * the stencil coefficients they are given are divided by nu. */
 template <typename T>
 struct CnK {
     T h, nu, xi, nu2, nuh;
@@ -157,15 +165,16 @@ __device__ __forceinline__ T rot_factor(T E, T B, T phi, T hh) {
 }
 
 /* The paper's stencil terms from central differences D x_r(m) of the other
- * grid: B^t = c (D b_{n+1} - D b_{n-1}) acts on a, A^t = c (chi(n) D a_{n-1}
- * - D a_{n+1}) on b (chi(1) = 2: the n = 1 row reads a_0 twice, Sec. 3). */
+ * grid, without their coefficient c: B^t = c (D b_{n+1} - D b_{n-1}) acts on
+ * a, A^t = c (chi(n) D a_{n-1} - D a_{n+1}) on b (chi(1) = 2: the n = 1 row
+ * reads a_0 twice, Sec. 3). */
 template <typename T>
-__device__ __forceinline__ T stencil_a(T c, T db_next, T db_prev) {
-    return Rn<T>::mul(c, Rn<T>::sub(db_next, db_prev));
+__device__ __forceinline__ T stencil_a(T db_next, T db_prev) {
+    return Rn<T>::sub(db_next, db_prev);
 }
 template <typename T>
-__device__ __forceinline__ T stencil_b(T c, T chi, T da_prev, T da_next) {
-    return Rn<T>::mul(c, Rn<T>::fma(chi, da_prev, -da_next));
+__device__ __forceinline__ T stencil_b(T chi, T da_prev, T da_next) {
+    return Rn<T>::fma(chi, da_prev, -da_next);
 }
 
 /* Crank-Nicolson update of one cell (Sec. 3, Eqs. a_t_plus_1, b_t_plus_1,
@@ -178,11 +187,21 @@ __device__ __forceinline__ T stencil_b(T c, T chi, T da_prev, T da_next) {
  * g = a xi - b th + Sa + h a0, q = b xi + a th + Sb.  Sa is the paper's B^t
  * stencil term (acts on a), Sb its A^t term (acts on b); h a0 = hr g with
  * hr = h times the row factor and g the column factor of the separable
- * equilibrium.  Each product, sum and fused multiply-add below is one
- * rounding, in this order. */
+ * equilibrium.
+ *
+ * FP64, bound by its pipe (about 1.9 operations per clock and SM), uses the
+ * form with the fewest operations: with every coefficient divided by nu, s =
+ * th + th1 (the sum is the first rotation factor, w0, that FP64 callers pass)
+ * and
+ *   G = Sa + h a0 - h a - s b,   H = Sb - h b + s a,   D = 1 + th1^2,
+ *   da = (G - th1 H) / D,        db = (th1 G + H) / D,
+ * 21 FP64 operations per cell and half-step with the reciprocal, where the
+ * coefficients of a and b taken apart need 33 and a division (401 x 4001, one
+ * launch per step: 226 -> 172 us).  Each product, sum and fused multiply-add below
+ * is one rounding, in this order. */
 template <typename T>
 struct CnCoef {
-    T th1, inv, ca, cb;
+    T th1, inv, ca, cb; /* FP64: ca holds s, cb is not used */
 };
 /* The part of the update that depends on the cell's (n, m) and the drive
  * only, not on the state: 1/D and the two coefficients of a and b. */
@@ -191,37 +210,66 @@ __device__ __forceinline__ CnCoef<T> cn_coef(T th, T th1, const CnK<T>& k) {
     using O = Rn<T>;
     CnCoef<T> c;
     c.th1 = th1;
-    const T D = O::fma(th1, th1, k.nu2);
-    c.inv = recip<T>(D);
-    c.ca = O::fma(th1, O::add(th, th1), k.nuh);
-    c.cb = O::fma(k.xi, th1, O::mul(th, k.nu));
+    if constexpr (sizeof(T) == 8) {
+        c.inv = recip<T>(O::fma(th1, th1, (T)1));
+        c.ca = th;
+        c.cb = (T)0;
+    } else {
+        const T D = O::fma(th1, th1, k.nu2);
+        c.inv = recip<T>(D);
+        c.ca = O::fma(th1, O::add(th, th1), k.nuh);
+        c.cb = O::fma(k.xi, th1, O::mul(th, k.nu));
+    }
     return c;
 }
-/* The rest: the new a, b from the old ones and the stencil terms. */
+/* FP64: the part of G and H that needs only the cell's own values, and the
+ * rest, from the stencil sums X = stencil_a, Y = stencil_b and their
+ * coefficient cc */
+__device__ __forceinline__ void cn_own(double a, double b, double hr, double g, const CnCoef<double>& c,
+                                       const CnK<double>& k, double& G0, double& H0) {
+    using O = Rn<double>;
+    G0 = O::fma(hr, g, O::fma(-k.h, a, -O::mul(c.ca, b)));
+    H0 = O::fma(-k.h, b, O::mul(c.ca, a));
+}
+__device__ __forceinline__ void cn_finish(double a, double b, double X, double Y, double cc, double G0,
+                                          double H0, const CnCoef<double>& c, double& an, double& bn) {
+    using O = Rn<double>;
+    const double G = O::fma(cc, X, G0), H = O::fma(cc, Y, H0);
+    an = O::fma(O::fma(-c.th1, H, G), c.inv, a);
+    bn = O::fma(O::fma(c.th1, G, H), c.inv, b);
+}
+/* The rest: the new a, b from the old ones and the stencil sums. */
 template <typename T>
-__device__ __forceinline__ void cn_update(T a, T b, T Sa, T Sb, T hr, T g, const CnCoef<T>& c,
+__device__ __forceinline__ void cn_update(T a, T b, T X, T Y, T cc, T hr, T g, const CnCoef<T>& c,
                                           const CnK<T>& k, T& an, T& bn) {
     using O = Rn<T>;
-    const T src = O::fma(hr, g, Sa);
-    T t = O::fma(k.nu, src, -O::mul(c.th1, Sb));
-    t = O::fma(-a, c.ca, t);
-    t = O::fma(-b, c.cb, t);
-    T u = O::fma(c.th1, src, O::mul(k.nu, Sb));
-    u = O::fma(a, c.cb, u);
-    u = O::fma(-b, c.ca, u);
-    an = O::add(a, O::mul(t, c.inv));
-    bn = O::add(b, O::mul(u, c.inv));
+    if constexpr (sizeof(T) == 8) {
+        T G0, H0;
+        cn_own(a, b, hr, g, c, k, G0, H0);
+        cn_finish(a, b, X, Y, cc, G0, H0, c, an, bn);
+    } else {
+        const T Sa = O::mul(cc, X), Sb = O::mul(cc, Y);
+        const T src = O::fma(hr, g, Sa);
+        T t = O::fma(k.nu, src, -O::mul(c.th1, Sb));
+        t = O::fma(-a, c.ca, t);
+        t = O::fma(-b, c.cb, t);
+        T u = O::fma(c.th1, src, O::mul(k.nu, Sb));
+        u = O::fma(a, c.cb, u);
+        u = O::fma(-b, c.ca, u);
+        an = O::add(a, O::mul(t, c.inv));
+        bn = O::add(b, O::mul(u, c.inv));
+    }
 }
 template <typename T>
-__device__ __forceinline__ void cn_cell(T a, T b, T Sa, T Sb, T hr, T g, T th, T th1,
+__device__ __forceinline__ void cn_cell(T a, T b, T X, T Y, T cc, T hr, T g, T th, T th1,
                                         const CnK<T>& k, T& an, T& bn) {
-    cn_update<T>(a, b, Sa, Sb, hr, g, cn_coef<T>(th, th1, k), k, an, bn);
+    cn_update<T>(a, b, X, Y, cc, hr, g, cn_coef<T>(th, th1, k), k, an, bn);
 }
 
 /* The update of V consecutive columns of one row (V = 2 or 4): the stencil
  * terms from the other grid's differences in rows n+1 (next) and n-1 (prev),
- * the rotations n w0, n w1 (w = rot_factor at the half-step's start and end)
- * and cn_cell.  FP32 runs two columns per instruction with Blackwell's paired
+ * the rotations n w0, n w1 (w = rot_factor at the half-step's start and end;
+ * FP64: w0 the sum of the two) and cn_cell.  FP32 runs two columns per instruction with Blackwell's paired
  * FP32 operations (__ffma2_rn, __fadd2_rn, __fmul2_rn), which round each
  * component exactly as the scalar _rn form: the same bits as cn_cell on
  * each column, in half the issue slots.  FP64 runs cn_cell per column. */
@@ -269,8 +317,8 @@ __device__ __forceinline__ void cn_row(const T (&a)[V], const T (&b)[V], const T
         using O = Rn<T>;
 #pragma unroll
         for (int e = 0; e < V; ++e)
-            cn_cell<T>(a[e], b[e], stencil_a<T>(cc, db_next[e], db_prev[e]),
-                       stencil_b<T>(cc, chi, da_prev[e], da_next[e]), hr, g[e],
+            cn_cell<T>(a[e], b[e], stencil_a<T>(db_next[e], db_prev[e]),
+                       stencil_b<T>(chi, da_prev[e], da_next[e]), cc, hr, g[e],
                        O::mul(nf, w0[e]), O::mul(nf, w1[e]), k, an[e], bn[e]);
     }
 }
@@ -297,9 +345,11 @@ __device__ __forceinline__ void st_release(unsigned* p, unsigned v) {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-/* Drive of one half-step: E and B at its start (E0, B0) and end (E1, B1),
- * and its stencil coefficient, read from a [3][stride] drive table (E, B,
- * coefficient; FP64 values rounded to T once on the host) at row kk. */
+/* Drive of one half-step: E and B at its start (E0, B0; FP64: the sums of
+ * the values at its start and end) and end (E1, B1), and its stencil
+ * coefficient, read from a [kDriveRows][stride] drive table (E, B,
+ * coefficient, and in FP64 the sums; computed in FP64 and rounded to T once
+ * on the host) at row kk. */
 template <typename T>
 struct Half {
     T E0, E1, B0, B1, cc;
@@ -307,9 +357,9 @@ struct Half {
 template <typename T>
 __device__ __forceinline__ Half<T> half_drive(const T* tab, int stride, int kk) {
     Half<T> d;
-    d.E0 = tab[kk];
+    d.E0 = tab[(sizeof(T) == 8 ? 3 * stride : 0) + kk];
     d.E1 = tab[kk + 1];
-    d.B0 = tab[stride + kk];
+    d.B0 = tab[(sizeof(T) == 8 ? 4 * stride : stride) + kk];
     d.B1 = tab[stride + kk + 1];
     d.cc = tab[2 * stride + kk];
     return d;

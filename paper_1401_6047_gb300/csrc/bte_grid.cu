@@ -20,7 +20,7 @@
  * exchange of edges per half-step, about 0.5 us through L2.
  *
  * Measured (GB300, us per step, one launch per step / here): 31 x 201 FP64
- * 29.2 / 4.5, FP32 9.3 / 2.0; 65 x 1000 FP64 65 / 12; 138 x 1533 FP32 14.4 /
+ * 23.0 / 3.9, FP32 9.3 / 2.0; 65 x 1000 FP64 45 / 9.4; 138 x 1533 FP32 14.4 /
  * 3.6; 120 x 4000 FP32 13.9 / 4.5; 401 x 4001 FP32 17.0 / 7.5.
  *
  * A half-step of a CTA:
@@ -170,6 +170,7 @@ __host__ __device__ inline size_t poll_offset(int R, int W, int V) {
 
 template <typename T, int V>
 __global__ void __launch_bounds__(kGridThreads, 1) grid_kernel(GridArgs<T> A) {
+    static_assert(sizeof(T) == 4 || V == 1, "FP64 takes one column per thread");
     constexpr int GG = Cols<T>::G;            /* global ghost columns before m = 0 */
     constexpr int E = sizeof(T) / 4;          /* word pairs per exchange entry */
     extern __shared__ __align__(16) unsigned char smem[];
@@ -366,6 +367,20 @@ __global__ void __launch_bounds__(kGridThreads, 1) grid_kernel(GridArgs<T> A) {
                 if (l1 < R) out[A.mpad + q] = s[arr + (l1 + 1) * P + V + q];
             }
         }
+        /* FP64: the part of the first boundary cell's update that needs no
+         * halo, while the edges are under way (15 of its 27 operations) */
+        CnCoef<T> pre{};
+        T preG = (T)0, preH = (T)0;
+        auto own_part = [&](int il, int m, CnCoef<T>& c, T& G0, T& H0) {
+            if constexpr (sizeof(T) == 8) {
+                const T nf = (T)(r0 + il), ph = sPh[V + m];
+                c = cn_coef<T>(Rn<T>::mul(nf, rot_factor<T>(D.E0, D.B0, ph, hh)),
+                               Rn<T>::mul(nf, rot_factor<T>(D.E1, D.B1, ph, hh)), cn);
+                const T* const po = so + (il + 1) * P + m;
+                cn_own(po[0], po[arr], sR[il + 1], sG[V + m], c, cn, G0, H0);
+            }
+        };
+        if (sizeof(T) == 8 && tid < nb) own_part((int)(sBnd[tid] >> 16), (int)(sBnd[tid] & 0xffffu), pre, preG, preH);
         /* the halo cells of the grid that is read (loaded with the block for
          * the first half-step) */
         bool ok = true;
@@ -431,16 +446,22 @@ __global__ void __launch_bounds__(kGridThreads, 1) grid_kernel(GridArgs<T> A) {
                 T* const po = so + (il + 1) * P + m;
                 ldv<T, V>(po, oa);
                 ldv<T, V>(po + arr, ob);
-                T gc[V], ph[V], t0[V], t1[V];
-                ldv<T, V>(sG + V + m, gc);
-                ldv<T, V>(sPh + V + m, ph);
+                if constexpr (sizeof(T) == 8) {
+                    if (u != tid) own_part(il, m, pre, preG, preH);
+                    cn_finish(oa[0], ob[0], stencil_a<T>(db_d[0], db_u[0]),
+                              stencil_b<T>(n == 1 ? (T)2 : (T)1, da_u[0], da_d[0]), D.cc, preG, preH, pre, an[0], bn[0]);
+                } else {
+                    T gc[V], ph[V], t0[V], t1[V];
+                    ldv<T, V>(sG + V + m, gc);
+                    ldv<T, V>(sPh + V + m, ph);
 #pragma unroll
-                for (int e = 0; e < V; ++e) {
-                    t0[e] = rot_factor<T>(D.E0, D.B0, ph[e], hh);
-                    t1[e] = rot_factor<T>(D.E1, D.B1, ph[e], hh);
+                    for (int e = 0; e < V; ++e) {
+                        t0[e] = rot_factor<T>(D.E0, D.B0, ph[e], hh);
+                        t1[e] = rot_factor<T>(D.E1, D.B1, ph[e], hh);
+                    }
+                    cn_row<T, V>(oa, ob, db_d, db_u, da_u, da_d, D.cc, n == 1 ? (T)2 : (T)1, sR[il + 1], gc, (T)n,
+                                 t0, t1, cn, an, bn);
                 }
-                cn_row<T, V>(oa, ob, db_d, db_u, da_u, da_d, D.cc, n == 1 ? (T)2 : (T)1, sR[il + 1], gc, (T)n, t0,
-                             t1, cn, an, bn);
                 /* b_0 = 0 (Eq. b_boundary); columns past m = M stay zero */
 #pragma unroll
                 for (int e = 0; e < V; ++e) {
@@ -526,8 +547,7 @@ const void* grid_fn(int vec) {
         return vec == 4 ? reinterpret_cast<const void*>(&grid_kernel<float, 4>)
                         : reinterpret_cast<const void*>(&grid_kernel<float, 2>);
     else
-        return vec == 2 ? reinterpret_cast<const void*>(&grid_kernel<double, 2>)
-                        : reinterpret_cast<const void*>(&grid_kernel<double, 1>);
+        return reinterpret_cast<const void*>(&grid_kernel<double, 1>);
 }
 
 }  // namespace

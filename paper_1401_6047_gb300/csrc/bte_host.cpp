@@ -212,21 +212,20 @@ constexpr int kBlkMaxSteps = 4096;
 constexpr int kBlkMinSteps = 4;
 
 /* Blocks of the on-chip mode of one block per SM: of all row splits GR and
- * the two column-group widths V, the one with the least estimated time of a
+ * the two column-group widths V (one in FP64), the one with the least estimated time of a
  * half-step in cycles.  The interior cells run while the neighbours' edges
  * are under way (about 1100 cycles from a store to its poll), the boundary
  * cells after them.  FP32: a pass over one group per thread takes about 700
  * cycles, and 166 (V = 4) or 100 (V = 2) issue slots per warp and row.  FP64:
- * a warp's pass takes about 3300 cycles per column, however many of its
- * lanes hold a cell, and one of four warps runs at a time on each quarter of
- * an SM.  Measured on a GB300 (us per step, this choice / best of a sweep of
- * 13 row splits, both widths and 64 to 512 threads): 31 x 201 FP64 4.5 /
- * 4.4, FP32 2.0 / 1.9; 138 x 1533 FP32 3.6 / 3.6; 120 x 4000 FP32 4.5 / 4.5;
- * 401 x 4001 FP32 7.5 / 7.5; 65 x 1000 FP64 11.9 / 11.9.  False when no
+ * a warp's pass takes about 1700 cycles, however many of its lanes hold a
+ * cell, and each quarter of an SM runs one at a time.  Measured on a GB300 (us per step, this choice / best of a sweep of
+ * 13 row splits, both widths and 64 to 512 threads): 31 x 201 FP64 4.0 /
+ * 3.8, FP32 3.1 / 2.1; 138 x 1533 FP32 4.8 / 3.8; 120 x 4000 FP32 4.8 / 4.8;
+ * 401 x 4001 FP32 8.5 / 7.9; 65 x 1000 FP64 9.5 / 9.8.  False when no
  * split fits the shared memory. */
 bool pick_blocks(int N1, int M1, size_t elem, Layout& L) {
     double best = 1e30;
-    for (int V = elem == 8 ? 1 : 2; V <= (elem == 8 ? 2 : 4); V *= 2)
+    for (int V = elem == 8 ? 1 : 2; V <= (elem == 8 ? 1 : 4); V *= 2)
         for (int gr = 1; gr <= std::min(N1, kBlkCtas); ++gr) {
             const int R = (N1 + gr - 1) / gr, GR = (N1 + R - 1) / R;
             if (GR != gr) continue;
@@ -241,8 +240,8 @@ bool pick_blocks(int N1, int M1, size_t elem, Layout& L) {
             thr = std::min(std::max(thr, 64), bte::kGridThreads);
             double t_int = 0.0, t_bnd;
             if (elem == 8) {
-                t_int = ni ? 3300.0 * V * std::max(1.0, ni / 128.0) : 0.0;
-                t_bnd = 3300.0 * V * std::max(1.0, nb / 128.0);
+                t_int = ni ? 1700.0 * std::max(1.0, ni / 128.0) : 0.0;
+                t_bnd = 1700.0 * std::max(1.0, nb / 128.0);
             } else {
                 if (ni) {
                     const int cpp = std::min(nci, thr), split = thr / cpp;
@@ -395,9 +394,9 @@ int plan(const bte_params* p, const bte_tuning* t, const TimeGrid& tg, Layout& L
     o += align_up((size_t)L.pitch * L.elem, 256);
     const long long Pt = tg.P > 0 ? tg.P : 1;
     L.off_ew = o;
-    o += align_up((size_t)3 * (Pt + 2) * L.elem, 256);
+    o += align_up((size_t)(L.elem == 8 ? bte::kDriveRows<double> : bte::kDriveRows<float>) * (Pt + 2) * L.elem, 256);
     L.off_ef = o;
-    o += align_up((size_t)3 * (Pt + 2) * L.elem, 256);
+    o += align_up((size_t)(L.elem == 8 ? bte::kDriveRows<double> : bte::kDriveRows<float>) * (Pt + 2) * L.elem, 256);
     L.off_tv = o;
     o += align_up((size_t)(tg.K + 1) * 8, 256);
     L.off_tn = o;
@@ -482,6 +481,17 @@ struct bte_handle {
 
 namespace {
 
+/* h, h/2, nu = 1 + h/2, xi = 1 - h/2 as the kernels take them (FP64: the
+ * first two divided by nu) */
+template <typename T>
+void set_step(double h, T& th, T& thh, T& nu, T& xi) {
+    const double s = sizeof(T) == 8 ? 1.0 + 0.5 * h : 1.0;
+    th = (T)(h / s);
+    thh = (T)(0.5 * h / s);
+    nu = (T)(1.0 + 0.5 * h);
+    xi = (T)(1.0 - 0.5 * h);
+}
+
 template <typename T>
 bte::StepArgs<T> step_args(const bte_handle* h) {
     bte::StepArgs<T> a;
@@ -520,10 +530,7 @@ bte::StepArgs<T> step_args(const bte_handle* h) {
     a.alt = L.walk == 2 ||
             (L.walk == 0 && 8 * L.elem * (size_t)(h->p.n_max + 1) * (size_t)L.pitch > bte::kAltStateBytes);
     const double dt = h->tg.dt_eff;
-    a.h = (T)dt;
-    a.hh = (T)(0.5 * dt);
-    a.nu = (T)(1.0 + 0.5 * dt);
-    a.xi = (T)(1.0 - 0.5 * dt);
+    set_step<T>(dt, a.h, a.hh, a.nu, a.xi);
     const double sq = std::sqrt(h->p.alpha);
     a.vscale = kPi * sq * h->dphi;
     a.nscale = 2.0 * kPi * sq * h->dphi;
@@ -534,11 +541,12 @@ bte::StepArgs<T> step_args(const bte_handle* h) {
  * column factors sqrt(mu/(2 pi alpha)) exp(-mu phi^2/2) and phi_m laid out
  * with G ghost columns, and the drive (FP64, rounded to T once) over one
  * period plus two entries
- * in two [3][P+2] tables: at the whole-grid times i dt (ew) and the
+ * in two [kDriveRows][P+2] tables: at the whole-grid times i dt (ew) and the
  * fractional-grid times (i + 1/2) dt (ef), E(t) (Sec. 2, E(t) = E_dc +
  * E_omega cos(omega t)), B(t) = B + B_omega cos(omega t + B_phase), and the
  * stencil coefficient B dt/(4 dphi) of the half-step starting at t, with B
- * taken at the time of the other grid, t + dt/2. */
+ * taken at the time of the other grid, t + dt/2; in FP64 that coefficient
+ * divided by nu, and the sums of E and of B at t and t + dt. */
 template <typename T>
 void build_tables(const bte_params& p, const TimeGrid& tg, int G, int pitch, double dphi,
                   std::vector<T>& row, std::vector<T>& colg, std::vector<T>& colp,
@@ -559,21 +567,30 @@ void build_tables(const bte_params& p, const TimeGrid& tg, int G, int pitch, dou
     }
     const long long Pt = tg.P > 0 ? tg.P : 1;
     const long long S = Pt + 2;
-    ew.assign(3 * S, (T)0);
-    ef.assign(3 * S, (T)0);
+    ew.assign(bte::kDriveRows<T> * S, (T)0);
+    ef.assign(bte::kDriveRows<T> * S, (T)0);
     const double dt = tg.dt_eff;
-    /* drive phase of time (q + s/2) dt: 2 pi (q + s/2)/P, or 0 when omega == 0 */
-    auto ph = [&](long long q, int s) {
-        return tg.P > 0 ? kTwoPi * ((double)q + 0.5 * s) / (double)Pt : 0.0;
-    };
-    auto Bt = [&](double x) { return p.B + p.B_omega * std::cos(x + p.B_phase); };
-    for (long long q = 0; q < S; ++q) {
-        ew[q] = (T)(p.E_dc + p.E_omega * std::cos(ph(q, 0)));
-        ef[q] = (T)(p.E_dc + p.E_omega * std::cos(ph(q, 1)));
-        ew[S + q] = (T)Bt(ph(q, 0));
-        ef[S + q] = (T)Bt(ph(q, 1));
-        ew[2 * S + q] = (T)(Bt(ph(q, 1)) * dt / (4.0 * dphi));
-        ef[2 * S + q] = (T)(Bt(ph(q, 2)) * dt / (4.0 * dphi));
+    const double scale = sizeof(T) == 8 ? 1.0 + 0.5 * dt : 1.0; /* FP64: divided by nu */
+    /* E and B at times q dt/2, q = 0 .. 2S + 1 (drive phase 2 pi (q/2)/P, or
+     * 0 when omega == 0); one cosine where B is constant */
+    std::vector<double> E(2 * S + 2), B(2 * S + 2);
+    for (long long q = 0; q < 2 * S + 2; ++q) {
+        const double x = tg.P > 0 ? kTwoPi * ((double)(q >> 1) + 0.5 * (double)(q & 1)) / (double)Pt : 0.0;
+        E[q] = p.E_dc + p.E_omega * std::cos(x);
+        B[q] = p.B + (p.B_omega != 0.0 ? p.B_omega * std::cos(x + p.B_phase) : 0.0);
+    }
+    for (int f = 0; f < 2; ++f) {
+        T* w = f ? ef.data() : ew.data();
+        for (long long q = 0; q < S; ++q) {
+            const long long i = 2 * q + f;
+            w[q] = (T)E[i];
+            w[S + q] = (T)B[i];
+            w[2 * S + q] = (T)(B[i + 1] * dt / (4.0 * dphi) / scale);
+            if (bte::kDriveRows<T> == 5) {
+                w[3 * S + q] = (T)E[i] + (T)E[i + 2];
+                w[4 * S + q] = (T)B[i] + (T)B[i + 2];
+            }
+        }
     }
 }
 
@@ -587,11 +604,13 @@ void startup_drive(const bte_params& p, double dt_eff, double dphi, bte::ApplyAr
     a.E_end = p.E_dc + p.E_omega * std::cos(p.omega * hs);
     a.B_start = p.B + p.B_omega * std::cos(p.B_phase);
     a.B_end = p.B + p.B_omega * std::cos(p.omega * hs + p.B_phase);
-    a.h = (T)hs;
-    a.hh = (T)(0.5 * hs);
-    a.nu = (T)(1.0 + 0.5 * hs);
-    a.xi = (T)(1.0 - 0.5 * hs);
+    set_step<T>(hs, a.h, a.hh, a.nu, a.xi);
     a.c = (T)(a.B_start * hs / (4.0 * dphi));
+    if (sizeof(T) == 8) {
+        a.c = (T)(a.c / (1.0 + 0.5 * hs));
+        a.E_start += a.E_end;
+        a.B_start += a.B_end;
+    }
 }
 
 template <typename T>
@@ -607,9 +626,9 @@ int upload_tables(bte_handle* h) {
                        cudaMemcpyHostToDevice, h->stream));
     CU(cudaMemcpyAsync(h->ptr<T>(L.off_col_phi), colp.data(), L.pitch * sizeof(T),
                        cudaMemcpyHostToDevice, h->stream));
-    CU(cudaMemcpyAsync(h->ptr<T>(L.off_ew), ew.data(), 3 * (Pt + 2) * sizeof(T), cudaMemcpyHostToDevice,
+    CU(cudaMemcpyAsync(h->ptr<T>(L.off_ew), ew.data(), ew.size() * sizeof(T), cudaMemcpyHostToDevice,
                        h->stream));
-    CU(cudaMemcpyAsync(h->ptr<T>(L.off_ef), ef.data(), 3 * (Pt + 2) * sizeof(T), cudaMemcpyHostToDevice,
+    CU(cudaMemcpyAsync(h->ptr<T>(L.off_ef), ef.data(), ef.size() * sizeof(T), cudaMemcpyHostToDevice,
                        h->stream));
     CU(cudaStreamSynchronize(h->stream)); /* host vectors go out of scope */
     return BTE_OK;
@@ -724,10 +743,7 @@ int enqueue_resident(bte_handle* h, long long n) {
     R.nty = L.nty;
     R.item0 = 0;
     const double dt = h->tg.dt_eff;
-    R.h = (T)dt;
-    R.hh = (T)(0.5 * dt);
-    R.nu = (T)(1.0 + 0.5 * dt);
-    R.xi = (T)(1.0 - 0.5 * dt);
+    set_step<T>(dt, R.h, R.hh, R.nu, R.xi);
     const double sq = std::sqrt(h->p.alpha);
     R.vscale = kPi * sq * h->dphi;
     R.nscale = 2.0 * kPi * sq * h->dphi;
@@ -785,10 +801,7 @@ int enqueue_wide(bte_handle* h, long long n) {
     w.Wc = L.wideWc;
     w.rows_per = L.wide_rp;
     const double dt = h->tg.dt_eff;
-    w.h = (T)dt;
-    w.hh = (T)(0.5 * dt);
-    w.nu = (T)(1.0 + 0.5 * dt);
-    w.xi = (T)(1.0 - 0.5 * dt);
+    set_step<T>(dt, w.h, w.hh, w.nu, w.xi);
     const double sq = std::sqrt(h->p.alpha);
     const double vscale = kPi * sq * h->dphi, nscale = 2.0 * kPi * sq * h->dphi;
     while (n > 0) {
@@ -1014,9 +1027,9 @@ int run_batch(const bte_params* p, std::vector<BatchPoint>& pts, size_t first, s
         b.o_colp = t;
         t += align_up((size_t)b.pitch * elem, 256);
         b.o_ew = t;
-        t += align_up((size_t)3 * (Pt + 2) * elem, 256);
+        t += align_up((size_t)bte::kDriveRows<T> * (Pt + 2) * elem, 256);
         b.o_ef = t;
-        t += align_up((size_t)3 * (Pt + 2) * elem, 256);
+        t += align_up((size_t)bte::kDriveRows<T> * (Pt + 2) * elem, 256);
         b.o_part = t;
         t += align_up((size_t)2 * b.ntx * 8, 256);
         b.o_ticket = t;
@@ -1099,10 +1112,7 @@ int run_batch(const bte_params* p, std::vector<BatchPoint>& pts, size_t first, s
         item0 += b.items;
         item_inst.insert(item_inst.end(), (size_t)b.items, (int)(i - first));
         const double dt = b.tg.dt_eff;
-        R.h = (T)dt;
-        R.hh = (T)(0.5 * dt);
-        R.nu = (T)(1.0 + 0.5 * dt);
-        R.xi = (T)(1.0 - 0.5 * dt);
+        set_step<T>(dt, R.h, R.hh, R.nu, R.xi);
         const double sq = std::sqrt(pp.alpha);
         R.vscale = kPi * sq * b.dphi;
         R.nscale = 2.0 * kPi * sq * b.dphi;
@@ -1497,8 +1507,8 @@ int bte_batch_run(const bte_params* p, int32_t n, bte_obs* out, const bte_batch_
                (resC > 0 || (int)(last - first) < max_batch)) {
             const BatchPoint& b = pts[last];
             const long long pitch = (long long)align_up((size_t)(128 / elem + b.ntx * tile + 32 / elem), 32);
-            /* state arrays, the two [3][P+2] drive tables, other tables */
-            const long long sb = (resC > 0 ? 4ll : 8ll) * b.N1 * pitch * elem + 6ll * (b.tg.P + 2) * elem + 4096;
+            /* state arrays, the two drive tables, other tables */
+            const long long sb = (resC > 0 ? 4ll : 8ll) * b.N1 * pitch * elem + 2ll * (elem == 8 ? bte::kDriveRows<double> : bte::kDriveRows<float>) * (b.tg.P + 2) * elem + 4096;
             if (last > first && bytes + sb > max_bytes) break;
             bytes += sb;
             ++last;

@@ -33,6 +33,11 @@ struct Cols {
     static constexpr int H = 16 / (int)sizeof(T);
 };
 
+/* rows of a drive table: E(t), B(t), the stencil coefficient, and in FP64
+ * the sums E(t) + E(t + dt), B(t) + B(t + dt) */
+template <typename T>
+constexpr int kDriveRows = sizeof(T) == 8 ? 5 : 3;
+
 /* Ping-pong state above this many bytes does not stay in L2 (129 MB on a
  * GB300) from one step to the next: the step kernel then alternates the
  * direction of its row walks, so that each step starts with the rows the
@@ -49,12 +54,12 @@ struct StepArgs {
     const T* row_a0;      /* [N+1]   sigma_n I_n/I_0 / pi                        */
     const T* col_g;       /* [pitch] sqrt(mu/(2 pi alpha)) exp(-mu phi^2/2), 0 in ghosts */
     const T* col_phi;     /* [pitch] phi_y(m), 0 in ghosts                      */
-    const T* e_whole;     /* [3][dstride] at t = i dt_eff: E(t), B(t), and the
-                             stencil coefficient B(t + dt/2) dt/(4 dphi) of the
-                             whole-grid half-step from t (i = 0..P+1); FP64
-                             values rounded to T once on the host             */
-    const T* e_frac;      /* [3][dstride] at t = (i + 1/2) dt_eff: E(t), B(t),
-                             and B(t + dt/2) dt/(4 dphi) of the fractional
+    const T* e_whole;     /* [kDriveRows][dstride] at t = i dt_eff: E(t), B(t),
+                             the stencil coefficient B(t + dt/2) dt/(4 dphi) of
+                             the whole-grid half-step from t (i = 0..P+1; FP64:
+                             divided by nu), and the sums; FP64 values rounded
+                             to T once on the host                            */
+    const T* e_frac;      /* the same at t = (i + 1/2) dt_eff, of the fractional
                              half-step from t                                   */
     const long long* base;/* device step counter: the launch advances step base+i */
     double* trace_v;      /* [K+1] whole-grid v_dr samples                       */
@@ -73,7 +78,9 @@ struct StepArgs {
     int grid;             /* persistent CTAs; items are ntx * nty              */
     int alt;              /* 1: one-step launches alternate the row-walk
                              direction (a state larger than L2)              */
-    T h, hh, nu, xi;      /* dt, dt/2, 1 + dt/2, 1 - dt/2                        */
+    T h, hh, nu, xi;      /* dt, dt/2, 1 + dt/2, 1 - dt/2; FP64: the first two
+                             divided by nu (the update works with the equations
+                             divided by nu)                                     */
     double vscale, nscale;/* pi sqrt(alpha) dphi, 2 pi sqrt(alpha) dphi          */
 };
 
@@ -197,8 +204,9 @@ struct ApplyArgs {
     T* an; T* bn;                /* output (may not alias the inputs)          */
     const T* row_a0; const T* col_g; const T* col_phi;
     int N, M, pitch;
-    double E_start, E_end, B_start, B_end;
-    T h, hh, nu, xi, c;   /* c: stencil coefficient at the source's time        */
+    double E_start, E_end, B_start, B_end; /* FP64: _start the sum of the two   */
+    T h, hh, nu, xi, c;   /* c: stencil coefficient at the source's time; FP64:
+                             h, hh, c divided by nu                             */
 };
 
 struct FinalArgs {

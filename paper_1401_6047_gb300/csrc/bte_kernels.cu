@@ -57,11 +57,9 @@ __global__ void apply_kernel(ApplyArgs<T> A) {
                               : (T)0;
     const T ad = ld_or0(A.as, n - 1, c + 1, N, P) - ld_or0(A.as, n - 1, c - 1, N, P);
     const T au = ld_or0(A.as, n + 1, c + 1, N, P) - ld_or0(A.as, n + 1, c - 1, N, P);
-    const T Sa = stencil_a<T>(A.c, bu, bd);
-    const T Sb = stencil_b<T>(A.c, chi, ad, au);
     const size_t g = (size_t)n * P + c;
     T an, bn;
-    cn_cell<T>(A.a[g], A.b[g], Sa, Sb, O::mul(A.h, A.row_a0[n]), A.col_g[c], th, th1,
+    cn_cell<T>(A.a[g], A.b[g], stencil_a<T>(bu, bd), stencil_b<T>(chi, ad, au), A.c, O::mul(A.h, A.row_a0[n]), A.col_g[c], th, th1,
                cn_constants<T>(A.h, A.nu, A.xi), an, bn);
     if (n == 0) bn = (T)0;
     A.an[g] = an;

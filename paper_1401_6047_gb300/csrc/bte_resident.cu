@@ -40,7 +40,6 @@ namespace {
 
 using dev::cluster_arrive;
 using dev::cluster_wait;
-using dev::cn_cell;
 using dev::F2;
 using dev::Half;
 using dev::half_drive;
@@ -50,8 +49,6 @@ using dev::warp_sum_f2;
 using dev::CnK;
 using dev::Rn;
 using dev::rot_factor;
-using dev::stencil_a;
-using dev::stencil_b;
 
 template <typename T>
 struct RV {

@@ -172,28 +172,26 @@ struct View {
     int N, M, pitch, ntx, inst, q0; /* q0: the instance's first item */
     long long k;
     bool active;                     /* instance still running       */
-    T Ews, Ewe, Efs, Efe; /* E at the start / end of the whole and fractional half-steps */
-    T Bws, Bwe, Bfs, Bfe; /* B at the same times                                         */
+    T Ews, Ewe, Efs, Efe; /* E of the whole and fractional half-steps (Half::E0, E1)     */
+    T Bws, Bwe, Bfs, Bfe; /* B of the same (Half::B0, B1)                                */
     T ccw, ccf;           /* stencil coefficients of the two half-steps                   */
     T h, hh, nu, xi;
 };
 
-/* Drive of the half-steps of step k (kk = k mod P): E and B at the start and
- * end of each half-step and the two stencil coefficients, from the
- * [3][stride] tables (FP64 values rounded to T once on the host, so no
- * conversion here). */
+/* Drive of the half-steps of step k (kk = k mod P), see half_drive. */
 template <typename T>
 __device__ __forceinline__ void drive(View<T>& v, const T* ew, const T* ef, int stride, int kk) {
-    v.Ews = ew[kk];
-    v.Ewe = ew[kk + 1];
-    v.Efs = ef[kk];
-    v.Efe = ef[kk + 1];
-    v.Bws = ew[stride + kk];
-    v.Bwe = ew[stride + kk + 1];
-    v.Bfs = ef[stride + kk];
-    v.Bfe = ef[stride + kk + 1];
-    v.ccw = ew[2 * stride + kk];
-    v.ccf = ef[2 * stride + kk];
+    const Half<T> w = half_drive<T>(ew, stride, kk), f = half_drive<T>(ef, stride, kk);
+    v.Ews = w.E0;
+    v.Ewe = w.E1;
+    v.Efs = f.E0;
+    v.Efe = f.E1;
+    v.Bws = w.B0;
+    v.Bwe = w.B1;
+    v.Bfs = f.B0;
+    v.Bfe = f.B1;
+    v.ccw = w.cc;
+    v.ccf = f.cc;
 }
 
 /* Instance of item q: single-instance launches use A; batched ones look the

@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kWideMaxThreads) wide_kernel(WideArgs<T> A) {
                 T* pa = s + (size_t)o * arr + c_own;
                 T* pb = pa + arr;
                 T an, bn;
-                cn_update<T>(*pa, *pb, stencil_a<T>(D.cc, db_d, db_u), stencil_b<T>(D.cc, chi, da_u, da_d),
+                cn_update<T>(*pa, *pb, stencil_a<T>(db_d, db_u), stencil_b<T>(chi, da_u, da_d), D.cc,
                              hr, gcol, cf, cn, an, bn);
                 const T na = col_ok ? an : (T)0;
                 const T nb = (col_ok && n > 0) ? bn : (T)0;
