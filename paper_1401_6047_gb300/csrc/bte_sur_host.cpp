@@ -33,13 +33,14 @@ struct bte_sur {
     bool own_stream;
     unsigned char* mem;
     float *p, *g, *m, *v;
-    bf16* wb;
+    bf16 *wb, *wbt; /* W2, W3 in BF16, and transposed */
     bf16* wti; /* W2, W3 in the tensor cores' canonical layout (inference) */
     int* err;
     float *Z1, *Z2, *Z3, *DY, *Yh, *partial;
     bf16 *H1, *H2, *H3, *DZ1, *DZ2, *DZ3;
     double* loss;
     int* idx;
+    size_t idx_bytes;
     float *xd, *yd;
     long long nd;
     long long t; /* Adam steps taken */
@@ -79,6 +80,7 @@ int fail(int code, const char* fmt, ...) {
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 const double kTwoPi = 6.283185307179586476925286766559;
+constexpr int kTrainSteps = 128; /* steps queued between two synchronisations */
 
 /* Forward pass of every member over rows [0, Bp) of the activation buffers;
  * Z buffers are written only when `train`. */
@@ -119,14 +121,16 @@ int forward(bte_sur* h, const float* x, const int* idx, long long row0, int nval
         a.ldz = H;
         a.sZ = (long long)Bp * H;
         a.err = h->err;
-        KL(bte::sur::launch_gemm(a, false, false, bte::sur::EPI_FWD, h->M, h->stream));
+        KL(bte::sur::launch_gemm(a, bte::sur::EPI_FWD, h->M, h->stream));
     }
     return BTE_OK;
 }
 
-/* Loss, gradients into h->g; forward must have run with train = true. */
+/* Loss (added into `loss`), the gradients of W2 and W3 into h->g and the
+ * others' partial sums into h->partial; forward must have run with train =
+ * true. */
 int backward(bte_sur* h, const float* x, const float* y, const int* idx, long long row0,
-             int nvalid, int Bp) {
+             int nvalid, int Bp, double* loss, bte::sur::RedArgs& r) {
     const int H = h->H;
     const long long sAct = (long long)Bp * H;
     bte::sur::HeadArgs hd{};
@@ -146,33 +150,16 @@ int backward(bte_sur* h, const float* x, const float* y, const int* idx, long lo
     hd.inv_n = 1.0f / (float)nvalid;
     hd.DY = h->DY;
     hd.DZ3 = h->DZ3;
-    hd.loss = h->loss;
+    hd.loss = loss;
     hd.sc = h->sc;
     KL(bte::sur::launch_head(hd, h->M, h->stream));
-    /* layers 3 and 2: weight gradient dZ^T H_prev, then dZ_prev = (dZ W) * silu'(Z_prev) */
+    /* back through layers 3 and 2: dZ_prev = (dZ W) * silu'(Z_prev) */
     for (int layer = 1; layer >= 0; --layer) {
-        const bf16* dZ = layer == 1 ? h->DZ3 : h->DZ2;
-        const bf16* Hprev = layer == 1 ? h->H2 : h->H1;
-        bte::sur::GemmArgs gw{};
-        gw.A = dZ;
-        gw.lda = H;
-        gw.sA = sAct;
-        gw.B = Hprev;
-        gw.ldb = H;
-        gw.sB = sAct;
-        gw.M = H;
-        gw.N = H;
-        gw.K = Bp;
-        gw.C = h->g + (layer == 1 ? h->off.W3 : h->off.W2);
-        gw.ldc = H;
-        gw.sC = h->pstride;
-        gw.err = h->err;
-        KL(bte::sur::launch_gemm(gw, true, true, bte::sur::EPI_F32, h->M, h->stream));
         bte::sur::GemmArgs dh{};
-        dh.A = dZ;
+        dh.A = layer == 1 ? h->DZ3 : h->DZ2;
         dh.lda = H;
         dh.sA = sAct;
-        dh.B = h->wb + (long long)layer * H * H;
+        dh.B = h->wbt + (long long)layer * H * H;
         dh.ldb = H;
         dh.sB = 2ll * H * H;
         dh.M = Bp;
@@ -183,9 +170,25 @@ int backward(bte_sur* h, const float* x, const float* y, const int* idx, long lo
         dh.ldz = H;
         dh.sZ = sAct;
         dh.err = h->err;
-        KL(bte::sur::launch_gemm(dh, false, true, bte::sur::EPI_BWD, h->M, h->stream));
+        KL(bte::sur::launch_gemm(dh, bte::sur::EPI_BWD, h->M, h->stream));
     }
-    bte::sur::RedArgs r{};
+    /* weight gradients dZ^T H_prev of both */
+    bte::sur::WgradArgs gw{};
+    gw.dZ[0] = h->DZ2;
+    gw.dZ[1] = h->DZ3;
+    gw.H[0] = h->H1;
+    gw.H[1] = h->H2;
+    gw.ld = H;
+    gw.sAct = sAct;
+    gw.H0 = H;
+    gw.K = Bp;
+    gw.grad = h->g;
+    gw.pstride = h->pstride;
+    gw.oW[0] = h->off.W2;
+    gw.oW[1] = h->off.W3;
+    gw.err = h->err;
+    KL(bte::sur::launch_wgrad(gw, h->M, h->stream));
+    r = bte::sur::RedArgs{};
     r.DZ1 = h->DZ1;
     r.DZ2 = h->DZ2;
     r.DZ3 = h->DZ3;
@@ -202,7 +205,7 @@ int backward(bte_sur* h, const float* x, const float* y, const int* idx, long lo
     r.pstride = h->pstride;
     r.off = h->off;
     r.sc = h->sc;
-    KL(bte::sur::launch_reduce(r, h->M, h->stream));
+    KL(bte::sur::launch_reduce_partial(r, h->M, h->stream));
     return BTE_OK;
 }
 
@@ -213,8 +216,10 @@ bte::sur::AdamArgs adam_args(bte_sur* h) {
     a.m = h->m;
     a.v = h->v;
     a.wb = h->wb;
+    a.wbt = h->wbt;
+    a.partial = h->partial;
     a.pstride = h->pstride;
-    a.count = h->off.count;
+    a.off = h->off;
     a.oW2 = h->off.W2;
     a.oW3 = h->off.W3;
     a.H = h->H;
@@ -323,7 +328,7 @@ int bte_sur_create(const bte_sur_config* cfg, bte_sur** out) {
         return at;
     };
     const size_t op = take(P), og = take(P), om = take(P), ov = take(P);
-    const size_t owb = take((size_t)M * 2 * H * H * 2);
+    const size_t owb = take((size_t)M * 2 * H * H * 2), owbt = take((size_t)M * 2 * H * H * 2);
     const size_t owti = take((size_t)M * 2 * H * H * 2);
     const size_t oerr = take(256);
     const size_t oz1 = take(act32), oz2 = take(act32), oz3 = take(act32);
@@ -331,8 +336,11 @@ int bte_sur_create(const bte_sur_config* cfg, bte_sur** out) {
     const size_t od1 = take(act16), od2 = take(act16), od3 = take(act16);
     const size_t ody = take((size_t)M * cap * kOut * 4), oyh = take((size_t)M * cap * kOut * 4);
     const size_t opart = take((size_t)M * (cap / 128) * nred * 4);
-    const size_t oloss = take((size_t)M * 8);
-    const size_t oidx = take((size_t)M * cap * 4);
+    /* minibatch indices and losses of several steps (4 MB: 128 steps of 8
+     * members on 1024 points), uploaded and read back together */
+    h->idx_bytes = std::max((size_t)M * cap * 4, (size_t)4 << 20);
+    const size_t oloss = take((size_t)M * 8 * kTrainSteps);
+    const size_t oidx = take(h->idx_bytes);
     size_t oxin[2], omean[2], ostd[2], omask[2];
     for (int s = 0; s < 2; ++s) {
         oxin[s] = take((size_t)cap * kIn * 4);
@@ -352,6 +360,7 @@ int bte_sur_create(const bte_sur_config* cfg, bte_sur** out) {
     h->m = (float*)(b + om);
     h->v = (float*)(b + ov);
     h->wb = (bf16*)(b + owb);
+    h->wbt = (bf16*)(b + owbt);
     h->wti = (bf16*)(b + owti);
     h->err = (int*)(b + oerr);
     h->Z1 = (float*)(b + oz1);
@@ -397,11 +406,13 @@ int64_t bte_sur_param_count(const bte_sur* h) { return h ? h->off.count : 0; }
 
 int bte_sur_set_params(bte_sur* h, const float* p) {
     if (!h || !p) return fail(BTE_EINVAL, "NULL argument");
-    for (long long i = 0; i < (long long)h->M * h->off.count; ++i)
-        if (!std::isfinite(p[i])) return fail(BTE_EINVAL, "non-finite parameter at %lld", i);
-    for (int m = 0; m < h->M; ++m)
-        CU(cudaMemcpyAsync(h->p + m * h->pstride, p + (long long)m * h->off.count,
-                           h->off.count * 4, cudaMemcpyHostToDevice, h->stream));
+    unsigned bad = 0;
+    for (long long i = 0; i < (long long)h->M * h->off.count; ++i) bad |= (unsigned)!(std::fabs(p[i]) <= 3.402823466e38f);
+    if (bad)
+        for (long long i = 0; i < (long long)h->M * h->off.count; ++i)
+            if (!std::isfinite(p[i])) return fail(BTE_EINVAL, "non-finite parameter at %lld", i);
+    CU(cudaMemcpy2DAsync(h->p, h->pstride * 4, p, h->off.count * 4, h->off.count * 4, h->M, cudaMemcpyHostToDevice,
+                         h->stream));
     CU(cudaMemsetAsync(h->m, 0, (size_t)h->pstride * h->M * 4, h->stream));
     CU(cudaMemsetAsync(h->v, 0, (size_t)h->pstride * h->M * 4, h->stream));
     h->t = 0;
@@ -412,9 +423,8 @@ int bte_sur_set_params(bte_sur* h, const float* p) {
 
 int bte_sur_get_params(bte_sur* h, float* p) {
     if (!h || !p) return fail(BTE_EINVAL, "NULL argument");
-    for (int m = 0; m < h->M; ++m)
-        CU(cudaMemcpyAsync(p + (long long)m * h->off.count, h->p + m * h->pstride,
-                           h->off.count * 4, cudaMemcpyDeviceToHost, h->stream));
+    CU(cudaMemcpy2DAsync(p, h->off.count * 4, h->p, h->pstride * 4, h->off.count * 4, h->M, cudaMemcpyDeviceToHost,
+                         h->stream));
     CU(cudaStreamSynchronize(h->stream));
     return BTE_OK;
 }
@@ -448,33 +458,46 @@ int bte_sur_train(bte_sur* h, const int32_t* order, int32_t steps, int32_t batch
     if (!h->xd) return fail(BTE_ESTATE, "no training set uploaded");
     if (batch < 1 || batch > h->cap) return fail(BTE_EINVAL, "batch must be 1..%d", h->cap);
     const long long per = (long long)h->M * batch;
-    for (long long i = 0; i < per * steps; ++i)
-        if (order[i] < 0 || order[i] >= h->nd) return fail(BTE_EINVAL, "order[%lld] out of range", i);
+    unsigned bad = 0;
+    for (long long i = 0; i < per * steps; ++i) bad |= (unsigned)((uint32_t)order[i] >= (uint64_t)h->nd);
+    if (bad)
+        for (long long i = 0; i < per * steps; ++i)
+            if (order[i] < 0 || order[i] >= h->nd) return fail(BTE_EINVAL, "order[%lld] out of range", i);
     for (int s = 0; s < steps; ++s)
         if (!(lr[s] >= 0) || !std::isfinite(lr[s])) return fail(BTE_EINVAL, "bad learning rate");
     const int Bp = round128(batch);
-    std::vector<int> idx((size_t)h->M * Bp, 0);
-    std::vector<double> lh(h->M);
-    for (int s = 0; s < steps; ++s) {
-        for (int m = 0; m < h->M; ++m)
-            std::memcpy(&idx[(size_t)m * Bp], order + (s * per + (long long)m * batch), batch * 4);
-        /* the copy reads `idx` before the next iteration rewrites it: the
-         * stream is synchronised at the end of every step below */
+    const size_t row = (size_t)h->M * Bp; /* indices of one step */
+    const int most = (int)std::min<size_t>(kTrainSteps, h->idx_bytes / (row * 4));
+    std::vector<int> idx;
+    for (int s0 = 0; s0 < steps; s0 += most) {
+        const int n = std::min(most, steps - s0);
+        idx.assign(row * n, 0);
+        for (int s = 0; s < n; ++s)
+            for (int m = 0; m < h->M; ++m)
+                std::memcpy(&idx[s * row + (size_t)m * Bp], order + ((s0 + s) * per + (long long)m * batch), batch * 4);
         CU(cudaMemcpyAsync(h->idx, idx.data(), idx.size() * 4, cudaMemcpyHostToDevice, h->stream));
-        CU(cudaMemsetAsync(h->loss, 0, h->M * 8, h->stream));
-        int rc = forward(h, h->xd, h->idx, 0, batch, Bp, true);
-        if (!rc) rc = backward(h, h->xd, h->yd, h->idx, 0, batch, Bp);
-        if (rc) return rc;
-        h->t += 1;
-        bte::sur::AdamArgs a = adam_args(h);
-        a.lr = lr[s];
-        a.c1 = (float)(1.0 / (1.0 - std::pow(0.9, (double)h->t)));
-        a.c2 = (float)(1.0 / (1.0 - std::pow(0.999, (double)h->t)));
-        KL(bte::sur::launch_adam(a, h->stream));
-        if (loss) CU(cudaMemcpyAsync(lh.data(), h->loss, h->M * 8, cudaMemcpyDeviceToHost, h->stream));
-        CU(cudaStreamSynchronize(h->stream));
+        CU(cudaMemsetAsync(h->loss, 0, (size_t)n * h->M * 8, h->stream));
+        for (int s = 0; s < n; ++s) {
+            const int* ix = h->idx + s * row;
+            bte::sur::RedArgs r;
+            int rc = forward(h, h->xd, ix, 0, batch, Bp, true);
+            if (!rc) rc = backward(h, h->xd, h->yd, ix, 0, batch, Bp, h->loss + (size_t)s * h->M, r);
+            if (rc) {
+                cudaStreamSynchronize(h->stream); /* the upload reads `idx` */
+                return rc;
+            }
+            h->t += 1;
+            bte::sur::AdamArgs a = adam_args(h);
+            a.nch = Bp / 128;
+            a.lr = lr[s0 + s];
+            a.c1 = (float)(1.0 / (1.0 - std::pow(0.9, (double)h->t)));
+            a.c2 = (float)(1.0 / (1.0 - std::pow(0.999, (double)h->t)));
+            KL(bte::sur::launch_adam(a, h->stream));
+        }
         if (loss)
-            for (int m = 0; m < h->M; ++m) loss[(long long)s * h->M + m] = lh[m];
+            CU(cudaMemcpyAsync(loss + (long long)s0 * h->M, h->loss, (size_t)n * h->M * 8, cudaMemcpyDeviceToHost,
+                               h->stream));
+        CU(cudaStreamSynchronize(h->stream));
     }
     int err = 0;
     CU(cudaMemcpy(&err, h->err, sizeof err, cudaMemcpyDeviceToHost));
@@ -500,7 +523,9 @@ int bte_sur_grad(bte_sur* h, const float* x, const float* t, int32_t n, float* g
         cudaMemsetAsync(h->loss, 0, h->M * 8, h->stream) != cudaSuccess)
         rc = fail(BTE_ECUDA, "upload failed");
     if (!rc) rc = forward(h, xd, nullptr, 0, n, Bp, true);
-    if (!rc) rc = backward(h, xd, td, nullptr, 0, n, Bp);
+    bte::sur::RedArgs r;
+    if (!rc) rc = backward(h, xd, td, nullptr, 0, n, Bp, h->loss, r);
+    if (!rc && bte::sur::launch_reduce_final(r, h->M, h->stream)) rc = fail(BTE_ECUDA, "reduction launch failed");
     if (!rc && grad)
         for (int m = 0; m < h->M && !rc; ++m)
             if (cudaMemcpyAsync(grad + (long long)m * h->off.count, h->g + m * h->pstride,

@@ -7,7 +7,8 @@
  * W2 [H][H], b2 [H], W3 [H][H], b3 [H], W4 [2][H], b4 [2]; members sit
  * `pstride` floats apart (pstride = the packed count rounded up to 8 so
  * every member starts on a 32-byte boundary).  BF16 copies of W2 and W3
- * (the tensor-core operands) sit in `wb` as [M][2][H][H].  Activations of a
+ * (the tensor-core operands) sit in `wb` as [M][2][H][H], their transposes
+ * in `wbt`.  Activations of a
  * batch of Bp samples (Bp a multiple of 128) are [M][Bp][H], row-major.
  */
 #pragma once
@@ -48,16 +49,15 @@ struct Scale {
     float y_mean[kOut], y_std[kOut];
 };
 
-enum Epi { EPI_FWD = 0, EPI_BWD = 1, EPI_F32 = 2 };
+enum Epi { EPI_FWD = 0, EPI_BWD = 1 };
 
-/* C[M][N] = sum_k A(m, k) B(k, n) per member (blockIdx.z), BF16 operands,
- * FP32 accumulation, then one epilogue:
+/* C[m][n] = sum_k A(m, k) B(n, k) per member (blockIdx.z) along the hidden
+ * units (K = H = 256), BF16 operands stored [m][k] and [n][k], FP32
+ * accumulation, then one epilogue:
  *   EPI_FWD: z = acc + bias[n]; Z[m][n] = z (if Z), Hout[m][n] = bf16(silu(z))
  *   EPI_BWD: Dout[m][n] = bf16(acc * silu'(Zin[m][n]))
- *   EPI_F32: C[m][n] = acc
- * A is stored [m][k] (a_kmajor = false) or [k][m]; B is stored [n][k]
- * (b_kmajor = false) or [k][n].  M, N multiples of 128; K of 64; every
- * leading dimension a multiple of 8 elements, bases 16-byte aligned. */
+ * M, N multiples of 128; every leading dimension a multiple of 8 elements,
+ * bases 16-byte aligned. */
 struct GemmArgs {
     const __nv_bfloat16* A;
     long long lda, sA;
@@ -71,9 +71,20 @@ struct GemmArgs {
     const float* Zin;
     __nv_bfloat16* Dout;
     long long ldz, sZ; /* leading dimension / member stride of Z, Hout, Zin, Dout */
-    float* C;
-    long long ldc, sC;
     int* err; /* set to 1 when a bounded wait gives up (may be null) */
+};
+
+/* Weight gradients of the hidden layers W2 (layer 0) and W3 (1): grad[out][in]
+ * = sum over the K samples of dZ[s][out] H[s][in], written at oW[layer] of
+ * each member; H0 units, ld between samples, sAct between members. */
+struct WgradArgs {
+    const __nv_bfloat16* dZ[2];
+    const __nv_bfloat16* H[2];
+    long long ld, sAct;
+    int H0, K;
+    float* grad;
+    long long pstride, oW[2];
+    int* err;
 };
 
 /* Layer 1 (K = 5, FP32 FMAs): Z1 = W1 xh + b1, H1 = bf16(silu(Z1)), for
@@ -136,8 +147,12 @@ struct AdamArgs {
     float* g;
     float* m;
     float* v;
-    __nv_bfloat16* wb; /* [M][2][H][H] BF16 copies of W2, W3 */
-    long long pstride, count, oW2, oW3;
+    __nv_bfloat16* wb;  /* [M][2][H][H] BF16 copies of W2, W3 */
+    __nv_bfloat16* wbt; /* ... and of their transposes */
+    const float* partial; /* partial sums of the other parameters' gradients (RedArgs) */
+    int nch;              /* their 128-sample blocks */
+    long long pstride, oW2, oW3;
+    ParamOffsets off;
     int H, members;
     float lr, beta1, beta2, eps, c1, c2; /* c1 = 1/(1-beta1^t), c2 = 1/(1-beta2^t) */
 };
@@ -170,11 +185,12 @@ struct EnsArgs {
     Scale sc;
 };
 
-int launch_gemm(const GemmArgs& a, bool a_kmajor, bool b_kmajor, int epi, int members,
-                void* stream);
+int launch_gemm(const GemmArgs& a, int epi, int members, void* stream);
+int launch_wgrad(const WgradArgs& a, int members, void* stream);
 int launch_l1(const L1Args& a, int members, void* stream);
 int launch_head(const HeadArgs& a, int members, void* stream);
-int launch_reduce(const RedArgs& a, int members, void* stream);
+int launch_reduce_partial(const RedArgs& a, int members, void* stream);
+int launch_reduce_final(const RedArgs& a, int members, void* stream); /* into grad */
 int launch_adam(const AdamArgs& a, void* stream);
 int launch_refresh_bf16(const AdamArgs& a, void* stream);
 int launch_ensemble(const EnsArgs& a, void* stream);

@@ -3,11 +3,18 @@
  *
  * The two 256 x 256 hidden layers and their backward products run on the
  * fifth-generation BF16 tensor cores (tcgen05.mma, FP32 accumulators in
- * tensor memory) in one GEMM kernel whose epilogue fuses the bias, the SiLU
- * activation and its derivative.  The thin layers (5 inputs, 2 outputs) are
- * FP32 FMA kernels; batch reductions are two-pass and deterministic; Adam
- * keeps FP32 master weights and refreshes the BF16 operand copies in the
- * same pass.
+ * tensor memory) in two GEMM kernels: one for the products along the hidden
+ * units (forward, and back through a layer), whose epilogue fuses the bias,
+ * the SiLU activation and its derivative, and one for the weight gradients
+ * (along the batch).  The thin layers (5 inputs, 2 outputs) are FP32 FMA
+ * kernels; batch reductions are two-pass and deterministic; Adam keeps FP32
+ * master weights and refreshes the BF16 operand copies in the same pass.
+ *
+ * A training step of 8 members on 1024 points each moves about 90 MB through
+ * L2 and 6.5 GFLOP through the tensor cores, 10 to 15 us of work; it is bound
+ * by the latency of its kernels, each a few microseconds long and waiting on
+ * the one before, so each is cut to fill the SMs once and to have its loads
+ * in flight together.
  */
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -20,14 +27,21 @@ namespace bte {
 namespace sur {
 namespace {
 
-/* tcgen05 GEMM tile: 128 x 128 outputs per CTA (one MMA of M = N = 128
- * per 16 of K), K in stages of 64, two stages in shared memory. */
-constexpr int GM = 128, GN = 128, GK = 64;
+/* GEMMs of 128 x 128 outputs per CTA (MMAs of M = N = 128 per 16 of K), K in
+ * stages of 64, four of them in shared memory: along the hidden units (K =
+ * 256) all of both operands, every load in flight at once.  What bounds them
+ * is that fill: asynchronous copies bring about 19 bytes per clock to an SM
+ * (128 KB: 7000 cycles, the same in several orders of the copies), the MMAs
+ * take 2500 and the epilogue 8000.  Core matrices (8 x 8, 128 bytes) sit 144
+ * bytes apart, so that eight threads that fill the same row of eight of them
+ * meet no bank twice and a warp reads whole 128-byte lines. */
+constexpr int GM = 128, GN = 128, GK = 64, kGStages = 4;
 constexpr int kGThreads = 256; /* 8 warps: two per tensor-memory lane quadrant */
-constexpr uint32_t kGTileBytes = (uint32_t)GM * GK * 2; /* 16 KB per operand tile */
-constexpr uint32_t kGCore = 128;                        /* one 8 x 8 core matrix */
-constexpr uint32_t kGGroup = (GK / 8) * kGCore;         /* 1024: next 8-row group */
-constexpr size_t kGSmem = 4 * (size_t)kGTileBytes + 64 + 1024; /* 2 stages x (A, B), barriers, align */
+constexpr uint32_t kGCore = 144;
+constexpr uint32_t kGGroup = (GK / 8) * kGCore;        /* K-major: next 8-row group */
+constexpr uint32_t kGTileBytes = (GM / 8) * kGGroup;   /* 18 KB per operand and stage */
+constexpr uint32_t kGGroupMN = (GM / 8) * kGCore;      /* MN-major: next 8 k */
+constexpr size_t kGSmem = 2 * kGStages * (size_t)kGTileBytes + 64 + 1024; /* A, B, barriers, align */
 
 /* sigmoid(z) = 1 / (1 + exp(-z)) with the fast exponential and reciprocal
  * (relative error ~1e-7, so the bfloat16 rounding that follows matches an
@@ -39,140 +53,134 @@ __device__ __forceinline__ float silu_grad_f(float z) {
     return s * (1.0f + z * (1.0f - s));
 }
 
-/* byte offset of element (r, k) of a [128][64] K-major stage tile in the
- * tensor cores' canonical layout without swizzle (8 x 8 core matrices of
- * 128 contiguous bytes, K-adjacent core matrices 128 bytes apart, 8-row
- * groups 1024 bytes apart) */
-__device__ __forceinline__ uint32_t gcanon(int r, int k) {
-    return (uint32_t)(((r >> 3) * (GK / 8) + (k >> 3)) * kGCore + (r & 7) * 16 + (k & 7) * 2);
+/* The 128 rows of a K-major operand ([row][k], leading dimension ld), all
+ * 256 k, into its four stage tiles by asynchronous copies: a warp takes a row
+ * at a time, lane l its l-th chunk of 8 k. */
+__device__ __forceinline__ void load_rows(unsigned char* s, const __nv_bfloat16* g, long long ld, int row0) {
+    const int warp = threadIdx.x >> 5, l = threadIdx.x & 31;
+    const uint32_t d = dev::smem_u32(s) + (l >> 3) * kGTileBytes + (l & 7) * kGCore;
+#pragma unroll
+    for (int q = 0; q < GM / 8; ++q) {
+        const int r = q * 8 + warp;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + (r >> 3) * kGGroup + (r & 7) * 16),
+                     "l"(g + (long long)(row0 + r) * ld + l * 8)
+                     : "memory");
+    }
+}
+__device__ __forceinline__ void commit_stage() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT>
+__device__ __forceinline__ void wait_stage() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory");
 }
 
-/* One 128-row x 64-k operand tile into shared memory (canonical layout).
- * K-major source ([row][k], leading dimension ld): 1024 chunks of 8 k, four
- * per thread; a quarter-warp writes one core matrix (8 rows of one chunk
- * column, 128 contiguous bytes).  MN-major source ([k][row]): 128 blocks
- * of 8 k x 8 rows, one per thread of `first` .. `first + 127`, read as
- * eight 16-byte rows and transposed in registers (byte permutes) into the
- * eight 16-byte rows of one core matrix. */
-template <bool MN>
-__device__ __forceinline__ void load_stage(unsigned char* s, const __nv_bfloat16* g, long long ld,
-                                           int row0, int k0, int first) {
-    const int t = threadIdx.x;
-    if constexpr (!MN) {
+/* One stage (64 k x 128 rows) of an MN-major operand ([k][row]): eight rows
+ * of one k are 16 contiguous bytes in the source and in a core matrix, which
+ * holds 8 k of 8 rows; a warp takes two k at a time. */
+__device__ __forceinline__ void load_stage_mn(unsigned char* s, const __nv_bfloat16* g, long long ld,
+                                              int row0, int k0) {
+    const uint32_t d = dev::smem_u32(s);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int c = t + q * kGThreads;
-            const int r = (c & 7) + 8 * (c >> 6), kc = (c >> 3) & 7;
-            const uint4 v =
-                __ldg(reinterpret_cast<const uint4*>(g + (long long)(row0 + r) * ld + k0 + kc * 8));
-            *reinterpret_cast<uint4*>(s + gcanon(r, kc * 8)) = v;
-        }
-    } else {
-        const int b = t - first;
-        if (b < 0 || b >= 128) return;
-        const int rb = b & 15, kb = b >> 4; /* 16 row blocks x 8 k blocks */
-        uint32_t w[8][4];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const uint4 v = __ldg(reinterpret_cast<const uint4*>(
-                g + (long long)(k0 + kb * 8 + i) * ld + row0 + rb * 8));
-            w[i][0] = v.x;
-            w[i][1] = v.y;
-            w[i][2] = v.z;
-            w[i][3] = v.w;
-        }
-        unsigned char* dst = s + (uint32_t)((rb * (GK / 8) + kb) * kGCore);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            /* row j of the core matrix: element j of input rows 0..7 */
-            const uint32_t sel = (j & 1) ? 0x7632u : 0x5410u;
-            uint4 o;
-            o.x = __byte_perm(w[0][j >> 1], w[1][j >> 1], sel);
-            o.y = __byte_perm(w[2][j >> 1], w[3][j >> 1], sel);
-            o.z = __byte_perm(w[4][j >> 1], w[5][j >> 1], sel);
-            o.w = __byte_perm(w[6][j >> 1], w[7][j >> 1], sel);
-            *reinterpret_cast<uint4*>(dst + j * 16) = o;
-        }
+    for (int q = 0; q < 4; ++q) {
+        const int c = threadIdx.x + q * kGThreads;
+        const int rb = c & 15, k = c >> 4; /* 16 row blocks x 64 k */
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + (k >> 3) * kGGroupMN + rb * kGCore +
+                                                                        (k & 7) * 16),
+                     "l"(g + (long long)(k0 + k) * ld + row0 + rb * 8)
+                     : "memory");
     }
 }
 
-/* C = A B^T on the tensor cores (see GemmArgs).  One CTA per 128 x 128
- * output tile of one member (blockIdx.z).  K advances in stages of 64: the
- * CTA's threads fill stage s (global loads, transposed where the operand
- * is stored MN-major) while the tensor cores still work on the other
- * stage; one thread issues the four M = N = 128, K = 16 MMAs of a stage
- * into 128 columns of tensor memory and commits them to the stage's
- * mbarrier, which tells the threads when they may refill it.  The
- * epilogue reads the accumulators back with tcgen05.ld (warp w: lanes
- * 32 (w mod 4) .., columns 64 (w / 4) ..).  Every wait is bounded; a wait
- * that gives up sets the error word, and the CTA still frees its tensor
- * memory before it exits. */
-template <bool AMN, bool BMN, int EPI>
-__global__ void __launch_bounds__(kGThreads) gemm_tc_kernel(GemmArgs a) {
-    extern __shared__ unsigned char gsm_raw[];
-    unsigned char* gsm = reinterpret_cast<unsigned char*>(
-        (reinterpret_cast<uintptr_t>(gsm_raw) + 1023) & ~(uintptr_t)1023);
-    /* stage s: A tile at s * 16 KB, B tile at (2 + s) * 16 KB; barrier s at 64 KB + 8 s */
-    uint64_t* bars = reinterpret_cast<uint64_t*>(gsm + 4 * kGTileBytes);
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gsm + 4 * kGTileBytes + 32);
-    const uint32_t bar0 = dev::smem_u32(bars);
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
-    const int mem = blockIdx.z;
-    const __nv_bfloat16* A = a.A + mem * a.sA;
-    const __nv_bfloat16* B = a.B + mem * a.sB;
-    const int m0 = blockIdx.y * GM, n0 = blockIdx.x * GN;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    bool ok = true;
-
-    if (tid == 0) {
-        dev::mbar_init(bar0, 1);
-        dev::mbar_init(bar0 + 8, 1);
-        dev::fence_proxy_async_smem();
-    }
+template <int COLS>
+__device__ __forceinline__ uint32_t tmem_begin(uint32_t* slot, int warp) {
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         dev::smem_u32(tmem_slot)),
-                     "r"(GN)
+                         dev::smem_u32(slot)),
+                     "r"(COLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
-    constexpr uint32_t idesc = tc::instr_desc(GM, GN);
+    return *slot;
+}
+template <int COLS>
+__device__ __forceinline__ void tmem_end(uint32_t tmem, int warp) {
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(COLS)
+                     : "memory");
+}
 
-    const int nk = a.K / GK;
-    for (int kt = 0; kt < nk; ++kt) {
-        const int st = kt & 1;
-        unsigned char* sA = gsm + st * kGTileBytes;
-        unsigned char* sB = gsm + (2 + st) * kGTileBytes;
-        const uint32_t bar = bar0 + 8 * st;
-        /* the MMAs that read this stage two rounds ago are complete */
-        if (kt >= 2 && !dev::mbar_wait(bar, (uint32_t)(((kt - 2) >> 1) & 1))) ok = false;
-        if (__syncthreads_or(!ok)) break;
-        load_stage<AMN>(sA, A, a.lda, m0, kt * GK, 0);
-        load_stage<BMN>(sB, B, a.ldb, n0, kt * GK, AMN ? 128 : 0);
-        /* generic-proxy writes -> visible to the tensor cores */
-        dev::fence_proxy_async_smem();
-        __syncthreads();
-        if (tid == 0) {
-            tc::tc_fence_after();
-            const uint32_t aA = dev::smem_u32(sA), aB = dev::smem_u32(sB);
+/* The four K = 16 MMAs of one stage.  The descriptor's two offsets: K-major,
+ * the next core matrix along k and along the rows; MN-major, the next along k
+ * and along the rows as well. */
+template <bool MN>
+__device__ __forceinline__ void stage_mma(uint32_t tmem, uint32_t aA, uint32_t aB, bool first) {
+    constexpr uint32_t idesc = tc::instr_desc(GM, GN) | (MN ? 3u << 15 : 0u); /* both operands MN-major */
+    constexpr uint32_t along_k = MN ? kGGroupMN : kGCore, along_rows = MN ? kGCore : kGGroup;
 #pragma unroll
-            for (int ks = 0; ks < GK / 16; ++ks) {
-                const uint64_t ad = tc::smem_desc(aA + ks * 2 * kGCore, kGCore, kGGroup);
-                const uint64_t bd = tc::smem_desc(aB + ks * 2 * kGCore, kGCore, kGGroup);
-                tc::tc_mma(tmem, ad, bd, idesc, (kt > 0 || ks > 0) ? 1u : 0u);
-            }
-            tc::tc_commit(bar);
-        }
+    for (int ks = 0; ks < GK / 16; ++ks) {
+        const uint64_t ad = tc::smem_desc(aA + ks * 2 * along_k, along_k, along_rows);
+        const uint64_t bd = tc::smem_desc(aB + ks * 2 * along_k, along_k, along_rows);
+        tc::tc_mma(tmem, ad, bd, idesc, (!first || ks > 0) ? 1u : 0u);
     }
-    /* the last commit covers every MMA issued before it */
-    if (ok && nk > 0 && !dev::mbar_wait(bar0 + 8 * ((nk - 1) & 1), (uint32_t)(((nk - 1) >> 1) & 1)))
-        ok = false;
-    if (ok && nk > 1 && !dev::mbar_wait(bar0 + 8 * (nk & 1), (uint32_t)(((nk - 2) >> 1) & 1)))
-        ok = false;
+}
+
+/* C = A B^T along the hidden units (see GemmArgs), both operands K-major.
+ * One CTA per 128 x 128 output tile of one member (blockIdx.z).  Once both
+ * operands have landed, one thread issues the MMAs into 128 columns of tensor
+ * memory.  The epilogue reads the accumulators back with tcgen05.ld (warp
+ * w: lanes 32 (w mod 4) .., columns 64 (w / 4) ..).  The wait is bounded; if
+ * it gives up the error word is set, and the CTA still frees its tensor
+ * memory before it exits.  Measured (8 members, 1024 rows, GB300): 19 us
+ * with two stages filled through registers, 12 us so. */
+template <int EPI>
+__global__ void __launch_bounds__(kGThreads) gemm_tc_kernel(GemmArgs a) {
+    extern __shared__ unsigned char gsm_raw[];
+    unsigned char* gsm = reinterpret_cast<unsigned char*>(
+        (reinterpret_cast<uintptr_t>(gsm_raw) + 1023) & ~(uintptr_t)1023);
+    /* the stages of A, those of B, the barrier */
+    uint64_t* bars = reinterpret_cast<uint64_t*>(gsm + 2 * kGStages * kGTileBytes);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2);
+    const uint32_t bar = dev::smem_u32(bars);
+
+    const int mem = blockIdx.z;
+    const __nv_bfloat16* A = a.A + mem * a.sA;
+    const __nv_bfloat16* B = a.B + mem * a.sB;
+    const int m0 = blockIdx.y * GM, n0 = blockIdx.x * GN;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+
+    if (tid == 0) {
+        dev::mbar_init(bar, 1);
+        dev::fence_proxy_async_smem();
+    }
+    const uint32_t tmem = tmem_begin<GN>(tmem_slot, warp);
+    pdl_wait();
+    pdl_trigger();
+    load_rows(gsm, A, a.lda, m0);
+    load_rows(gsm + kGStages * kGTileBytes, B, a.ldb, n0);
+    commit_stage();
+    wait_stage<0>();
+    /* generic-proxy writes -> visible to the tensor cores */
+    dev::fence_proxy_async_smem();
+    __syncthreads();
+    if (tid == 0) {
+        tc::tc_fence_after();
+#pragma unroll
+        for (int st = 0; st < kGStages; ++st)
+            stage_mma<false>(tmem, dev::smem_u32(gsm + st * kGTileBytes),
+                             dev::smem_u32(gsm + (kGStages + st) * kGTileBytes), st == 0);
+        tc::tc_commit(bar);
+    }
+    const bool ok = dev::mbar_wait(bar, 0u);
     tc::tc_fence_after();
 
     if (ok) {
@@ -184,9 +192,9 @@ __global__ void __launch_bounds__(kGThreads) gemm_tc_kernel(GemmArgs a) {
             float v[32];
             tc::tc_ld32(tmem + ((uint32_t)(sub * 32) << 16) + (uint32_t)cl, v);
             const int col = n0 + cl;
+            const long long o = mem * a.sZ + (long long)row * a.ldz + col;
             if (EPI == EPI_FWD) {
                 const float* bias = a.bias + mem * a.sBias + col;
-                const long long o = mem * a.sZ + (long long)row * a.ldz + col;
 #pragma unroll
                 for (int c8 = 0; c8 < 32; c8 += 8) {
                     float z[8];
@@ -202,8 +210,7 @@ __global__ void __launch_bounds__(kGThreads) gemm_tc_kernel(GemmArgs a) {
                         pk[e] = __floats2bfloat162_rn(silu_f(z[2 * e]), silu_f(z[2 * e + 1]));
                     *reinterpret_cast<uint4*>(a.Hout + o + c8) = *reinterpret_cast<const uint4*>(pk);
                 }
-            } else if (EPI == EPI_BWD) {
-                const long long o = mem * a.sZ + (long long)row * a.ldz + col;
+            } else {
 #pragma unroll
                 for (int c8 = 0; c8 < 32; c8 += 8) {
                     const float4 z0 = *reinterpret_cast<const float4*>(a.Zin + o + c8);
@@ -216,22 +223,89 @@ __global__ void __launch_bounds__(kGThreads) gemm_tc_kernel(GemmArgs a) {
                                                       v[c8 + 2 * e + 1] * silu_grad_f(z[2 * e + 1]));
                     *reinterpret_cast<uint4*>(a.Dout + o + c8) = *reinterpret_cast<const uint4*>(pk);
                 }
-            } else {
-                const long long o = mem * a.sC + (long long)row * a.ldc + col;
-#pragma unroll
-                for (int c4 = 0; c4 < 32; c4 += 4)
-                    *reinterpret_cast<float4*>(a.C + o + c4) =
-                        make_float4(v[c4], v[c4 + 1], v[c4 + 2], v[c4 + 3]);
             }
         }
     }
     if (!ok && tid == 0 && a.err) atomicExch(a.err, 1);
-    tc::tc_fence_before();
-    __syncthreads();
+    tmem_end<GN>(tmem, warp);
+}
+
+/* Weight gradients dW = dZ^T H of both hidden layers (see WgradArgs): 128 x
+ * 128 outputs per CTA, blockIdx.z = 2 member + layer, K the batch.  Both
+ * operands are stored [sample][unit], so they go to shared memory as they
+ * are and the tensor cores take them MN-major; stages of 64 samples, three
+ * in flight while one is multiplied.  The tile is square because the loads
+ * bound it (34 MB through L2 for 8 members x 1024, 25 us; 128 x 32 tiles,
+ * which fill more SMs, move 84 MB: 29 us), and K stays whole to keep the
+ * order of the sum.  Every wait is bounded, as above. */
+__global__ void __launch_bounds__(kGThreads) wgrad_tc_kernel(WgradArgs a) {
+    extern __shared__ unsigned char gsm_raw[];
+    unsigned char* gsm = reinterpret_cast<unsigned char*>(
+        (reinterpret_cast<uintptr_t>(gsm_raw) + 1023) & ~(uintptr_t)1023);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(gsm + 2 * kGStages * kGTileBytes);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kGStages);
+    const uint32_t bar0 = dev::smem_u32(bars);
+
+    const int layer = blockIdx.z & 1, mem = blockIdx.z >> 1;
+    const __nv_bfloat16* A = a.dZ[layer] + mem * a.sAct;
+    const __nv_bfloat16* B = a.H[layer] + mem * a.sAct;
+    const int m0 = blockIdx.y * GM, n0 = blockIdx.x * GN;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) {
+        for (int st = 0; st < kGStages; ++st) dev::mbar_init(bar0 + 8 * st, 1);
+        dev::fence_proxy_async_smem();
+    }
+    const uint32_t tmem = tmem_begin<GN>(tmem_slot, warp);
+    pdl_wait();
+    pdl_trigger(); /* reduce_partial_kernel reads nothing of this one's */
+
+    const int nk = a.K / GK;
+    auto load = [&](int kt) { /* one group per stage, empty past the end */
+        if (kt < nk) {
+            load_stage_mn(gsm + (kt % kGStages) * kGTileBytes, A, a.ld, m0, kt * GK);
+            load_stage_mn(gsm + (kGStages + kt % kGStages) * kGTileBytes, B, a.ld, n0, kt * GK);
+        }
+        commit_stage();
+    };
+    bool ok = true;
+    for (int kt = 0; kt < kGStages - 1; ++kt) load(kt);
+    for (int kt = 0; kt < nk; ++kt) {
+        const int st = kt % kGStages;
+        wait_stage<kGStages - 2>();
+        /* generic-proxy writes -> visible to the tensor cores */
+        dev::fence_proxy_async_smem();
+        if (__syncthreads_or(!ok)) break;
+        if (tid == 0) {
+            tc::tc_fence_after();
+            stage_mma<true>(tmem, dev::smem_u32(gsm + st * kGTileBytes),
+                            dev::smem_u32(gsm + (kGStages + st) * kGTileBytes), kt == 0);
+            tc::tc_commit(bar0 + 8 * st);
+        }
+        /* the stage before this one is free once its MMAs are complete */
+        if (kt >= 1 && !dev::mbar_wait(bar0 + 8 * ((kt - 1) % kGStages), (uint32_t)(((kt - 1) / kGStages) & 1)))
+            ok = false;
+        if (ok) load(kt + kGStages - 1);
+        else commit_stage();
+    }
+    /* the last commit covers every MMA issued before it */
+    if (ok && !dev::mbar_wait(bar0 + 8 * ((nk - 1) % kGStages), (uint32_t)(((nk - 1) / kGStages) & 1))) ok = false;
+    wait_stage<0>();
     tc::tc_fence_after();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(GN)
-                     : "memory");
+    if (ok) {
+        const int sub = warp & 3, half = warp >> 2;
+        float* o = a.grad + mem * a.pstride + a.oW[layer] + (long long)(m0 + sub * 32 + lane) * a.ld + n0;
+#pragma unroll 1
+        for (int cb = 0; cb < GN / 2; cb += 32) {
+            const int cl = half * (GN / 2) + cb;
+            float v[32];
+            tc::tc_ld32(tmem + ((uint32_t)(sub * 32) << 16) + (uint32_t)cl, v);
+#pragma unroll
+            for (int c4 = 0; c4 < 32; c4 += 4)
+                *reinterpret_cast<float4*>(o + cl + c4) = make_float4(v[c4], v[c4 + 1], v[c4 + 2], v[c4 + 3]);
+        }
+    }
+    if (!ok && tid == 0 && a.err) atomicExch(a.err, 1);
+    tmem_end<GN>(tmem, warp);
 }
 
 __device__ __forceinline__ void load_xh(const float* x, const int* idx, long long row0, int r,
@@ -246,47 +320,76 @@ __device__ __forceinline__ void load_xh(const float* x, const int* idx, long lon
     }
 }
 
+/* 16 rows of one member per CTA: thread o holds hidden unit o's weights,
+ * the rows' inputs sit in shared memory (8 members x 1024 rows: 14 us with
+ * one output per thread, 5 us so) */
+constexpr int kL1Rows = 16;
 __global__ void l1_kernel(L1Args a) {
-    const int mem = blockIdx.y;
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (long long)a.Bp * a.H) return;
-    const int r = (int)(e / a.H), o = (int)(e - (long long)r * a.H);
+    const int mem = blockIdx.y, r0 = blockIdx.x * kL1Rows, o = threadIdx.x;
+    __shared__ float sxh[kL1Rows][kIn];
+    pdl_wait();
+    pdl_trigger();
     const int* idx = a.idx ? a.idx + (long long)mem * a.Bp : nullptr;
-    float xh[kIn];
-    load_xh(a.x, idx, a.row0, r, a.nvalid, a.sc, xh);
-    const float* P = a.params + mem * a.pstride;
-    float z = P[a.ob1 + o];
+    if (o < kL1Rows) {
+        float xh[kIn];
+        load_xh(a.x, idx, a.row0, r0 + o, a.nvalid, a.sc, xh);
 #pragma unroll
-    for (int i = 0; i < kIn; ++i) z = fmaf(P[a.oW1 + (long long)o * kIn + i], xh[i], z);
-    const long long out = ((long long)mem * a.Bp + r) * a.H + o;
-    if (a.Z1) a.Z1[out] = z;
-    a.H1[out] = __float2bfloat16_rn(silu_f(z));
+        for (int i = 0; i < kIn; ++i) sxh[o][i] = xh[i];
+    }
+    const float* P = a.params + mem * a.pstride;
+    const float b = P[a.ob1 + o];
+    float w[kIn];
+#pragma unroll
+    for (int i = 0; i < kIn; ++i) w[i] = P[a.oW1 + (long long)o * kIn + i];
+    __syncthreads();
+    const long long out = ((long long)mem * a.Bp + r0) * a.H + o;
+#pragma unroll
+    for (int r = 0; r < kL1Rows; ++r) {
+        float z = b;
+#pragma unroll
+        for (int i = 0; i < kIn; ++i) z = fmaf(w[i], sxh[r][i], z);
+        if (a.Z1) a.Z1[out + (long long)r * a.H] = z;
+        a.H1[out + (long long)r * a.H] = __float2bfloat16_rn(silu_f(z));
+    }
 }
 
-/* one warp per sample; lane l covers hidden units 8l .. 8l+7 (H = 256) */
+/* 8 consecutive floats at a 16-byte aligned address */
+__device__ __forceinline__ void ld8(const float* p, float (&x)[8]) {
+    const float4 u = reinterpret_cast<const float4*>(p)[0], v = reinterpret_cast<const float4*>(p)[1];
+    x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w;
+    x[4] = v.x; x[5] = v.y; x[6] = v.z; x[7] = v.w;
+}
+
+/* one warp per sample; lane l covers hidden units 8l .. 8l+7 (H = 256); the
+ * loss of the CTA's 8 samples is formed by eight lanes of one warp (FP64
+ * instructions cost a warp the same however few lanes they serve) and added
+ * with one atomic */
 __global__ void head_kernel(HeadArgs a) {
     const int mem = blockIdx.y;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int r = blockIdx.x * (blockDim.x >> 5) + warp;
-    if (r >= a.Bp) return;
+    const int r = blockIdx.x * (blockDim.x >> 5) + warp; /* < Bp: a multiple of 128 */
+    __shared__ float s_e[8][2];
+    pdl_wait();
+    pdl_trigger();
     const float* P = a.params + mem * a.pstride;
     const long long base = ((long long)mem * a.Bp + r) * a.H;
     float y0 = 0.0f, y1 = 0.0f;
-    float hv[8];
-    for (int c0 = lane * 8; c0 < a.H; c0 += 256) {
-        const uint4 raw = *reinterpret_cast<const uint4*>(a.H3 + base + c0);
-        const __nv_bfloat162* hp = reinterpret_cast<const __nv_bfloat162*>(&raw);
+    const int c0 = lane * 8;
+    float hv[8], w0[8], w1[8];
+    ld8(P + a.oW4 + c0, w0);
+    ld8(P + a.oW4 + a.H + c0, w1);
+    const uint4 raw = *reinterpret_cast<const uint4*>(a.H3 + base + c0);
+    const __nv_bfloat162* hp = reinterpret_cast<const __nv_bfloat162*>(&raw);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float2 f = __bfloat1622float2(hp[i]);
-            hv[2 * i] = f.x;
-            hv[2 * i + 1] = f.y;
-        }
+    for (int i = 0; i < 4; ++i) {
+        const float2 f = __bfloat1622float2(hp[i]);
+        hv[2 * i] = f.x;
+        hv[2 * i + 1] = f.y;
+    }
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            y0 = fmaf(P[a.oW4 + c0 + i], hv[i], y0);
-            y1 = fmaf(P[a.oW4 + a.H + c0 + i], hv[i], y1);
-        }
+    for (int i = 0; i < 8; ++i) {
+        y0 = fmaf(w0[i], hv[i], y0);
+        y1 = fmaf(w1[i], hv[i], y1);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -303,87 +406,140 @@ __global__ void head_kernel(HeadArgs a) {
     if (!a.y) return;
     /* training: loss gradient and the output layer's backward product */
     float d0 = 0.0f, d1 = 0.0f;
+    float e0 = 0.0f, e1 = 0.0f;
     if (r < a.nvalid) {
         const int* idx = a.idx ? a.idx + (long long)mem * a.Bp : nullptr;
         const long long s = idx ? (long long)idx[r] : a.row0 + r;
         const float t0 = (a.y[s * kOut] - a.sc.y_mean[0]) / a.sc.y_std[0];
         const float t1 = (a.y[s * kOut + 1] - a.sc.y_mean[1]) / a.sc.y_std[1];
-        d0 = (y0 - t0) * a.inv_n;
-        d1 = (y1 - t1) * a.inv_n;
-        if (lane == 0) {
-            const double l = 0.5 * ((double)(y0 - t0) * (y0 - t0) + (double)(y1 - t1) * (y1 - t1));
-            atomicAdd(a.loss + mem, l * a.inv_n);
-        }
+        e0 = y0 - t0;
+        e1 = y1 - t1;
+        d0 = e0 * a.inv_n;
+        d1 = e1 * a.inv_n;
+    }
+    if (lane == 0) {
+        s_e[warp][0] = e0;
+        s_e[warp][1] = e1;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        double l = 0.0;
+        if (lane < 8) l = 0.5 * ((double)s_e[lane][0] * s_e[lane][0] + (double)s_e[lane][1] * s_e[lane][1]) * a.inv_n;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) l += __shfl_down_sync(0xffffffffu, l, o);
+        if (lane == 0) atomicAdd(a.loss + mem, l);
     }
     if (lane == 0) {
         a.DY[yo] = d0;
         a.DY[yo + 1] = d1;
     }
-    for (int c0 = lane * 8; c0 < a.H; c0 += 256) {
-        __nv_bfloat162 outv[4];
+    float z[8];
+    ld8(a.Z3 + base + c0, z);
+    __nv_bfloat162 outv[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float v[2];
+    for (int i = 0; i < 4; ++i) {
+        float v[2];
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int c = c0 + 2 * i + u;
-                const float dh = d0 * P[a.oW4 + c] + d1 * P[a.oW4 + a.H + c];
-                v[u] = dh * silu_grad_f(a.Z3[base + c]);
-            }
-            outv[i] = __floats2bfloat162_rn(v[0], v[1]);
+        for (int u = 0; u < 2; ++u) {
+            const float dh = fmaf(d0, w0[2 * i + u], d1 * w1[2 * i + u]);
+            v[u] = dh * silu_grad_f(z[2 * i + u]);
         }
-        *reinterpret_cast<uint4*>(a.DZ3 + base + c0) = *reinterpret_cast<const uint4*>(outv);
+        outv[i] = __floats2bfloat162_rn(v[0], v[1]);
     }
+    *reinterpret_cast<uint4*>(a.DZ3 + base + c0) = *reinterpret_cast<const uint4*>(outv);
 }
 
 /* values per 128-sample block: b1, W1 (5 per unit), b2, b3, W4 (2 per unit), b4 */
 __host__ __device__ inline int red_count(int H) { return H * (1 + kIn + 1 + 1 + kOut) + kOut; }
 
-__global__ void reduce_partial_kernel(RedArgs a) {
-    const int mem = blockIdx.y, chunk = blockIdx.x;
-    const int r0 = chunk * 128;
-    __shared__ float sxh[128][kIn];
-    __shared__ float sdy[128][kOut];
-    const int* idx = a.idx ? a.idx + (long long)mem * a.Bp : nullptr;
-    for (int r = threadIdx.x; r < 128; r += blockDim.x) {
-        float xh[kIn];
-        load_xh(a.x, idx, a.row0, r0 + r, a.nvalid, a.sc, xh);
+/* Partial sums over 128 samples (blockIdx.x) of one member (blockIdx.y).
+ * blockIdx.z = 4 part + quarter of the hidden units; part 0: b1 and W1 (from
+ * DZ1 and the inputs), 1: b2, 2: b3, 3: W4 and b4 (from H3 and DY).  One
+ * hidden unit per thread, the samples added in order, 32 loads in flight (one
+ * CTA per 128 samples that did all four arrays: 107 us for 8 members x 1024,
+ * one load of each array in flight; so: 10 us).  Launched beside the weight
+ * gradients (programmatic dependent launch: that kernel starts after the
+ * activations' gradients are complete, and this one reads only those); it
+ * ends after them, so what follows it in the stream follows both. */
+constexpr int kRedThreads = 64, kRedFly = 32;
+template <class F>
+__device__ __forceinline__ void over_samples(const __nv_bfloat16* p, int H, F f) {
+    for (int r0 = 0; r0 < 128; r0 += kRedFly) {
+        __nv_bfloat16 v[kRedFly];
 #pragma unroll
-        for (int i = 0; i < kIn; ++i) sxh[r][i] = xh[i];
-        const long long yo = ((long long)mem * a.Bp + r0 + r) * kOut;
-        sdy[r][0] = a.DY[yo];
-        sdy[r][1] = a.DY[yo + 1];
+        for (int q = 0; q < kRedFly; ++q) v[q] = p[(long long)(r0 + q) * H];
+#pragma unroll
+        for (int q = 0; q < kRedFly; ++q) f(r0 + q, __bfloat162float(v[q]));
     }
-    __syncthreads();
-    const int nred = red_count(a.H);
+}
+__global__ void __launch_bounds__(kRedThreads) reduce_partial_kernel(RedArgs a) {
+    const int mem = blockIdx.y, chunk = blockIdx.x, part = blockIdx.z >> 2;
+    const int r0 = chunk * 128, o = (blockIdx.z & 3) * kRedThreads + threadIdx.x;
+    __shared__ float sx[128][kIn];
+    const int H = a.H, nred = red_count(H);
     float* out = a.partial + ((long long)mem * (a.Bp / 128) + chunk) * nred;
-    for (int o = threadIdx.x; o < a.H; o += blockDim.x) {
-        float gb1 = 0, gw1[kIn] = {0, 0, 0, 0, 0}, gb2 = 0, gb3 = 0, gw4[kOut] = {0, 0};
-        for (int r = 0; r < 128; ++r) {
-            const long long e = ((long long)mem * a.Bp + r0 + r) * a.H + o;
-            const float d1 = __bfloat162float(a.DZ1[e]);
-            gb1 += d1;
+    const long long e = ((long long)mem * a.Bp + r0) * H + o;
+    if (part == 0) {
+        const int* idx = a.idx ? a.idx + (long long)mem * a.Bp : nullptr;
+        for (int r = threadIdx.x; r < 128; r += kRedThreads) {
+            float xh[kIn];
+            load_xh(a.x, idx, a.row0, r0 + r, a.nvalid, a.sc, xh);
 #pragma unroll
-            for (int i = 0; i < kIn; ++i) gw1[i] = fmaf(d1, sxh[r][i], gw1[i]);
-            gb2 += __bfloat162float(a.DZ2[e]);
-            gb3 += __bfloat162float(a.DZ3[e]);
-            const float h3 = __bfloat162float(a.H3[e]);
-            gw4[0] = fmaf(sdy[r][0], h3, gw4[0]);
-            gw4[1] = fmaf(sdy[r][1], h3, gw4[1]);
+            for (int i = 0; i < kIn; ++i) sx[r][i] = xh[i];
         }
-        out[o] = gb1;
+        __syncthreads();
+        float gb = 0, gw[kIn] = {0, 0, 0, 0, 0};
+        over_samples(a.DZ1 + e, H, [&](int r, float d) {
+            gb += d;
 #pragma unroll
-        for (int i = 0; i < kIn; ++i) out[a.H + o * kIn + i] = gw1[i];
-        out[a.H * (1 + kIn) + o] = gb2;
-        out[a.H * (2 + kIn) + o] = gb3;
-        out[a.H * (3 + kIn) + o] = gw4[0];
-        out[a.H * (4 + kIn) + o] = gw4[1];
+            for (int i = 0; i < kIn; ++i) gw[i] = fmaf(d, sx[r][i], gw[i]);
+        });
+        out[o] = gb;
+#pragma unroll
+        for (int i = 0; i < kIn; ++i) out[H + o * kIn + i] = gw[i];
+    } else if (part < 3) {
+        float gb = 0;
+        over_samples((part == 1 ? a.DZ2 : a.DZ3) + e, H, [&](int, float d) { gb += d; });
+        out[H * (kIn + part) + o] = gb;
+    } else {
+        for (int r = threadIdx.x; r < 128; r += kRedThreads) {
+            const long long yo = ((long long)mem * a.Bp + r0 + r) * kOut;
+            sx[r][0] = a.DY[yo];
+            sx[r][1] = a.DY[yo + 1];
+        }
+        __syncthreads();
+        float gw[kOut] = {0, 0};
+        over_samples(a.H3 + e, H, [&](int r, float h3) {
+            gw[0] = fmaf(sx[r][0], h3, gw[0]);
+            gw[1] = fmaf(sx[r][1], h3, gw[1]);
+        });
+        out[H * (3 + kIn) + o] = gw[0];
+        out[H * (4 + kIn) + o] = gw[1];
+        if (o < kOut) {
+            float s = 0;
+            for (int r = 0; r < 128; ++r) s += sx[r][o];
+            out[H * (3 + kIn + kOut) + o] = s;
+        }
     }
-    if (threadIdx.x < kOut) {
-        float s = 0;
-        for (int r = 0; r < 128; ++r) s += sdy[r][threadIdx.x];
-        out[a.H * (3 + kIn + kOut) + threadIdx.x] = s;
-    }
+    pdl_wait();
+}
+
+/* value q of a member's packed reductions: its sum over the 128-sample
+ * blocks, and its place among the member's parameters */
+__device__ __forceinline__ float reduced(const float* partial, int mem, int nch, int nred, int q) {
+    const float* part = partial + (long long)mem * nch * nred;
+    float s = 0;
+    for (int c = 0; c < nch; ++c) s += part[(long long)c * nred + q];
+    return s;
+}
+__device__ __forceinline__ long long reduced_place(const ParamOffsets& off, int H, int q) {
+    if (q < H) return off.b1 + q;
+    if (q < H * (1 + kIn)) return off.W1 + (q - H);
+    if (q < H * (2 + kIn)) return off.b2 + (q - H * (1 + kIn));
+    if (q < H * (3 + kIn)) return off.b3 + (q - H * (2 + kIn));
+    if (q < H * (4 + kIn)) return off.W4 + (q - H * (3 + kIn));
+    if (q < H * (5 + kIn)) return off.W4 + H + (q - H * (4 + kIn));
+    return off.b4 + (q - H * (5 + kIn));
 }
 
 __global__ void reduce_final_kernel(RedArgs a) {
@@ -391,51 +547,63 @@ __global__ void reduce_final_kernel(RedArgs a) {
     const int nred = red_count(a.H);
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= nred) return;
-    const int nch = a.Bp / 128;
-    const float* part = a.partial + (long long)mem * nch * nred;
-    float s = 0;
-    for (int c = 0; c < nch; ++c) s += part[(long long)c * nred + q];
-    /* destination of value q in the packed member */
-    const int H = a.H;
-    long long dst;
-    if (q < H) dst = a.off.b1 + q;
-    else if (q < H * (1 + kIn)) dst = a.off.W1 + (q - H);
-    else if (q < H * (2 + kIn)) dst = a.off.b2 + (q - H * (1 + kIn));
-    else if (q < H * (3 + kIn)) dst = a.off.b3 + (q - H * (2 + kIn));
-    else if (q < H * (4 + kIn)) dst = a.off.W4 + (q - H * (3 + kIn));
-    else if (q < H * (5 + kIn)) dst = a.off.W4 + H + (q - H * (4 + kIn));
-    else dst = a.off.b4 + (q - H * (5 + kIn));
-    a.grad[mem * a.pstride + dst] = s;
+    a.grad[mem * a.pstride + reduced_place(a.off, a.H, q)] = reduced(a.partial, mem, a.Bp / 128, nred, q);
 }
 
-__global__ void adam_kernel(AdamArgs a) {
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= a.pstride * a.members) return;
-    const int mem = (int)(e / a.pstride);
-    const long long q = e - (long long)mem * a.pstride;
-    if (q >= a.count) return;
-    const float g = a.g[e];
-    const float m = a.beta1 * a.m[e] + (1.0f - a.beta1) * g;
-    const float v = a.beta2 * a.v[e] + (1.0f - a.beta2) * g * g;
+/* one Adam update of parameter e with gradient g; the new value */
+__device__ __forceinline__ float adam_one(const AdamArgs& a, long long e, float g) {
+    const float m = fmaf(1.0f - a.beta1, g, a.beta1 * a.m[e]);
+    const float v = fmaf((1.0f - a.beta2) * g, g, a.beta2 * a.v[e]);
     a.m[e] = m;
     a.v[e] = v;
     const float p = a.p[e] - a.lr * (m * a.c1) / (sqrtf(v * a.c2) + a.eps);
     a.p[e] = p;
-    const long long HH = (long long)a.H * a.H;
-    if (q >= a.oW2 && q < a.oW2 + HH)
-        a.wb[(long long)mem * 2 * HH + (q - a.oW2)] = __float2bfloat16_rn(p);
-    else if (q >= a.oW3 && q < a.oW3 + HH)
-        a.wb[(long long)mem * 2 * HH + HH + (q - a.oW3)] = __float2bfloat16_rn(p);
+    return p;
 }
 
-__global__ void refresh_kernel(AdamArgs a) {
-    const long long HH = (long long)a.H * a.H;
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= 2 * HH * a.members) return;
-    const int mem = (int)(e / (2 * HH));
-    const long long q = e - mem * 2 * HH;
-    const long long src = mem * a.pstride + (q < HH ? a.oW2 + q : a.oW3 + (q - HH));
-    a.wb[e] = __float2bfloat16_rn(a.p[src]);
+/* a 32 x 32 tile (blockIdx.x of 2 x 64) of a hidden layer's weights: f(e)
+ * gives the value of parameter e, which goes as BF16 to W [out][in] and,
+ * through shared memory, to its transpose [in][out] (the operands of the
+ * forward and the backward products, both K-major) */
+template <class F>
+__device__ __forceinline__ void weight_tile(const AdamArgs& a, int mem, int tile, F f) {
+    __shared__ __nv_bfloat16 t[32][34];
+    const int layer = tile >> 6, o0 = ((tile >> 3) & 7) * 32, i0 = (tile & 7) * 32;
+    const int c = threadIdx.x & 31, r0 = threadIdx.x >> 5;
+    const long long base = mem * a.pstride + (layer ? a.oW3 : a.oW2);
+    const long long wo = ((long long)mem * 2 + layer) * a.H * a.H;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int o = o0 + r0 + 8 * j;
+        const __nv_bfloat16 p = __float2bfloat16_rn(f(base + (long long)o * a.H + i0 + c));
+        a.wb[wo + (long long)o * a.H + i0 + c] = p;
+        t[r0 + 8 * j][c] = p;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int i = r0 + 8 * j;
+        a.wbt[wo + (long long)(i0 + i) * a.H + o0 + c] = t[c][i];
+    }
+}
+
+/* Adam of every member (blockIdx.y): 128 tiles of W2 and W3, then the other
+ * parameters, whose gradients are still partial sums over 128-sample blocks */
+__global__ void __launch_bounds__(256) adam_kernel(AdamArgs a) {
+    const int mem = blockIdx.y;
+    pdl_wait();
+    pdl_trigger();
+    if (blockIdx.x < 128) {
+        weight_tile(a, mem, blockIdx.x, [&](long long e) { return adam_one(a, e, a.g[e]); });
+        return;
+    }
+    const int nred = red_count(a.H), q = (blockIdx.x - 128) * 256 + threadIdx.x;
+    if (q < nred)
+        adam_one(a, mem * a.pstride + reduced_place(a.off, a.H, q), reduced(a.partial, mem, a.nch, nred, q));
+}
+
+__global__ void __launch_bounds__(256) refresh_kernel(AdamArgs a) {
+    weight_tile(a, blockIdx.y, blockIdx.x, [&](long long e) { return a.p[e]; });
 }
 
 __global__ void ensemble_kernel(EnsArgs a) {
@@ -473,59 +641,71 @@ int ok_or(cudaError_t e) { return e == cudaSuccess ? 0 : (int)e; }
 
 int reduce_count(int H) { return red_count(H); }
 
-template <bool AMN, bool BMN, int EPI>
-static int launch_tc(const GemmArgs& a, int members, cudaStream_t s) {
-    const void* fn = reinterpret_cast<const void*>(&gemm_tc_kernel<AMN, BMN, EPI>);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGSmem);
-    if (e != cudaSuccess) return (int)e;
-    const dim3 grid(a.N / GN, a.M / GM, members);
-    gemm_tc_kernel<AMN, BMN, EPI><<<grid, kGThreads, kGSmem, s>>>(a);
-    return ok_or(cudaGetLastError());
+/* A launch that may begin while the one before it drains: the kernel reads
+ * and writes nothing of it before its griddepcontrol.wait. */
+template <class K, class A>
+static int launch_pdl(K* kernel, dim3 grid, int threads, size_t smem, void* stream, const A& args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = (cudaStream_t)stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return ok_or(cudaLaunchKernelEx(&cfg, kernel, args));
 }
 
-int launch_gemm(const GemmArgs& a, bool a_kmajor, bool b_kmajor, int epi, int members,
-                void* stream) {
-    if (a.M % GM || a.N % GN || a.K % GK || a.M <= 0 || a.N <= 0 || a.K <= 0)
-        return (int)cudaErrorInvalidValue;
+template <int EPI>
+static int launch_tc(const GemmArgs& a, int members, cudaStream_t s) {
+    const void* fn = reinterpret_cast<const void*>(&gemm_tc_kernel<EPI>);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGSmem);
+    if (e != cudaSuccess) return (int)e;
+    return launch_pdl(gemm_tc_kernel<EPI>, dim3(a.N / GN, a.M / GM, members), kGThreads, kGSmem, s, a);
+}
+
+int launch_gemm(const GemmArgs& a, int epi, int members, void* stream) {
+    if (a.M % GM || a.N % GN || a.K != kGStages * GK || a.M <= 0 || a.N <= 0) return (int)cudaErrorInvalidValue;
     cudaStream_t s = (cudaStream_t)stream;
-    if (!a_kmajor && !b_kmajor && epi == EPI_FWD) return launch_tc<false, false, EPI_FWD>(a, members, s);
-    if (!a_kmajor && b_kmajor && epi == EPI_BWD) return launch_tc<false, true, EPI_BWD>(a, members, s);
-    if (a_kmajor && b_kmajor && epi == EPI_F32) return launch_tc<true, true, EPI_F32>(a, members, s);
-    if (!a_kmajor && !b_kmajor && epi == EPI_F32) return launch_tc<false, false, EPI_F32>(a, members, s);
+    if (epi == EPI_FWD) return launch_tc<EPI_FWD>(a, members, s);
+    if (epi == EPI_BWD) return launch_tc<EPI_BWD>(a, members, s);
     return (int)cudaErrorInvalidValue;
 }
 
+int launch_wgrad(const WgradArgs& a, int members, void* stream) {
+    if (a.H0 % GM || a.K % GK || a.K <= 0) return (int)cudaErrorInvalidValue;
+    const cudaError_t e =
+        cudaFuncSetAttribute(wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGSmem);
+    if (e != cudaSuccess) return (int)e;
+    return launch_pdl(wgrad_tc_kernel, dim3(a.H0 / GN, a.H0 / GM, 2 * members), kGThreads, kGSmem, stream, a);
+}
+
 int launch_l1(const L1Args& a, int members, void* stream) {
-    const long long n = (long long)a.Bp * a.H;
-    const dim3 grid((unsigned)((n + 255) / 256), members);
-    l1_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(a);
-    return ok_or(cudaGetLastError());
+    return launch_pdl(l1_kernel, dim3(a.Bp / kL1Rows, members), a.H, 0, stream, a);
 }
 
 int launch_head(const HeadArgs& a, int members, void* stream) {
-    const dim3 grid((unsigned)((a.Bp + 7) / 8), members);
-    head_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(a);
-    return ok_or(cudaGetLastError());
+    return launch_pdl(head_kernel, dim3(a.Bp / 8, members), 256, 0, stream, a);
 }
 
-int launch_reduce(const RedArgs& a, int members, void* stream) {
-    reduce_partial_kernel<<<dim3(a.Bp / 128, members), 256, 0, (cudaStream_t)stream>>>(a);
-    int rc = ok_or(cudaGetLastError());
-    if (rc) return rc;
+int launch_reduce_partial(const RedArgs& a, int members, void* stream) {
+    return launch_pdl(reduce_partial_kernel, dim3(a.Bp / 128, members, 16), kRedThreads, 0, stream, a);
+}
+
+int launch_reduce_final(const RedArgs& a, int members, void* stream) {
     const int nred = red_count(a.H);
     reduce_final_kernel<<<dim3((nred + 255) / 256, members), 256, 0, (cudaStream_t)stream>>>(a);
     return ok_or(cudaGetLastError());
 }
 
 int launch_adam(const AdamArgs& a, void* stream) {
-    const long long n = a.pstride * a.members;
-    adam_kernel<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(a);
-    return ok_or(cudaGetLastError());
+    return launch_pdl(adam_kernel, dim3(128 + (red_count(a.H) + 255) / 256, a.members), 256, 0, stream, a);
 }
 
 int launch_refresh_bf16(const AdamArgs& a, void* stream) {
-    const long long n = 2ll * a.H * a.H * a.members;
-    refresh_kernel<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(a);
+    refresh_kernel<<<dim3(128, a.members), 256, 0, (cudaStream_t)stream>>>(a);
     return ok_or(cudaGetLastError());
 }
 
