@@ -167,8 +167,9 @@ typedef struct {
                             cooperative launch per up to 4096 steps whose
                             CTAs exchange their blocks' edges through
                             global memory (bounded waits: BTE_ETIMEOUT);
-                            otherwise one fused step kernel launch per
-                            step.  Both give the same bits.                */
+                            FP32 grids that do not fit take two steps per
+                            launch; otherwise one fused step kernel launch
+                            per step.  All give the same bits.             */
     int32_t walk;        /* order in which one-step launches walk the
                             harmonic rows of a work item: 0 automatic
                             (alternate when the ping-pong state exceeds 96

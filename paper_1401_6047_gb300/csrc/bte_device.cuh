@@ -276,7 +276,8 @@ __device__ __forceinline__ void cn_cell(T a, T b, T X, T Y, T cc, T hr, T g, T t
 __device__ __forceinline__ float2 pair(float x, float y) { return make_float2(x, y); }
 __device__ __forceinline__ float2 neg2(float2 v) { return make_float2(-v.x, -v.y); }
 
-template <typename T, int V>
+/* CHI1: chi is 1 (every row but n = 1), a sum in place of a multiply-add. */
+template <typename T, int V, bool CHI1 = false>
 __device__ __forceinline__ void cn_row(const T (&a)[V], const T (&b)[V], const T (&db_next)[V],
                                        const T (&db_prev)[V], const T (&da_prev)[V],
                                        const T (&da_next)[V], T cc, T chi, T hr, const T (&g)[V],
@@ -291,8 +292,8 @@ __device__ __forceinline__ void cn_row(const T (&a)[V], const T (&b)[V], const T
             const float2 A = pair(a[e], a[e + 1]), Bv = pair(b[e], b[e + 1]);
             const float2 Sa = __fmul2_rn(cc2, __fadd2_rn(pair(db_next[e], db_next[e + 1]),
                                                          neg2(pair(db_prev[e], db_prev[e + 1]))));
-            const float2 Sb = __fmul2_rn(cc2, __ffma2_rn(chi2, pair(da_prev[e], da_prev[e + 1]),
-                                                         neg2(pair(da_next[e], da_next[e + 1]))));
+            const float2 dp = pair(da_prev[e], da_prev[e + 1]), dn = neg2(pair(da_next[e], da_next[e + 1]));
+            const float2 Sb = __fmul2_rn(cc2, CHI1 ? __fadd2_rn(dp, dn) : __ffma2_rn(chi2, dp, dn));
             const float2 th = __fmul2_rn(nf2, pair(w0[e], w0[e + 1]));
             const float2 th1 = __fmul2_rn(nf2, pair(w1[e], w1[e + 1]));
             const float2 D = __ffma2_rn(th1, th1, nu2);

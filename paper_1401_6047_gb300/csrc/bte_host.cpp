@@ -198,6 +198,9 @@ struct Layout {
     size_t blk_smem, blk_words; /* shared memory per CTA; bytes of exchange words */
     int blk_steps, blk_mpad;    /* steps per launch at most; pitch of the kept rows */
     size_t off_blkx, off_blkq, off_blkrows;
+    /* two steps per launch (FP32 grids that do not fit on chip): the kept
+     * rows of blk_steps steps (a multiple of 4) at off_blkrows */
+    bool pair;
 };
 
 /* On chip, one block per SM: CTAs (the SMs of a GB300), bytes of kept rows
@@ -210,6 +213,11 @@ constexpr size_t kBlkSmemMax = 232448;
 constexpr size_t kBlkRowBytesMin = 2u << 20, kBlkRowBytesMax = 16u << 20;
 constexpr int kBlkMaxSteps = 4096;
 constexpr int kBlkMinSteps = 4;
+
+/* Two-step kernel: fewest rows of a chunk (each is read with eight more) and
+ * most (their row factors sit beside the ring; up to 192 rows leave room for
+ * three CTAs on an SM). */
+constexpr int kPairMinRows = 8, kPairMaxRows = 192;
 
 /* Blocks of the on-chip mode of one block per SM: of all row splits GR and
  * the two column-group widths V (one in FP64), the one with the least estimated time of a
@@ -431,6 +439,7 @@ int plan(const bte_params* p, const bte_tuning* t, const TimeGrid& tg, Layout& L
     }
     /* one block per SM, where the launch shape is left to the library */
     L.blkGR = 0;
+    L.pair = false;
     const bool shaped = t && (t->tile_m || t->chunk_n || t->graph_steps || t->vec || t->walk);
     if (!shaped && pick_blocks(N1, M1, L.elem, L)) {
         L.blk_mpad = (int)align_up(M1, 32);
@@ -444,6 +453,15 @@ int plan(const bte_params* p, const bte_tuning* t, const TimeGrid& tg, Layout& L
         o += align_up(L.blk_words, 256);
         L.off_blkq = o; /* cleared together with the words */
         o += 256;
+        L.off_blkrows = o;
+        o += align_up((size_t)L.blk_steps * row_bytes, 256);
+    }
+    if (!shaped && !L.blkGR && L.elem == 4 && (size_t)N1 * L.pitch < (1ull << 31)) {
+        L.pair = true;
+        L.blk_mpad = (int)align_up(M1, 32);
+        const size_t row_bytes = 2 * (size_t)L.blk_mpad * L.elem;
+        const long long steps = std::min<long long>(kBlkRowBytesMax / row_bytes, kBlkMaxSteps);
+        L.blk_steps = (int)std::max<long long>(std::min(steps, tg.K + 3) / 4 * 4, 4);
         L.off_blkrows = o;
         o += align_up((size_t)L.blk_steps * row_bytes, 256);
     }
@@ -468,6 +486,8 @@ struct bte_handle {
     int graph_len; /* steps per captured graph (a multiple of the fused step count) */
     int grid[3];   /* persistent CTAs of the step kernel fusing 1 / 2 steps */
     int grid_persist; /* CTAs of a persistent (multi-step) launch, all co-resident */
+    bool pair;     /* steps go in pairs, one launch each */
+    int pair_ntile, pair_nchunk, pair_rows;
     bool blk;      /* calls of kBlkMinSteps steps or more run on chip, one block per SM */
     int set;       /* ping-pong set holding the current state (flips per launch) */
     cudaGraphExec_t graph[2]; /* one graph per starting set */
@@ -902,8 +922,93 @@ int enqueue_blocks(bte_handle* h, long long n) {
     return BTE_OK;
 }
 
+/* Two steps per launch: graphs of blk_steps steps (an even number of
+ * launches, so the ping-pong set is the same after each; captured on first
+ * use), then launches for the pairs left, each run of them followed by the
+ * sums of the rows it kept.  Leaves an odd step to the caller. */
+bte::PairArgs pair_args(const bte_handle* h) {
+    const bte::StepArgs<float> sa = step_args<float>(h);
+    bte::PairArgs a{};
+    for (int s = 0; s < 2; ++s) {
+        a.a_w[s] = sa.a_w[s];
+        a.b_w[s] = sa.b_w[s];
+        a.a_f[s] = sa.a_f[s];
+        a.b_f[s] = sa.b_f[s];
+    }
+    a.row_a0 = sa.row_a0;
+    a.col_g = sa.col_g;
+    a.col_phi = sa.col_phi;
+    a.e_whole = sa.e_whole;
+    a.e_frac = sa.e_frac;
+    a.kept = h->ptr<float>(h->L.off_blkrows);
+    a.base = sa.base;
+    a.N = sa.N;
+    a.M = sa.M;
+    a.pitch = sa.pitch;
+    a.P = sa.P;
+    a.dstride = sa.dstride;
+    a.mpad = h->L.blk_mpad;
+    a.ntile = h->pair_ntile;
+    a.nchunk = h->pair_nchunk;
+    a.rows = h->pair_rows;
+    a.alt = sa.alt;
+    a.h = sa.h;
+    a.hh = sa.hh;
+    a.nu = sa.nu;
+    a.xi = sa.xi;
+    return a;
+}
+
+int queue_pairs(bte_handle* h, int launches, int set, cudaStream_t st) {
+    const bte::PairArgs a = pair_args(h);
+    const bte::StepArgs<float> sa = step_args<float>(h);
+    int rc = 0;
+    for (int i = 0; i < launches && !rc; ++i) rc = bte::launch_pair(a, i, set, i > 0, st);
+    if (!rc)
+        rc = bte::launch_fold_rows<float>(a.kept, a.mpad, a.M, h->L.tile_m, h->L.vec, 2 * launches, sa.vscale,
+                                          sa.nscale, a.base, sa.trace_v, sa.trace_n, st);
+    if (!rc) rc = bte::launch_advance_base(h->ptr<long long>(h->L.off_base), 2 * launches, st);
+    return rc;
+}
+
+int enqueue_pairs(bte_handle* h, long long& n) {
+    const int most = h->L.blk_steps / 2;
+    while (n >= 2 * most) {
+        const int set = h->set;
+        if (!h->graph[set]) {
+            cudaGraph_t g = nullptr;
+            CU(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
+            const int rc = queue_pairs(h, most, set, h->cap_stream);
+            cudaError_t e = cudaStreamEndCapture(h->cap_stream, &g);
+            if (!rc && e == cudaSuccess) e = cudaGraphInstantiate(&h->graph[set], g, 0);
+            if (g) cudaGraphDestroy(g);
+            if (rc || e != cudaSuccess) {
+                h->graph[set] = nullptr;
+                return fail(BTE_ECUDA, "graph of step pairs: %s",
+                            cudaGetErrorString(e != cudaSuccess ? e : (cudaError_t)rc));
+            }
+        }
+        CU(cudaGraphLaunch(h->graph[set], h->stream));
+        h->k += 2 * most;
+        n -= 2 * most;
+    }
+    if (n >= 2) {
+        const int launches = (int)(n / 2);
+        const int rc = queue_pairs(h, launches, h->set, h->stream);
+        if (rc) return fail(BTE_ECUDA, "two-step kernel: %s", cudaGetErrorString((cudaError_t)rc));
+        h->k += 2 * launches;
+        h->set ^= launches & 1;
+        n -= 2 * launches;
+    }
+    return BTE_OK;
+}
+
 template <typename T>
 int enqueue_steps(bte_handle* h, long long n) {
+    if (h->pair && n >= 2) {
+        const int rc = enqueue_pairs(h, n);
+        if (rc || n == 0) return rc;
+    }
     if (h->blk && n >= kBlkMinSteps) return enqueue_blocks<T>(h, n);
     if (h->L.resC) return n > 0 ? enqueue_resident<T>(h, n) : BTE_OK;
     if (h->L.wideG) return n > 0 ? enqueue_wide<T>(h, n) : BTE_OK;
@@ -1774,7 +1879,25 @@ int bte_create_ex(const bte_params* p, void* stream, const bte_tuning* tune, voi
             h->grid_persist = (int)items;
         }
     }
-    h->blk = false;
+    h->blk = h->pair = false;
+    if (h->L.pair && !h->L.resC && !h->L.wideG && !h->L.persist) {
+        /* about one warp per place: chunks of rows for each tile of columns */
+        int wps = 0, dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        /* the kernel's shared-memory limit covers every chunk it may be
+         * launched with; a short chunk's occupancy decides the split */
+        const int N1 = h->p.n_max + 1;
+        rc = bte::pair_configure(kPairMaxRows, &wps);
+        if (!rc) rc = bte::pair_configure(kPairMinRows, &wps, false);
+        if (rc) return bail(fail(BTE_ECUDA, "two-step kernel configure: %s", cudaGetErrorString((cudaError_t)rc)));
+        h->pair_ntile = (h->p.m_points + bte::kPairCols - 1) / bte::kPairCols;
+        int chunks = std::max(1, std::min(wps * sms / h->pair_ntile, N1 / kPairMinRows));
+        chunks = std::max(chunks, (N1 + kPairMaxRows - 1) / kPairMaxRows);
+        h->pair_rows = (N1 + chunks - 1) / chunks;
+        h->pair_nchunk = (N1 + h->pair_rows - 1) / h->pair_rows;
+        h->pair = wps > 0;
+    }
     if (h->L.blkGR && !h->L.resC && !h->L.wideG && !h->L.persist) {
         /* every block must be resident at once */
         int bps = 0, dev = 0, sms = 0, coop = 0;

@@ -196,6 +196,27 @@ struct GridArgs {
     T h, hh, nu, xi;
 };
 
+/* columns that a warp of the two-step kernel keeps (of 128: four more on
+ * each side are read and advanced for their neighbours' sake) */
+constexpr int kPairCols = 120;
+
+/* Arguments of the FP32 kernel of two steps per launch (bte_pair.cu): launch
+ * i advances steps base + 2 i, base + 2 i + 1, reading ping-pong set (parity
+ * + i) & 1 and writing the other one.  Work items: ntile tiles of kPairCols
+ * columns x nchunk chunks of `rows` rows, one warp each. */
+struct PairArgs {
+    float* a_w[2]; float* b_w[2]; float* a_f[2]; float* b_f[2];
+    const float* row_a0; const float* col_g; const float* col_phi;
+    const float* e_whole; const float* e_frac; /* drive tables as in StepArgs    */
+    float* kept;      /* [2 launches][2][mpad]: rows 0 (a) and 1 (b) of each new
+                         whole grid, for launch_fold_rows                      */
+    const long long* base;
+    int N, M, pitch, P, dstride, mpad;
+    int ntile, nchunk, rows;
+    int alt;          /* as StepArgs::alt                                      */
+    float h, hh, nu, xi;
+};
+
 /* One plain application of T (start-up half step), unfused. */
 template <typename T>
 struct ApplyArgs {
@@ -293,6 +314,10 @@ template <typename T>
 int launch_fold_rows(const T* rows, int mpad, int M, int tile_m, int vec, int K, double vscale,
                      double nscale, const long long* base, double* trace_v, double* trace_n,
                      void* stream);
+/* Two-step kernel: warps that fit an SM with chunks of `rows` rows (sets the
+ * kernel's attributes), and launch i of a run of them. */
+int pair_configure(int rows, int* warps_per_sm, bool set_limit = true);
+int launch_pair(const PairArgs& a, int i, int parity, bool pdl, void* stream);
 /* Sets the calling thread's bte_last_error() message; returns code. */
 int report_error(int code, const char* msg);
 template <typename T>
