@@ -158,8 +158,10 @@ typedef struct {
                             One thread per cell: BTE_EINVAL when a CTA's
                             block has more than 480 cells or does not fit
                             232,448 bytes, or the G clusters do not fit the
-                            GPU at once (small grids: 31 x 201 FP64 runs
-                            5.5 instead of 16.1 us per step on a GB300).
+                            GPU at once (small grids).  With wide_cols = 0
+                            and no other field set, calls of four steps or
+                            more run in the faster form of mode 0's small
+                            grids instead.
                             0: with every field of this struct zero, a
                             grid that fits the shared memory of the SMs
                             together runs there in calls of four steps or

@@ -20,13 +20,16 @@
  * exchange of edges per half-step, about 0.5 us through L2.
  *
  * Measured (GB300, us per step, one launch per step / here): 31 x 201 FP64
- * 23.0 / 3.9, FP32 9.3 / 2.0; 65 x 1000 FP64 45 / 9.4; 138 x 1533 FP32 14.4 /
- * 3.6; 120 x 4000 FP32 13.9 / 4.5; 401 x 4001 FP32 17.0 / 7.5.
+ * 23.0 / 2.9, FP32 9.3 / 2.1; 65 x 1000 FP64 45 / 7.9; 138 x 1533 FP32 14.4 /
+ * 3.3; 120 x 4000 FP32 13.9 / 3.9; 401 x 4001 FP32 17.0 / 7.2.  (With the
+ * compute threads polling: 3.9, 2.5, 9.4, 3.6, 4.5 and 7.5.)
  *
- * A half-step of a CTA:
+ * A half-step of a CTA (its last 128 threads only poll, keep rows 0 and 1 and
+ * make the next half-step's rotation factors; a poll is an L2 round trip, 700
+ * to 1000 cycles, even when the word is there, so it runs beside 1.):
  *   1. cells that read no halo (all but the block's first and last rows and
- *      column groups): they need only this CTA's own cells, so they run
- *      while the neighbours' edges are still under way;
+ *      column groups), and in FP64 the part of the boundary cells that needs
+ *      none, while the neighbours' edges are still under way;
  *   2. the halo cells of the grid that is read, polled from exchange words;
  *   3. the remaining cells; the outermost ones are published as exchange
  *      words as they are made.
@@ -164,7 +167,7 @@ __device__ __forceinline__ void publish(Words2* e, unsigned tag, T a, T b) {
 /* shared memory: arrays and factors, then the poll and boundary tables */
 template <typename T>
 __host__ __device__ inline size_t poll_offset(int R, int W, int V) {
-    const size_t b = ((4 * (size_t)(R + 2) + 2) * (W + 2 * V) + R + 2) * sizeof(T);
+    const size_t b = ((4 * (size_t)(R + 2) + 6) * (W + 2 * V) + 2 * (R + 2)) * sizeof(T);
     return (b + 15) / 16 * 16;
 }
 
@@ -187,7 +190,9 @@ __global__ void __launch_bounds__(kGridThreads, 1) grid_kernel(GridArgs<T> A) {
     T* s = reinterpret_cast<T*>(smem); /* [4][R + 2][P]: a_w, b_w, a_f, b_f */
     T* sG = s + 4 * arr;               /* [P] column factor of a0 */
     T* sPh = sG + P;                   /* [P] phi_m */
-    T* sR = sPh + P;                   /* [R + 2] h times the row factor of a0 */
+    T* sT = sPh + P;                   /* [2][2][P] rotation factors of this and the next half-step */
+    T* sR = sT + 4 * P;                /* [R + 2] h times the row factor of a0 */
+    T* sN = sR + A.R + 2;              /* [R + 2] n */
     /* the block's polls: {entry within one (buffer, grid) of the words,
      * place in an a array | column entry << 31}, and its boundary groups:
      * local row << 16 | group */
@@ -196,7 +201,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) grid_kernel(GridArgs<T> A) {
     T* const gs[4] = {A.a_w, A.b_w, A.a_f, A.b_f};
 
     /* ---- load: zero everything, then the block and its halo cells ---- */
-    for (int q = tid; q < 4 * arr + 2 * P + A.R + 2; q += nthr) s[q] = (T)0;
+    for (int q = tid; q < 4 * arr + 6 * P + 2 * (A.R + 2); q += nthr) s[q] = (T)0;
     __syncthreads();
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
@@ -219,7 +224,10 @@ __global__ void __launch_bounds__(kGridThreads, 1) grid_kernel(GridArgs<T> A) {
         sG[V + q] = A.col_g[GG + c0 + q];
         sPh[V + q] = A.col_phi[GG + c0 + q];
     }
-    for (int q = tid; q < R; q += nthr) sR[q + 1] = Rn<T>::mul(A.h, A.row_a0[r0 + q]);
+    for (int q = tid; q < R; q += nthr) {
+        sR[q + 1] = Rn<T>::mul(A.h, A.row_a0[r0 + q]);
+        sN[q + 1] = (T)(r0 + q);
+    }
     const CnK<T> cn = cn_constants<T>(A.h, A.nu, A.xi);
     const T hh = A.hh;
     Words2* const rowx = reinterpret_cast<Words2*>(A.rowx);
@@ -276,19 +284,32 @@ __global__ void __launch_bounds__(kGridThreads, 1) grid_kernel(GridArgs<T> A) {
     Words2* const left = colx + (size_t)((bj * 2) * N1 + r0) * E;
     Words2* const right = left + (size_t)N1 * E;
 
-    /* interior work starts at the threads that have no boundary group, so
-     * that in a small block different warps do the two */
-    const int cpp = max(min(nci, nthr), 1);
-    const int rsplit = nthr / cpp;
-    const int ntid = nb < nthr ? tid - round_warp(nb) + (tid < round_warp(nb) ? nthr : 0) : tid;
+    /* The last A.help threads poll.  Interior work starts at the threads that have
+     * no boundary group, so that in a small block different warps do the two. */
+    const int nc = nthr - A.help;
+    const bool comp = tid < nc;
+    const int ptid = tid - nc, pthr = A.help; /* polling threads: ptid >= 0 */
+    const int cpp = max(min(nci, nc), 1);
+    const int rsplit = nc / cpp;
+    const int ntid = nb < nc ? tid - round_warp(nb) + (tid < round_warp(nb) ? nc : 0) : tid;
     const int gl = ntid % cpp, rpart = ntid / cpp;
     const int nrow = (nri + rsplit - 1) / rsplit;
     const int lo = 1 + rpart * nrow;
-    const bool has_int = nci > 0 && nri > 0;
+    const bool has_int = nci > 0 && nri > 0 && comp;
 
     const long long k0 = *A.base;
     int kk = (int)(k0 % A.P);
     Half<T> D = half_drive<T>(A.e_whole, A.dstride, kk);
+    __syncthreads();
+    /* rotation factors of the block's columns for a half-step */
+    auto rotations = [&](T* t, const Half<T>& H, int q0, int step) {
+        for (int q = q0; q < Wb; q += step) {
+            const T ph = sPh[V + q];
+            t[V + q] = rot_factor<T>(H.E0, H.B0, ph, hh);
+            t[P + V + q] = rot_factor<T>(H.E1, H.B1, ph, hh);
+        }
+    };
+    rotations(sT, D, tid, nthr);
     __syncthreads();
 
     const long long nhs = 2ll * A.K;
@@ -299,6 +320,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) grid_kernel(GridArgs<T> A) {
         T* const so = s + (hf ? 2 * arr : 0) + V;       /* own grid, column c0 */
         const T* const sx = s + (hf ? 0 : 2 * arr) + V; /* grid that is read */
         const unsigned tag = (unsigned)hs;
+        const T* const rot = sT + (hs & 1) * 2 * P;
         /* the drive of the next half-step, long before it is needed */
         if (hf) kk = kk + 1 == A.P ? 0 : kk + 1;
         const Half<T> Dn = half_drive<T>(hf ? A.e_whole : A.e_frac, A.dstride, kk);
@@ -310,14 +332,10 @@ __global__ void __launch_bounds__(kGridThreads, 1) grid_kernel(GridArgs<T> A) {
                 const int m = (g_on ? g + 1 : 1) * V;
                 const bool l_adj = lane > 0 && gl > 0;
                 const bool r_adj = lane < 31 && gl + 1 < cpp && g + 1 < nci;
-                T gc[V], ph[V], t0[V], t1[V];
+                T gc[V], t0[V], t1[V];
                 ldv<T, V>(sG + V + m, gc);
-                ldv<T, V>(sPh + V + m, ph);
-#pragma unroll
-                for (int e = 0; e < V; ++e) {
-                    t0[e] = rot_factor<T>(D.E0, D.B0, ph[e], hh);
-                    t1[e] = rot_factor<T>(D.E1, D.B1, ph[e], hh);
-                }
+                ldv<T, V>(rot + V + m, t0);
+                ldv<T, V>(rot + P + V + m, t1);
 #pragma unroll 1
                 for (int ch = 0; ch < 2; ++ch) {
                     const int len = (nrow + 1 - ch) / 2; /* same for every thread */
@@ -343,7 +361,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) grid_kernel(GridArgs<T> A) {
                         ldv<T, V>(po, oa);
                         ldv<T, V>(po + arr, ob);
                         cn_row<T, V>(oa, ob, db_d, db_u, da_u, da_d, D.cc, n == 1 ? (T)2 : (T)1, sR[il + 1], gc,
-                                     (T)n, t0, t1, cn, an, bn);
+                                     sN[il + 1], t0, t1, cn, an, bn);
                         if (on) {
                             stv<T, V>(po, an);
                             stv<T, V>(po + arr, bn);
@@ -361,26 +379,25 @@ __global__ void __launch_bounds__(kGridThreads, 1) grid_kernel(GridArgs<T> A) {
          * leaves unchanged, for the step's sums */
         if (hf && r0 <= 1) {
             T* out = A.rows + (size_t)(hs >> 1) * 2 * A.mpad + c0;
-            for (int q = tid; q < Wb; q += nthr) {
+            for (int q = ptid; q >= 0 && q < Wb; q += pthr) {
                 if (r0 == 0) out[q] = s[P + V + q];
                 const int l1 = 1 - r0; /* local row of harmonic 1 */
                 if (l1 < R) out[A.mpad + q] = s[arr + (l1 + 1) * P + V + q];
             }
         }
         /* FP64: the part of the first boundary cell's update that needs no
-         * halo, while the edges are under way (15 of its 27 operations) */
+         * halo, while the edges are under way (11 of its 23 operations) */
         CnCoef<T> pre{};
         T preG = (T)0, preH = (T)0;
         auto own_part = [&](int il, int m, CnCoef<T>& c, T& G0, T& H0) {
             if constexpr (sizeof(T) == 8) {
-                const T nf = (T)(r0 + il), ph = sPh[V + m];
-                c = cn_coef<T>(Rn<T>::mul(nf, rot_factor<T>(D.E0, D.B0, ph, hh)),
-                               Rn<T>::mul(nf, rot_factor<T>(D.E1, D.B1, ph, hh)), cn);
+                const T nf = sN[il + 1];
+                c = cn_coef<T>(Rn<T>::mul(nf, rot[V + m]), Rn<T>::mul(nf, rot[P + V + m]), cn);
                 const T* const po = so + (il + 1) * P + m;
                 cn_own(po[0], po[arr], sR[il + 1], sG[V + m], c, cn, G0, H0);
             }
         };
-        if (sizeof(T) == 8 && tid < nb) own_part((int)(sBnd[tid] >> 16), (int)(sBnd[tid] & 0xffffu), pre, preG, preH);
+        if (sizeof(T) == 8 && comp && tid < nb) own_part((int)(sBnd[tid] >> 16), (int)(sBnd[tid] & 0xffffu), pre, preG, preH);
         /* the halo cells of the grid that is read (loaded with the block for
          * the first half-step) */
         bool ok = true;
@@ -388,7 +405,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) grid_kernel(GridArgs<T> A) {
             const uint32_t set = ((uint32_t)(hs - 1) >> 1 & 1) * 2 + (hf ? 0 : 1);
             const Words2* const rx = rowx + (size_t)set * row_set;
             const Words2* const cx = colx + (size_t)set * col_set;
-            for (int q = tid; q < nq; q += nthr) {
+            for (int q = ptid; q >= 0 && q < nq; q += pthr) {
                 const uint2 pe = sPoll[q];
                 if (pe.x == 0xffffffffu) continue;
                 const Words2* const e = ((pe.y >> 31) ? cx : rx) + pe.x;
@@ -429,10 +446,12 @@ __global__ void __launch_bounds__(kGridThreads, 1) grid_kernel(GridArgs<T> A) {
             }
             return;
         }
-        {
+        /* the next half-step's rotation factors */
+        if (!comp) rotations(sT + ((hs + 1) & 1) * 2 * P, Dn, ptid, pthr);
+        if (comp) {
             const uint32_t set = ((uint32_t)hs >> 1 & 1) * 2 + hf;
             const size_t rs = (size_t)set * row_set, cs = (size_t)set * col_set;
-            for (int u = tid; u < nb; u += nthr) {
+            for (int u = tid; u < nb; u += nc) {
                 const uint32_t be = sBnd[u];
                 const int il = (int)(be >> 16), g = (int)(be & 0xffffu);
                 const int m = g * V, n = r0 + il;
@@ -451,16 +470,12 @@ __global__ void __launch_bounds__(kGridThreads, 1) grid_kernel(GridArgs<T> A) {
                     cn_finish(oa[0], ob[0], stencil_a<T>(db_d[0], db_u[0]),
                               stencil_b<T>(n == 1 ? (T)2 : (T)1, da_u[0], da_d[0]), D.cc, preG, preH, pre, an[0], bn[0]);
                 } else {
-                    T gc[V], ph[V], t0[V], t1[V];
+                    T gc[V], t0[V], t1[V];
                     ldv<T, V>(sG + V + m, gc);
-                    ldv<T, V>(sPh + V + m, ph);
-#pragma unroll
-                    for (int e = 0; e < V; ++e) {
-                        t0[e] = rot_factor<T>(D.E0, D.B0, ph[e], hh);
-                        t1[e] = rot_factor<T>(D.E1, D.B1, ph[e], hh);
-                    }
-                    cn_row<T, V>(oa, ob, db_d, db_u, da_u, da_d, D.cc, n == 1 ? (T)2 : (T)1, sR[il + 1], gc, (T)n,
-                                 t0, t1, cn, an, bn);
+                    ldv<T, V>(rot + V + m, t0);
+                    ldv<T, V>(rot + P + V + m, t1);
+                    cn_row<T, V>(oa, ob, db_d, db_u, da_u, da_d, D.cc, n == 1 ? (T)2 : (T)1, sR[il + 1], gc,
+                                 sN[il + 1], t0, t1, cn, an, bn);
                 }
                 /* b_0 = 0 (Eq. b_boundary); columns past m = M stay zero */
 #pragma unroll

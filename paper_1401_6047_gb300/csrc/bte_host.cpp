@@ -194,7 +194,7 @@ struct Layout {
     size_t wide_words;         /* bytes of the tagged words */
     /* on chip, one block per SM (blkGR = 0: the grid does not fit): blkGR x
      * blkGC blocks of blkR rows x blkW columns, blkV columns per thread */
-    int blkGR, blkGC, blkR, blkW, blkV, blk_threads;
+    int blkGR, blkGC, blkR, blkW, blkV, blk_threads, blk_help;
     size_t blk_smem, blk_words; /* shared memory per CTA; bytes of exchange words */
     int blk_steps, blk_mpad;    /* steps per launch at most; pitch of the kept rows */
     size_t off_blkx, off_blkq, off_blkrows;
@@ -219,55 +219,66 @@ constexpr int kBlkMinSteps = 4;
  * three CTAs on an SM). */
 constexpr int kPairMinRows = 8, kPairMaxRows = 192;
 
-/* Blocks of the on-chip mode of one block per SM: of all row splits GR and
- * the two column-group widths V (one in FP64), the one with the least estimated time of a
- * half-step in cycles.  The interior cells run while the neighbours' edges
- * are under way (about 1100 cycles from a store to its poll), the boundary
- * cells after them.  FP32: a pass over one group per thread takes about 700
- * cycles, and 166 (V = 4) or 100 (V = 2) issue slots per warp and row.  FP64:
- * a warp's pass takes about 1700 cycles, however many of its lanes hold a
- * cell, and each quarter of an SM runs one at a time.  Measured on a GB300 (us per step, this choice / best of a sweep of
- * 13 row splits, both widths and 64 to 512 threads): 31 x 201 FP64 4.0 /
- * 3.8, FP32 3.1 / 2.1; 138 x 1533 FP32 4.8 / 3.8; 120 x 4000 FP32 4.8 / 4.8;
- * 401 x 4001 FP32 8.5 / 7.9; 65 x 1000 FP64 9.5 / 9.8.  False when no
- * split fits the shared memory. */
+/* Blocks of the on-chip mode of one block per SM: of all row splits GR,
+ * column-group widths V (one in FP64) and compute threads, the choice with
+ * the least estimated time of a half-step in cycles.  The interior cells run
+ * while the polling threads wait for the neighbours' edges (about 1150 cycles
+ * for one poll per thread), the boundary cells after both.
+ * FP32: a row of a thread takes about 300 cycles on its own, and 42 (V = 4)
+ * or 28 (V = 2) per warp where the warps fill the issue slots; a pass over
+ * the boundary 650 to 750.  FP64: each quarter of an SM takes about 1500
+ * cycles for a warp's cells, however many of its lanes hold one, and 900 for
+ * the part of a boundary cell that waits.
+ * Measured on a GB300 (us per step, this choice / best of a sweep of 14 row
+ * splits, both widths, 64 to 512 threads and 0 to 128 polling ones): 31 x 201
+ * FP64 2.9 / 2.8, FP32 2.1 / 2.0; 65 x 1000 FP64 7.9 / 7.9, FP32 2.3 / 2.3;
+ * 120 x 4000 FP64 39.4 / 39.4, FP32 3.9 / 3.8; 138 x 1533 FP32 3.3 / 3.1;
+ * 401 x 4001 FP32 7.2 / 7.2.  False when no split fits the shared memory. */
+constexpr int kBlkHelp = 128; /* polling threads */
 bool pick_blocks(int N1, int M1, size_t elem, Layout& L) {
+    auto cdiv = [](int a, int b) { return (a + b - 1) / b; };
     double best = 1e30;
     for (int V = elem == 8 ? 1 : 2; V <= (elem == 8 ? 1 : 4); V *= 2)
         for (int gr = 1; gr <= std::min(N1, kBlkCtas); ++gr) {
-            const int R = (N1 + gr - 1) / gr, GR = (N1 + R - 1) / R;
+            const int R = cdiv(N1, gr), GR = cdiv(N1, R);
             if (GR != gr) continue;
-            const int gc = kBlkCtas / GR;
-            const int W = ((M1 + gc - 1) / gc + V - 1) / V * V, GC = (M1 + W - 1) / W;
+            const int W = cdiv(cdiv(M1, kBlkCtas / GR), V) * V, GC = cdiv(M1, W);
             const size_t smem = elem == 8 ? bte::grid_smem_bytes<double>(R, W, V) : bte::grid_smem_bytes<float>(R, W, V);
             if (smem > kBlkSmemMax) continue;
             const int ncg = W / V, nci = std::max(ncg - 2, 0), nri = std::max(R - 2, 0);
-            const int ni = nci * nri, nb = (R >= 2 ? 2 : 1) * ncg + (ncg >= 2 ? 2 : 1) * nri;
+            const int nb = (R >= 2 ? 2 : 1) * ncg + (ncg >= 2 ? 2 : 1) * nri;
             const int nq = 2 * (W + 2) + 2 * R;
-            int thr = std::max((ni / 3 + 127) / 128 * 128, (std::max(nb, nq / 2) + 31) / 32 * 32);
-            thr = std::min(std::max(thr, 64), bte::kGridThreads);
-            double t_int = 0.0, t_bnd;
-            if (elem == 8) {
-                t_int = ni ? 1700.0 * std::max(1.0, ni / 128.0) : 0.0;
-                t_bnd = 1700.0 * std::max(1.0, nb / 128.0);
-            } else {
-                if (ni) {
-                    const int cpp = std::min(nci, thr), split = thr / cpp;
-                    const int rows = (nri + split - 1) / split, passes = (nci + cpp - 1) / cpp;
-                    t_int = std::max(330.0 * passes * (rows + 2), ni * (V == 4 ? 1.3 : 0.8));
+            const double t_x = 800.0 + 350.0 * cdiv(nq, kBlkHelp);
+            for (int thr : {64, 96, 128, 192, 256, 384}) {
+                double t_int = 0.0, t_bnd = 0.0;
+                if (nci && nri) {
+                    const int cpp = std::min(nci, thr), passes = cdiv(nci, cpp), rows = cdiv(nri, thr / cpp);
+                    const double warps = thr / 32.0;
+                    if (elem == 8)
+                        t_int = passes * (rows * std::max(warps / 4.0, 1.0) * 1500.0 + 600.0);
+                    else
+                        t_int = std::max(passes * (rows + 1) * warps * (V == 4 ? 42.0 : 28.0),
+                                         passes * (rows + 2) * (V == 4 ? 300.0 : 260.0));
                 }
-                t_bnd = (nb + thr - 1) / thr * 700.0 + 2.0 * nb;
-            }
-            const double t = std::max(t_int, 1100.0) + t_bnd + 0.5 * nq;
-            if (t < best) {
-                best = t;
-                L.blkGR = GR;
-                L.blkGC = GC;
-                L.blkR = R;
-                L.blkW = W;
-                L.blkV = V;
-                L.blk_smem = smem;
-                L.blk_threads = thr;
+                const int bp = cdiv(nb, thr);
+                if (elem == 8) {
+                    for (int i = 0; i < bp; ++i) t_bnd += 900.0 * cdiv(std::min(thr, nb - i * thr), 128);
+                    t_bnd += 800.0 * (bp - 1);
+                } else {
+                    t_bnd = V == 2 ? 650.0 * bp + nb : 750.0 * bp + 1.6 * nb;
+                }
+                const double t = std::max(t_int, t_x) + t_bnd + 0.4 * nq;
+                if (t < best) {
+                    best = t;
+                    L.blkGR = GR;
+                    L.blkGC = GC;
+                    L.blkR = R;
+                    L.blkW = W;
+                    L.blkV = V;
+                    L.blk_smem = smem;
+                    L.blk_help = kBlkHelp;
+                    L.blk_threads = thr + kBlkHelp;
+                }
             }
         }
     return best < 1e30;
@@ -902,6 +913,7 @@ int enqueue_blocks(bte_handle* h, long long n) {
     g.R = L.blkR;
     g.W = L.blkW;
     g.mpad = L.blk_mpad;
+    g.help = L.blk_help;
     g.h = sa.h;
     g.hh = sa.hh;
     g.nu = sa.nu;
@@ -1898,8 +1910,9 @@ int bte_create_ex(const bte_params* p, void* stream, const bte_tuning* tune, voi
         h->pair_nchunk = (N1 + h->pair_rows - 1) / h->pair_rows;
         h->pair = wps > 0;
     }
-    if (h->L.blkGR && !h->L.resC && !h->L.wideG && !h->L.persist) {
-        /* every block must be resident at once */
+    if (h->L.blkGR && !h->L.resC && !h->L.persist && !(h->L.wideG && tune->wide_cols)) {
+        /* every block must be resident at once (mode 3 with its shape left
+         * to the library takes this form too: 31 x 201 FP64 5.0 -> 2.9 us) */
         int bps = 0, dev = 0, sms = 0, coop = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

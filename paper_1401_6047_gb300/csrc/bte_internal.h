@@ -193,6 +193,7 @@ struct GridArgs {
     int K;            /* steps of this launch                                  */
     int N, M, pitch, P, dstride;
     int GR, GC, R, W, mpad;
+    int help;         /* the last threads, which only poll (a multiple of 32)  */
     T h, hh, nu, xi;
 };
 
