@@ -309,7 +309,7 @@ int wide_threads(int rp, int Wc) { return (rp * Wc + 31) / 32 * 32 + 32; }
 /* bytes of the on-chip mode's device record: the point's BatchInst, its
  * order entry and queue counter, and the kernel's window-sum scratch */
 constexpr size_t kResBytes = 1024;
-constexpr int kResThreads = 512; /* threads per CTA of the on-chip kernel */
+using bte::kResThreads; /* threads per CTA of the on-chip kernel */
 
 int plan(const bte_params* p, const bte_tuning* t, const TimeGrid& tg, Layout& L) {
     if (t && (t->walk < 0 || t->walk > 2)) return fail(BTE_EINVAL, "tuning.walk must be 0, 1 or 2");

@@ -128,10 +128,14 @@ struct BatchArgs {
     int alt;              /* as StepArgs::alt, for the batch's total state     */
 };
 
+/* threads per CTA of the on-chip batched kernel; the last warp holds no cell
+ * (a seventeenth warp would leave 96 registers a thread) */
+constexpr int kResThreads = 512;
+
 /* Arguments of the on-chip batched kernel (bte_resident.cu): clusters of C
  * CTAs take points order[0..count) from the queue counter; each CTA holds
- * ceil((N+1)/C) harmonic rows of its point in shared memory; the per-warp
- * partial sums start at byte red_off, after the largest point's arrays. */
+ * ceil((N+1)/C) harmonic rows of its point in shared memory; the window
+ * sums start at byte red_off, after the largest point's arrays. */
 template <typename T>
 struct ResArgs {
     const BatchInst<T>* inst;

@@ -123,20 +123,25 @@ __device__ __forceinline__ void cell_group(T* oA, T* oB, const T (&da_u)[RV<T>::
                                            const T (&da_d)[RV<T>::V], const T (&db_u)[RV<T>::V],
                                            const T (&db_d)[RV<T>::V], int n, int m0, int M, T hr,
                                            const T (&gc)[RV<T>::V], const T (&t0)[RV<T>::V],
-                                           const T (&t1)[RV<T>::V], const CnK<T>& K, T cc,
+                                           const T (&t1)[RV<T>::V], const CnK<T>& K, T cc, T nf,
                                            bool on, T* remU = nullptr, T* remD = nullptr,
                                            size_t rem_db = 0) {
     constexpr int V = RV<T>::V;
-    T oa[V], ob[V], an[V], bn[V], na[V], nb[V];
+    T oa[V], ob[V], na[V], nb[V];
     ld_vec<T>(oA, oa);
     ld_vec<T>(oB, ob);
     const T chi = (n == 1) ? (T)2 : (T)1;
-    dev::cn_row<T, V>(oa, ob, db_d, db_u, da_u, da_d, cc, chi, hr, gc, (T)n, t0, t1, K, an, bn);
+    dev::cn_row<T, V>(oa, ob, db_d, db_u, da_u, da_d, cc, chi, hr, gc, nf, t0, t1, K, na, nb);
+    if (m0 + V - 1 > M) { /* the last group's columns past m = M stay zero */
 #pragma unroll
-    for (int e = 0; e < V; ++e) {
-        const bool ok = m0 + e <= M;
-        na[e] = ok ? an[e] : (T)0;
-        nb[e] = (ok && n > 0) ? bn[e] : (T)0;
+        for (int e = 0; e < V; ++e) {
+            na[e] = m0 + e <= M ? na[e] : (T)0;
+            nb[e] = m0 + e <= M ? nb[e] : (T)0;
+        }
+    }
+    if (n == 0) {
+#pragma unroll
+        for (int e = 0; e < V; ++e) nb[e] = (T)0;
     }
     if (!on) return;
     st_vec<T>(oA, na);
@@ -161,7 +166,7 @@ __device__ __forceinline__ T* gsel(const BatchInst<T>& I, int a) {
 }
 
 template <typename T>
-__global__ void __launch_bounds__(512, 1) resident_kernel(ResArgs<T> A) {
+__global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs<T> A) {
     constexpr int V = RV<T>::V;
     constexpr int LG = V;              /* local ghost columns before m = 0 */
     constexpr int GG = Cols<T>::G;     /* global ghost columns before m = 0 */
@@ -169,10 +174,12 @@ __global__ void __launch_bounds__(512, 1) resident_kernel(ResArgs<T> A) {
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     const int C = A.C;
-    double* red = reinterpret_cast<double*>(smem + A.red_off); /* [2][32] warp partials */
-    int* s_next = reinterpret_cast<int*>(red + 64);
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    const int lane = tid & 31, warp = tid >> 5, nwarp = (nthr + 31) >> 5;
+    double* acc = reinterpret_cast<double*>(smem + A.red_off); /* [6] window sums, [4] rotation */
+    int* s_next = reinterpret_cast<int*>(acc + 10);
+    /* the last warp of every CTA holds no cell; rank 0's adds the row sums */
+    const int tid = threadIdx.x, nthr = (int)blockDim.x - 32;
+    const int lane = tid & 31;
+    const bool comp = tid < nthr, observer = rank == 0 && !comp;
 
     for (;;) {
         if (rank == 0 && tid == 0) *s_next = (int)atomicAdd(A.queue, 1u);
@@ -198,14 +205,14 @@ __global__ void __launch_bounds__(512, 1) resident_kernel(ResArgs<T> A) {
         T* sBf = sAf + arr;
         T* sG = sBf + arr; /* [P] column factor of a0 */
         T* sPh = sG + P;   /* [P] phi_m */
-        T* sR = sPh + P;   /* [rows_per + 2] row factor of a0, rows r0-1 .. r0+rows_per */
+        T* sR = sPh + P;   /* [rows_per + 2] h times the row factor of a0, rows r0-1 .. r0+rows_per */
 
         /* ---- load: zero everything, then rows r0-1 .. r1 that exist ---- */
-        for (size_t q = tid; q < 4 * arr + 2 * (size_t)P + rows_per + 2; q += nthr) sAw[q] = (T)0;
+        for (size_t q = tid; q < 4 * arr + 2 * (size_t)P + rows_per + 2; q += blockDim.x) sAw[q] = (T)0;
         __syncthreads();
         {
             const int rows = R + 2;
-            for (int q = tid; q < 4 * rows * ncg; q += nthr) {
+            for (int q = tid; q < 4 * rows * ncg; q += blockDim.x) {
                 const int a = q / (rows * ncg);
                 const int rem = q - a * rows * ncg;
                 const int li = rem / ncg, g = rem - li * ncg;
@@ -215,24 +222,20 @@ __global__ void __launch_bounds__(512, 1) resident_kernel(ResArgs<T> A) {
                 ld_vec<T>(gsel(I, a) + (size_t)n * gp + GG + g * V, v);
                 st_vec<T>(sAw + a * arr + (size_t)li * P + LG + g * V, v);
             }
-            for (int q = tid; q < ncg * V; q += nthr) {
+            for (int q = tid; q < ncg * V; q += blockDim.x) {
                 sG[LG + q] = I.col_g[GG + q];
                 sPh[LG + q] = I.col_phi[GG + q];
             }
-            for (int q = tid; q < R + 2; q += nthr) {
+            for (int q = tid; q < R + 2; q += blockDim.x) {
                 const int n = r0 - 1 + q;
-                sR[q] = (n >= 0 && n <= N) ? I.row_a0[n] : (T)0;
+                sR[q] = (n >= 0 && n <= N) ? Rn<T>::mul(h, I.row_a0[n]) : (T)0;
             }
         }
         __syncthreads();
 
-        /* window accumulators (thread 0 of rank 0) */
-        /* window accumulators in shared memory (thread 0 of rank 0 only
-         * touches them; keeping them out of every thread's registers) */
-        double* acc = red + 64 + 2; /* [6], after the warp partials and s_next */
-        double* rot = acc + 6;      /* [4]: window cos, sin and the per-step rotation */
-        if (tid == 0)
-            for (int q = 0; q < 6; ++q) acc[q] = 0.0;
+        /* window accumulators in shared memory (only the observer's first
+         * lane touches them) */
+        double* rot = acc + 6; /* [4]: window cos, sin and the per-step rotation */
         /* halo rows: shared row 0 holds row r0-1 (the last row of rank-1),
          * shared row R+1 row r1 (the first row of rank+1), both as loaded
          * and then as the neighbours push them each half-step (the four
@@ -294,8 +297,9 @@ __global__ void __launch_bounds__(512, 1) resident_kernel(ResArgs<T> A) {
                         diff_sh<T>(xa + (size_t)il * P, l_adj, r_adj, da_u);
                         diff_sh<T>(xa + arr + (size_t)il * P, l_adj, r_adj, db_u);
                     }
+                    T nf = (T)(r0 + i0); /* n of row i (rows past R - 2 store nothing) */
 #pragma unroll 1
-                    for (int ii = 0; ii < len; ++ii) {
+                    for (int ii = 0; ii < len; ++ii, nf += (T)2) {
                         const int i = i0 + 2 * ii;
                         const bool on = g_on && i < R - 1;
                         const int il = min(i, R - 2);
@@ -304,8 +308,8 @@ __global__ void __launch_bounds__(512, 1) resident_kernel(ResArgs<T> A) {
                         diff_sh<T>(xa + arr + (size_t)(il + 2) * P, l_adj, r_adj, db_d);
                         const size_t c = (size_t)(il + 1) * P + LG + m0;
                         cell_group<T>(sAw + o * arr + c, sAw + (o + 1) * arr + c, da_u, da_d, db_u,
-                                      db_d, r0 + il, m0, M, Rn<T>::mul(h, sR[il + 1]), gc, t0, t1,
-                                      cn, D.cc, on);
+                                      db_d, r0 + il, m0, M, sR[il + 1], gc, t0, t1, cn, D.cc,
+                                      nf, on);
 #pragma unroll
                         for (int e = 0; e < V; ++e) {
                             da_u[e] = da_d[e];
@@ -341,131 +345,124 @@ __global__ void __launch_bounds__(512, 1) resident_kernel(ResArgs<T> A) {
                 T* remU = (il == 0 && halo_up) ? halo_up + o * arr + LG + m0 : nullptr;
                 T* remD = (il == R - 1 && halo_dn) ? halo_dn + o * arr + LG + m0 : nullptr;
                 cell_group<T>(sAw + o * arr + c, sAw + (o + 1) * arr + c, da_u, da_d, db_u, db_d,
-                              r0 + il, m0, M, Rn<T>::mul(h, sR[il + 1]), gc, t0, t1, cn, D.cc,
+                              r0 + il, m0, M, sR[il + 1], gc, t0, t1, cn, D.cc, (T)(r0 + il),
                               true, remU, remD, arr);
             }
         };
 
-        /* split cluster barriers: a CTA signals when its rows of one grid are
-         * complete, updates its interior rows of the other grid meanwhile,
-         * and waits only before the rows that read a neighbour.  Rank 0 adds
-         * the new whole grid's rows 0 (a) and 1 (b) while the fractional
-         * half-step runs (that half-step leaves the whole grid unchanged);
-         * thread 0 folds the warp partials into the window sums after the
-         * step's last block barrier. */
-        /* drive phase (k0 + k) mod P of step k, kept as a counter */
-        int kk = PP > 0 ? (int)(I.k0 % PP) : 0;
-        /* thread 0 of rank 0: cos of the window phase 2 pi ((k + 1) mod P) / P,
-         * advanced by one rotation per step and reset to its exact value at
-         * the start of every period (rounding grows over at most P steps) */
-        int kc = PP > 0 ? 1 % PP : 0;
-        if (rank == 0 && tid == 0) {
+        /* The observer adds the new whole grid's rows 0 (a) and 1 (b) while
+         * the fractional half-step, which leaves them unchanged, runs, and
+         * folds them into the window sums: some 50 FP64 operations in a row,
+         * each about 64 cycles of a quarter of an SM, that no other warp
+         * waits for (in a computing warp they held up every step).  Local rows
+         * 0 and 1 are shared rows 1 and 2; without a row 1 (N = 0) shared row
+         * 2 is a zero halo row.  FP64 states add in FP64; FP32 states in hi +
+         * lo pairs of FP32 (FP64-grade). */
+        /* cos of the window phase 2 pi ((k + 1) mod P) / P, advanced by one
+         * rotation per step and reset to its exact value at the start of
+         * every period (rounding grows over at most P steps) */
+        int kc = PP > 0 ? (int)((I.k0 + 1) % PP) : 0;
+        if (observer && lane == 0) {
             const double two_pi = 6.283185307179586476925286766559;
+            for (int q = 0; q < 6; ++q) acc[q] = 0.0;
             rot[0] = PP > 0 ? cos(two_pi * (double)kc / (double)PP) : 1.0;
             rot[1] = PP > 0 ? sin(two_pi * (double)kc / (double)PP) : 0.0;
             rot[2] = PP > 0 ? cos(two_pi / (double)PP) : 1.0;
             rot[3] = PP > 0 ? sin(two_pi / (double)PP) : 0.0;
         }
+        auto observe = [&](long long k1) {
+            double sn, sv;
+            if constexpr (sizeof(T) == 8) {
+                double pn = 0.0, pv = 0.0;
+                for (int g = lane; g < ncg; g += 32) {
+                    T va[V], vb[V];
+                    ld_vec<T>(sAw + P + LG + g * V, va);
+                    ld_vec<T>(sBw + 2 * P + LG + g * V, vb);
+#pragma unroll
+                    for (int e = 0; e < V; ++e) {
+                        pn += (double)va[e];
+                        pv += (double)vb[e];
+                    }
+                }
+                sn = warp_sum(pn);
+                sv = warp_sum(pv);
+            } else {
+                F2 fn{0.0f, 0.0f}, fv{0.0f, 0.0f};
+                for (int g = lane; g < ncg; g += 32) {
+                    T va[V], vb[V];
+                    ld_vec<T>(sAw + P + LG + g * V, va);
+                    ld_vec<T>(sBw + 2 * P + LG + g * V, vb);
+#pragma unroll
+                    for (int e = 0; e < V; ++e) {
+                        fn = dev::f2_add1(fn, (float)va[e]);
+                        fv = dev::f2_add1(fv, (float)vb[e]);
+                    }
+                }
+                sn = warp_sum_f2(fn);
+                sv = warp_sum_f2(fv);
+            }
+            if (lane != 0) return;
+            const double vv = I.vscale * sv, nn = I.nscale * sn;
+            if (k1 > K - Kw) {
+                /* omega = 0 (P = 0): the angle omega t is 0 */
+                acc[0] += vv * rot[0];
+                acc[1] += vv;
+            }
+            if (PP > 0) {
+                if (++kc == PP) {
+                    kc = 0;
+                    rot[0] = 1.0;
+                    rot[1] = 0.0;
+                } else {
+                    const double c = rot[0], s1 = rot[1];
+                    rot[0] = c * rot[2] - s1 * rot[3];
+                    rot[1] = s1 * rot[2] + c * rot[3];
+                }
+            }
+            acc[2] = fmax(acc[2], fabs(nn - 1.0));
+            if (!isfinite(vv) || !isfinite(nn)) acc[3] = 1.0;
+            acc[4] = vv;
+            acc[5] = nn;
+            if (I.trace_v) {
+                I.trace_v[I.k0 + k1] = vv;
+                I.trace_n[I.k0 + k1] = nn;
+            }
+        };
+
+        /* split cluster barriers: a CTA signals when its rows of one grid are
+         * complete, updates its interior rows of the other grid meanwhile,
+         * and waits only before the rows that read a neighbour. */
+        /* drive phase (k0 + k) mod P of step k, kept as a counter; the next
+         * step's drive is read a step ahead */
+        int kk = PP > 0 ? (int)(I.k0 % PP) : 0;
+        Half<T> Dw = half_drive<T>(I.e_whole, I.dstride, kk), Df = half_drive<T>(I.e_frac, I.dstride, kk);
         cluster_arrive(); /* initial state loaded */
         for (long long k = 0; k < K; ++k) {
-            const Half<T> Dw = half_drive<T>(I.e_whole, I.dstride, kk);
-            const Half<T> Df = half_drive<T>(I.e_frac, I.dstride, kk);
-            /* ---- whole grid: z_w^{k+1} = T(z_w^k; S(z_f^{k+1/2})) ---- */
-            half_interior(0, 2, Dw);
-            cluster_wait();
-            half_boundary(0, 2, Dw);
-            __syncthreads();
-            cluster_arrive();
-            if (rank == 0) {
-                /* local rows 0 and 1 are shared rows 1 and 2; without a row 1
-                 * (N = 0) shared row 2 is a zero halo row.  FP64 states add in
-                 * FP64; FP32 states in hi + lo pairs of FP32 (FP64-grade) */
-                double pn, pv;
-                if constexpr (sizeof(T) == 8) {
-                    pn = 0.0;
-                    pv = 0.0;
-                    for (int g = tid; g < ncg; g += nthr) {
-                        T va[V], vb[V];
-                        ld_vec<T>(sAw + P + LG + g * V, va);
-                        ld_vec<T>(sBw + 2 * P + LG + g * V, vb);
-#pragma unroll
-                        for (int e = 0; e < V; ++e) {
-                            pn += (double)va[e];
-                            pv += (double)vb[e];
-                        }
-                    }
-                    pn = warp_sum(pn);
-                    pv = warp_sum(pv);
-                } else {
-                    F2 fn{0.0f, 0.0f}, fv{0.0f, 0.0f};
-                    for (int g = tid; g < ncg; g += nthr) {
-                        T va[V], vb[V];
-                        ld_vec<T>(sAw + P + LG + g * V, va);
-                        ld_vec<T>(sBw + 2 * P + LG + g * V, vb);
-#pragma unroll
-                        for (int e = 0; e < V; ++e) {
-                            const F2 tn = two_sum(fn.hi, (float)va[e]);
-                            fn = F2{tn.hi, __fadd_rn(fn.lo, tn.lo)};
-                            const F2 tv = two_sum(fv.hi, (float)vb[e]);
-                            fv = F2{tv.hi, __fadd_rn(fv.lo, tv.lo)};
-                        }
-                    }
-                    pn = warp_sum_f2(fn);
-                    pv = warp_sum_f2(fv);
-                }
-                if (lane == 0) {
-                    red[warp] = pn;
-                    red[32 + warp] = pv;
-                }
-            }
-            /* ---- fractional grid: z_f^{k+3/2} = T(z_f^{k+1/2}; S(z_w^{k+1})) ---- */
-            half_interior(2, 0, Df);
-            cluster_wait();
-            half_boundary(2, 0, Df);
-            __syncthreads();
-            cluster_arrive();
-            if (rank == 0 && tid == 0) {
-                double sn = 0, sv = 0;
-                for (int w = 0; w < nwarp; ++w) {
-                    sn += red[w];
-                    sv += red[32 + w];
-                }
-                const double vv = I.vscale * sv, nn = I.nscale * sn;
-                const long long k1 = k + 1;
-                if (k1 > K - Kw) {
-                    /* omega = 0 (P = 0): the angle omega t is 0 */
-                    acc[0] += vv * rot[0];
-                    acc[1] += vv;
-                }
-                if (PP > 0) {
-                    if (++kc == PP) {
-                        kc = 0;
-                        rot[0] = 1.0;
-                        rot[1] = 0.0;
-                    } else {
-                        const double c = rot[0], sn = rot[1];
-                        rot[0] = c * rot[2] - sn * rot[3];
-                        rot[1] = sn * rot[2] + c * rot[3];
-                    }
-                }
-                acc[2] = fmax(acc[2], fabs(nn - 1.0));
-                if (!isfinite(vv) || !isfinite(nn)) acc[3] = 1.0;
-                acc[4] = vv;
-                acc[5] = nn;
-                if (I.trace_v) {
-                    I.trace_v[I.k0 + k1] = vv;
-                    I.trace_n[I.k0 + k1] = nn;
-                }
-            }
             if (PP > 0 && ++kk == PP) kk = 0; /* P = 0 (omega = 0): row 0 every step */
+            const Half<T> Nw = half_drive<T>(I.e_whole, I.dstride, kk), Nf = half_drive<T>(I.e_frac, I.dstride, kk);
+            /* ---- whole grid: z_w^{k+1} = T(z_w^k; S(z_f^{k+1/2})) ---- */
+            if (comp) half_interior(0, 2, Dw);
+            cluster_wait();
+            if (comp) half_boundary(0, 2, Dw);
+            __syncthreads();
+            cluster_arrive();
+            /* ---- fractional grid: z_f^{k+3/2} = T(z_f^{k+1/2}; S(z_w^{k+1})) ---- */
+            if (comp) half_interior(2, 0, Df);
+            else if (observer) observe(k + 1);
+            cluster_wait();
+            if (comp) half_boundary(2, 0, Df);
+            __syncthreads();
+            cluster_arrive();
+            Dw = Nw;
+            Df = Nf;
         }
         cluster_wait(); /* pairs the last arrive */
 
         /* ---- results: window sums, final state ---- */
-        if (rank == 0 && tid == 0) {
+        if (observer && lane == 0) {
             for (int q = 0; q < 6; ++q) I.acc[q] = acc[q];
         }
-        for (int q = tid; q < 4 * R * ncg; q += nthr) {
+        for (int q = tid; q < 4 * R * ncg; q += blockDim.x) {
             const int a = q / (R * ncg);
             const int rem = q - a * R * ncg;
             const int i = rem / ncg, g = rem - i * ncg;
@@ -491,7 +488,7 @@ size_t resident_smem_bytes(int N, int M, int C, size_t* arrays_bytes) {
     size_t b = (4 * arr + 2 * P + rows_per + 2) * sizeof(T);
     b = (b + 15) / 16 * 16;
     if (arrays_bytes) *arrays_bytes = b;
-    return b + 64 * sizeof(double) + 16 + 10 * sizeof(double);
+    return b + 64 * sizeof(double) + 16 + 10 * sizeof(double); /* sums, queue index */
 }
 
 template <typename T>
