@@ -340,7 +340,11 @@ typedef struct bte_batch_opts {
  *     memory each) that advance in lock-step, one fused launch per time
  *     step covering every point's tiles; a point whose run is over is
  *     skipped by later launches of its batch.
- * Both give the same per-cell arithmetic; the per-step sums over phi_y are
+ * With every shape field of the options zero (tile_m, chunk_n, vec,
+ * graph_steps, walk, resident, resident_smem), points that fit no cluster run
+ * one after another as single instances instead of streamed, and few points
+ * get larger clusters than they need.
+ * All give the same per-cell arithmetic; the per-step sums over phi_y are
  * added in different orders.  out[i] receives the
  * final observables of p[i] exactly as bte_observables reports them after
  * bte_run (absorption NaN when omega == 0), with a per-point status
@@ -352,8 +356,8 @@ BTE_API int bte_batch_run(const bte_params* p, int32_t n, bte_obs* out,
                           const bte_batch_opts* opts);
 
 /* The tier bte_batch_run would give each point (same validation, no GPU
- * work): tier[i] = CTAs per cluster of the on-chip tier (1..16) or 0 when
- * p[i] is streamed.  HOST arrays; BTE_EINVAL as bte_batch_run. */
+ * work): tier[i] = CTAs per cluster of the on-chip tier (1..16; the fewest
+ * that hold the point) or 0 when p[i] fits no cluster or is streamed.  HOST arrays; BTE_EINVAL as bte_batch_run. */
 BTE_API int bte_batch_plan(const bte_params* p, int32_t n, const bte_batch_opts* opts,
                            int32_t* tier);
 

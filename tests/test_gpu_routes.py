@@ -76,3 +76,30 @@ def test_routes_replay_in_a_captured_graph():
         got = (*s.get_state(0), *s.get_state(1))
     for x, y in zip(got, want):
         assert np.array_equal(x, y)
+
+
+def _obs(o):
+    return np.array([o.v_dr, o.norm, o.v_dc_avg, o.absorption, o.norm_max_abs_err])
+
+
+def test_batched_points_that_fit_no_cluster_run_alone():
+    """Two FP64 points too large for a cluster of 16 CTAs (tier 0 of the plan)
+    among one that fits: run as single instances by default, streamed with
+    resident = 1.  FP64 sums in another order: 1e-12 relative (the norm's
+    error to 1e-13 absolute)."""
+    pts = [_params(n, m, W.FP64).replace(periods=0.05 + 0.01 * n / 90, avg_window=0.02)
+           for n, m in ((88, 1001), (30, 201), (90, 1345))]
+    assert list(bte.batch_plan(pts)) [::2] == [0, 0]
+    for o, r in zip(bte.batch_run(pts), bte.batch_run(pts, resident=1)):
+        assert o.status == r.status == bte.OK and o.step == r.step == o.steps_total
+        assert np.all(np.abs(_obs(o) - _obs(r))[:4] <= 1e-12 * np.abs(_obs(r))[:4])
+        assert abs(o.norm_max_abs_err - r.norm_max_abs_err) <= 1e-13
+
+
+@pytest.mark.parametrize("prec", [W.FP64, W.FP32_MIXED])
+def test_larger_clusters_for_few_points_give_the_same_bits(prec):
+    """Few points get larger clusters than they need; with resident_smem given
+    (here its default) they keep the smallest."""
+    pts = [_params(n, m, prec).replace(periods=0.1, avg_window=0.05) for n, m in ((60, 501), (33, 402), (9, 37))]
+    for o, r in zip(bte.batch_run(pts), bte.batch_run(pts, resident_smem=232448)):
+        assert np.array_equal(_obs(o), _obs(r))
