@@ -43,6 +43,11 @@
  * after reading it (blocks read each other's edges in both directions, the
  * corners included), so no reader can find it gone.
  *
+ * FP32 cells are updated in column pairs (cn_row), whose products and sums
+ * the compiler joins into other multiply-adds than the one-column form's;
+ * grid_kernel<float, 1> has the latter's bits, those of bte_wide.cu, for the
+ * mode that gives them.
+ *
  * Every wait is bounded by %globaltimer.  A wait that gives up sets the
  * launch's quit word, at which every other waiting CTA gives up too, and the
  * error word that the host reports as BTE_ETIMEOUT.
@@ -559,8 +564,9 @@ __global__ void fold_rows_kernel(const T* rows, int mpad, int M, int tile_m, dou
 template <typename T>
 const void* grid_fn(int vec) {
     if constexpr (sizeof(T) == 4)
-        return vec == 4 ? reinterpret_cast<const void*>(&grid_kernel<float, 4>)
-                        : reinterpret_cast<const void*>(&grid_kernel<float, 2>);
+        return vec == 4   ? reinterpret_cast<const void*>(&grid_kernel<float, 4>)
+               : vec == 2 ? reinterpret_cast<const void*>(&grid_kernel<float, 2>)
+                          : reinterpret_cast<const void*>(&grid_kernel<float, 1>);
     else
         return reinterpret_cast<const void*>(&grid_kernel<double, 1>);
 }

@@ -17,6 +17,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "../../include/bte.h"
@@ -220,7 +221,8 @@ constexpr int kBlkMinSteps = 4;
 constexpr int kPairMinRows = 8, kPairMaxRows = 192;
 
 /* Blocks of the on-chip mode of one block per SM: of all row splits GR,
- * column-group widths V (one in FP64) and compute threads, the choice with
+ * column-group widths V (one column in FP64, and where `scalar` asks for the
+ * one-column arithmetic of mode 3) and compute threads, the choice with
  * the least estimated time of a half-step in cycles.  The interior cells run
  * while the polling threads wait for the neighbours' edges (about 1150 cycles
  * for one poll per thread), the boundary cells after both.
@@ -235,10 +237,11 @@ constexpr int kPairMinRows = 8, kPairMaxRows = 192;
  * 120 x 4000 FP64 39.4 / 39.4, FP32 3.9 / 3.8; 138 x 1533 FP32 3.3 / 3.1;
  * 401 x 4001 FP32 7.2 / 7.2.  False when no split fits the shared memory. */
 constexpr int kBlkHelp = 128; /* polling threads */
-bool pick_blocks(int N1, int M1, size_t elem, Layout& L) {
+bool pick_blocks(int N1, int M1, size_t elem, bool scalar, Layout& L) {
     auto cdiv = [](int a, int b) { return (a + b - 1) / b; };
     double best = 1e30;
-    for (int V = elem == 8 ? 1 : 2; V <= (elem == 8 ? 1 : 4); V *= 2)
+    const bool one = elem == 8 || scalar;
+    for (int V = one ? 1 : 2; V <= (one ? 1 : 4); V *= 2)
         for (int gr = 1; gr <= std::min(N1, kBlkCtas); ++gr) {
             const int R = cdiv(N1, gr), GR = cdiv(N1, R);
             if (GR != gr) continue;
@@ -265,7 +268,7 @@ bool pick_blocks(int N1, int M1, size_t elem, Layout& L) {
                     for (int i = 0; i < bp; ++i) t_bnd += 900.0 * cdiv(std::min(thr, nb - i * thr), 128);
                     t_bnd += 800.0 * (bp - 1);
                 } else {
-                    t_bnd = V == 2 ? 650.0 * bp + nb : 750.0 * bp + 1.6 * nb;
+                    t_bnd = V <= 2 ? 650.0 * bp + nb : 750.0 * bp + 1.6 * nb;
                 }
                 const double t = std::max(t_int, t_x) + t_bnd + 0.4 * nq;
                 if (t < best) {
@@ -452,14 +455,19 @@ int plan(const bte_params* p, const bte_tuning* t, const TimeGrid& tg, Layout& L
     L.blkGR = 0;
     L.pair = false;
     const bool shaped = t && (t->tile_m || t->chunk_n || t->graph_steps || t->vec || t->walk);
-    if (!shaped && pick_blocks(N1, M1, L.elem, L)) {
+    /* FP32 in mode 3 keeps that mode's arithmetic, one column at a time; the
+     * words' region serves both, so that it is as large in every mode */
+    const bool mode3 = t && t->resident == 3;
+    if (!shaped && pick_blocks(N1, M1, L.elem, !mode3, L)) {
+        const size_t other = (size_t)8 * ((size_t)L.blkGR * M1 + (size_t)L.blkGC * N1) * 4 * L.elem;
+        pick_blocks(N1, M1, L.elem, mode3, L);
         L.blk_mpad = (int)align_up(M1, 32);
         const size_t row_bytes = 2 * (size_t)L.blk_mpad * L.elem;
         const size_t keep = std::min(std::max(4 * arr, kBlkRowBytesMin), kBlkRowBytesMax);
         const long long steps = std::min<long long>(keep / row_bytes, kBlkMaxSteps);
         L.blk_steps = (int)std::max<long long>(std::min(steps, tg.K), 1);
         /* 2 buffers x 2 grids x 2 sides, 16 bytes per FP32 cell, 32 per FP64 */
-        L.blk_words = (size_t)8 * ((size_t)L.blkGR * M1 + (size_t)L.blkGC * N1) * 4 * L.elem;
+        L.blk_words = std::max(other, (size_t)8 * ((size_t)L.blkGR * M1 + (size_t)L.blkGC * N1) * 4 * L.elem);
         L.off_blkx = o;
         o += align_up(L.blk_words, 256);
         L.off_blkq = o; /* cleared together with the words */
@@ -1057,23 +1065,80 @@ int enqueue_steps(bte_handle* h, long long n) {
     return BTE_OK;
 }
 
+/* f(part, parts) on a few threads (the calling one among them) when there is
+ * enough work, else f(0, 1). */
+template <class F>
+void in_parts(size_t bytes, F f) {
+    const int parts = (int)std::min<size_t>(std::min<size_t>(8, std::max(1u, std::thread::hardware_concurrency())),
+                                            bytes >> 22);
+    if (parts < 2) {
+        f(0, 1);
+        return;
+    }
+    std::vector<std::thread> others;
+    int started = 1;
+    try {
+        for (; started < parts; ++started) others.emplace_back(f, started, parts);
+    } catch (...) { /* no thread to be had: this one does the rest */
+    }
+    f(0, parts);
+    for (int i = started; i < parts; ++i) f(i, parts);
+    for (auto& t : others) t.join();
+}
+
+/* FP32 values in the second half of x's n doubles -> the n doubles, in place.
+ * The first half of the doubles covers none of the values, the next quarter
+ * only values already taken, and so on; each such stretch in parallel (one
+ * thread over a staging buffer took 7 ms for 17 million values). */
+void widen(double* x, size_t n) {
+    const float* src = reinterpret_cast<const float*>(x) + n;
+    size_t done = 0;
+    while (done < n) {
+        /* doubles up to (n + done) / 2 end at or before value `done` */
+        const size_t to = std::max((n + done) / 2, done + 1), len = to - done;
+        if (len < 64) {
+            for (; done < n; ++done) {
+                float v;
+                std::memcpy(&v, src + done, sizeof v);
+                x[done] = (double)v;
+            }
+            break;
+        }
+        in_parts(8 * len, [=](int part, int parts) {
+            const size_t lo = done + len * part / parts, hi = done + len * (part + 1) / parts;
+            double* __restrict__ d = x;
+            const float* __restrict__ f = src;
+            for (size_t q = lo; q < hi; ++q) d[q] = (double)f[q];
+        });
+        done = to;
+    }
+}
+
+/* Both arrays of one grid: FP64 straight into the caller's arrays, FP32 into
+ * their second halves and widened there. */
 template <typename T>
 int get_grid(bte_handle* h, int grid, double* a, double* b) {
     const Layout& L = h->L;
     const int set = h->set;
-    const int N1 = h->p.n_max + 1, M1 = h->p.m_points;
-    const T* da = h->ptr<T>(L.off_state[4 * set + 2 * grid + 0]);
-    const T* db = h->ptr<T>(L.off_state[4 * set + 2 * grid + 1]);
-    std::vector<T> buf((size_t)N1 * M1);
+    const size_t N1 = h->p.n_max + 1, M1 = h->p.m_points, n = N1 * M1;
+    double* const dst[2] = {a, b};
     for (int which = 0; which < 2; ++which) {
-        const T* src = which ? db : da;
-        double* dst = which ? b : a;
-        if (!dst) continue;
-        CU(cudaMemcpy2DAsync(buf.data(), M1 * sizeof(T), src + L.G, L.pitch * sizeof(T),
-                             M1 * sizeof(T), N1, cudaMemcpyDeviceToHost, h->stream));
-        CU(cudaStreamSynchronize(h->stream));
-        for (size_t q = 0; q < buf.size(); ++q) dst[q] = (double)buf[q];
+        if (!dst[which]) continue;
+        /* fresh pages are faulted in here (by several threads where there are
+         * many): a copy to pages not yet there took milliseconds */
+        in_parts(8 * n, [=](int part, int parts) {
+            volatile char* c = reinterpret_cast<volatile char*>(dst[which]);
+            for (size_t q = 8 * n * part / parts; q < 8 * n * (part + 1) / parts; q += 4096) c[q] = 0;
+        });
+        const T* src = h->ptr<T>(L.off_state[4 * set + 2 * grid + which]) + L.G;
+        T* to = sizeof(T) == 8 ? reinterpret_cast<T*>(dst[which]) : reinterpret_cast<T*>(dst[which]) + n;
+        CU(cudaMemcpy2DAsync(to, M1 * sizeof(T), src, L.pitch * sizeof(T), M1 * sizeof(T), N1, cudaMemcpyDeviceToHost,
+                             h->stream));
     }
+    CU(cudaStreamSynchronize(h->stream));
+    if (sizeof(T) == 4)
+        for (double* d : dst)
+            if (d) widen(d, n);
     return BTE_OK;
 }
 
@@ -1993,9 +2058,12 @@ int bte_create_ex(const bte_params* p, void* stream, const bte_tuning* tune, voi
         h->pair_nchunk = (N1 + h->pair_rows - 1) / h->pair_rows;
         h->pair = wps > 0;
     }
-    if (h->L.blkGR && !h->L.resC && !h->L.persist && !(h->L.wideG && tune->wide_cols)) {
-        /* every block must be resident at once (mode 3 with its shape left
-         * to the library takes this form too: 31 x 201 FP64 5.0 -> 2.9 us) */
+    if (h->L.blkGR && !h->L.resC && !h->L.persist && !(h->L.wideG && (tune->wide_cols || h->L.wideG == 1))) {
+        /* every block must be resident at once.  Mode 3 with its shape left
+         * to the library takes this form too (us per step: 31 x 201 FP64 5.0
+         * -> 2.9, FP32 3.1 -> 2.1; 48 x 256 FP32 3.2 -> 2.1), except on one
+         * cluster, which exchanges nothing through L2 (17 x 96 FP32: 2.0
+         * there, 2.2 here) */
         int bps = 0, dev = 0, sms = 0, coop = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -2085,20 +2153,18 @@ int bte_observables(bte_handle* h, bte_obs* out) {
     f.dt_eff = h->tg.dt_eff;
     f.inv_r1 = 1.0 / h->r1;
     f.out = h->ptr<double>(L.off_fin);
+    f.err = h->ptr<int>(L.off_err);
     int rc = bte::launch_finalize(f, h->stream);
     if (rc) return fail(BTE_ECUDA, "finalize kernel: %s", cudaGetErrorString((cudaError_t)rc));
-    double fin[4], vn[2];
-    int err = 0;
+    double fin[7];
     CU(cudaMemcpyAsync(fin, f.out, sizeof fin, cudaMemcpyDeviceToHost, h->stream));
-    CU(cudaMemcpyAsync(&vn[0], f.trace_v + h->k, 8, cudaMemcpyDeviceToHost, h->stream));
-    CU(cudaMemcpyAsync(&vn[1], f.trace_n + h->k, 8, cudaMemcpyDeviceToHost, h->stream));
-    CU(cudaMemcpyAsync(&err, h->ptr<int>(L.off_err), sizeof err, cudaMemcpyDeviceToHost, h->stream));
     CU(cudaStreamSynchronize(h->stream));
+    const int err = (int)fin[6];
     const bool done = h->k == h->tg.K;
     out->t = h->k * h->tg.dt_eff;
     out->step = h->k;
-    out->v_dr = vn[0];
-    out->norm = vn[1];
+    out->v_dr = fin[4];
+    out->norm = fin[5];
     out->v_dc_avg = done ? fin[1] : NAN;
     out->absorption = (done && h->p.omega > 0) ? fin[0] : NAN;
     out->norm_max_abs_err = fin[2];

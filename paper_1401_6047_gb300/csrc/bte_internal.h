@@ -241,7 +241,9 @@ struct FinalArgs {
     long long k;          /* current step: samples 0..k are valid */
     long long K, Kw, P;
     double omega, dt_eff, inv_r1;
-    double* out;          /* [4]: A, vbar, max|norm-1|, nonfinite flag */
+    const int* err;       /* error word */
+    double* out;          /* [7]: A, vbar, max|norm-1|, nonfinite flag, v and norm
+                             of step k, error word */
 };
 
 /* Kernel launchers (bte_kernels.cu). */

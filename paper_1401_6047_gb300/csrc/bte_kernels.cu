@@ -129,6 +129,9 @@ __global__ void finalize_kernel(FinalArgs A) {
         A.out[1] = s_sum[0] * inv;
         A.out[2] = s_err[0];
         A.out[3] = (double)s_bad[0];
+        A.out[4] = A.trace_v[A.k];
+        A.out[5] = A.trace_n[A.k];
+        A.out[6] = (double)*A.err;
     }
 }
 
