@@ -20,7 +20,7 @@
  * exchange of edges per half-step, about 0.5 us through L2.
  *
  * Measured (GB300, us per step, one launch per step / here): 31 x 201 FP64
- * 23.0 / 2.9, FP32 9.3 / 2.1; 65 x 1000 FP64 45 / 7.9; 138 x 1533 FP32 14.4 /
+ * 23.0 / 2.6, FP32 9.3 / 2.1; 65 x 1000 FP64 45 / 7.9; 138 x 1533 FP32 14.4 /
  * 3.3; 120 x 4000 FP32 13.9 / 3.9; 401 x 4001 FP32 17.0 / 7.2.  (With the
  * compute threads polling: 3.9, 2.5, 9.4, 3.6, 4.5 and 7.5.)
  *
@@ -317,6 +317,15 @@ __global__ void __launch_bounds__(kGridThreads, 1) grid_kernel(GridArgs<T> A) {
     rotations(sT, D, tid, nthr);
     __syncthreads();
 
+    /* FP64, where twice the boundary cells find threads: two adjacent lanes per
+     * cell, one for a and one for b (the two halves of an update are the same
+     * operations, so a warp's instruction serves both; it costs the same
+     * however few of its lanes hold a cell) */
+    const bool two = sizeof(T) == 8 && 2 * nb <= nc;
+    const bool two_on = two && comp && (tid >> 1) < nb;
+    const int ab = tid & 1;
+    const int il2 = two_on ? (int)(sBnd[tid >> 1] >> 16) : 0, m2 = two_on ? (int)(sBnd[tid >> 1] & 0xffffu) : 0;
+
     const long long nhs = 2ll * A.K;
     for (long long hs = 0; hs < nhs; ++hs) {
         /* even: whole grid z_w^{k+1} = T(z_w^k; S(z_f^{k+1/2})); odd:
@@ -402,7 +411,19 @@ __global__ void __launch_bounds__(kGridThreads, 1) grid_kernel(GridArgs<T> A) {
                 cn_own(po[0], po[arr], sR[il + 1], sG[V + m], c, cn, G0, H0);
             }
         };
-        if (sizeof(T) == 8 && comp && tid < nb) own_part((int)(sBnd[tid] >> 16), (int)(sBnd[tid] & 0xffffu), pre, preG, preH);
+        T own = (T)0, own0 = (T)0, sth1 = (T)0; /* two lanes: a and G0, or b and H0 */
+        if constexpr (sizeof(T) == 8) {
+            if (two_on) {
+                const T nf = sN[il2 + 1];
+                pre = cn_coef<T>(Rn<T>::mul(nf, rot[V + m2]), Rn<T>::mul(nf, rot[P + V + m2]), cn);
+                const T* const po = so + (il2 + 1) * P + m2;
+                own = po[ab ? arr : 0];
+                const T p = Rn<T>::mul(pre.ca, po[ab ? 0 : arr]);
+                own0 = Rn<T>::fma(ab ? (T)0 : sR[il2 + 1], sG[V + m2], Rn<T>::fma(-cn.h, own, ab ? p : -p));
+                sth1 = ab ? pre.th1 : -pre.th1;
+            }
+        }
+        if (sizeof(T) == 8 && !two && comp && tid < nb) own_part((int)(sBnd[tid] >> 16), (int)(sBnd[tid] & 0xffffu), pre, preG, preH);
         /* the halo cells of the grid that is read (loaded with the block for
          * the first half-step) */
         bool ok = true;
@@ -456,7 +477,31 @@ __global__ void __launch_bounds__(kGridThreads, 1) grid_kernel(GridArgs<T> A) {
         if (comp) {
             const uint32_t set = ((uint32_t)hs >> 1 & 1) * 2 + hf;
             const size_t rs = (size_t)set * row_set, cs = (size_t)set * col_set;
-            for (int u = tid; u < nb; u += nc) {
+            if constexpr (sizeof(T) == 8) {
+                if (two) { /* cn_finish, one half per lane */
+                    const int n = r0 + il2;
+                    T gh = (T)0;
+                    if (two_on) {
+                        const T* x = sx + (ab ? 0 : arr) + il2 * P + m2; /* row n - 1 of b (a's lane) or a */
+                        const T d_prev = x[1] - x[-1], d_next = x[2 * P + 1] - x[2 * P - 1];
+                        gh = Rn<T>::fma(D.cc, Rn<T>::fma(ab && n == 1 ? (T)2 : (T)1, ab ? d_prev : d_next,
+                                                         ab ? -d_next : -d_prev),
+                                        own0);
+                    }
+                    const T other = __shfl_xor_sync(0xffffffffu, gh, 1);
+                    if (two_on) {
+                        T v = Rn<T>::fma(Rn<T>::fma(sth1, other, gh), pre.inv, own);
+                        if (ab && n == 0) v = (T)0;
+                        so[(ab ? arr : 0) + (il2 + 1) * P + m2] = v;
+                        const unsigned vl = (unsigned)__double2loint(v), vh = (unsigned)__double2hiint(v);
+                        if (il2 == 0 && bi > 0) st_words(top + rs + m2 * E + ab, tag + 1, vl, vh);
+                        if (il2 == R - 1 && bi + 1 < A.GR) st_words(bottom + rs + m2 * E + ab, tag + 1, vl, vh);
+                        if (m2 == 0 && bj > 0) st_words(left + cs + il2 * E + ab, tag + 1, vl, vh);
+                        if (m2 == ncg - 1 && bj + 1 < A.GC) st_words(right + cs + il2 * E + ab, tag + 1, vl, vh);
+                    }
+                }
+            }
+            for (int u = two ? nb : tid; u < nb; u += nc) {
                 const uint32_t be = sBnd[u];
                 const int il = (int)(be >> 16), g = (int)(be & 0xffffu);
                 const int m = g * V, n = r0 + il;

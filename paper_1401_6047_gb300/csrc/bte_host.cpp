@@ -233,7 +233,7 @@ constexpr int kPairMinRows = 8, kPairMaxRows = 192;
  * the part of a boundary cell that waits.
  * Measured on a GB300 (us per step, this choice / best of a sweep of 14 row
  * splits, both widths, 64 to 512 threads and 0 to 128 polling ones): 31 x 201
- * FP64 2.9 / 2.8, FP32 2.1 / 2.0; 65 x 1000 FP64 7.9 / 7.9, FP32 2.3 / 2.3;
+ * FP64 2.6 / 2.6, FP32 2.1 / 2.0; 65 x 1000 FP64 8.2 / 7.9, FP32 2.3 / 2.3;
  * 120 x 4000 FP64 39.4 / 39.4, FP32 3.9 / 3.8; 138 x 1533 FP32 3.3 / 3.1;
  * 401 x 4001 FP32 7.2 / 7.2.  False when no split fits the shared memory. */
 constexpr int kBlkHelp = 128; /* polling threads */
@@ -265,7 +265,10 @@ bool pick_blocks(int N1, int M1, size_t elem, bool scalar, Layout& L) {
                 }
                 const int bp = cdiv(nb, thr);
                 if (elem == 8) {
-                    for (int i = 0; i < bp; ++i) t_bnd += 900.0 * cdiv(std::min(thr, nb - i * thr), 128);
+                    /* two lanes per cell where there are threads for it */
+                    if (2 * nb <= thr) t_bnd = 550.0 * cdiv(2 * nb, 128);
+                    else
+                        for (int i = 0; i < bp; ++i) t_bnd += 900.0 * cdiv(std::min(thr, nb - i * thr), 128);
                     t_bnd += 800.0 * (bp - 1);
                 } else {
                     t_bnd = V <= 2 ? 650.0 * bp + nb : 750.0 * bp + 1.6 * nb;
@@ -2061,7 +2064,7 @@ int bte_create_ex(const bte_params* p, void* stream, const bte_tuning* tune, voi
     if (h->L.blkGR && !h->L.resC && !h->L.persist && !(h->L.wideG && (tune->wide_cols || h->L.wideG == 1))) {
         /* every block must be resident at once.  Mode 3 with its shape left
          * to the library takes this form too (us per step: 31 x 201 FP64 5.0
-         * -> 2.9, FP32 3.1 -> 2.1; 48 x 256 FP32 3.2 -> 2.1), except on one
+         * -> 2.6, FP32 3.1 -> 2.1; 48 x 256 FP32 3.2 -> 2.1), except on one
          * cluster, which exchanges nothing through L2 (17 x 96 FP32: 2.0
          * there, 2.2 here) */
         int bps = 0, dev = 0, sms = 0, coop = 0;
