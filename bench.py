@@ -40,7 +40,7 @@ sys.path.insert(0, ROOT)
 
 METRIC = "cell-updates/s & sweep points/s at ≤1e-5 abs absorption error; % mem roofline"
 UNIT = "cell-updates/s"
-PROFILE_FILE = os.path.join(ROOT, "profiles", "fused_step_c3_fp32.md")
+PROFILE_FILE = os.path.join(ROOT, "profiles", "pair_step_c3_fp32.md")
 
 
 def workload(name: str, precision: str):
@@ -109,17 +109,41 @@ def measure_l2_gbs(dev, mb: int = 24, reps: int = 50) -> float:
 
 
 def kernel_sha() -> str:
-    """Hash of the step kernel's sources (the kernel file and the device
+    """Hash of the two-step kernel's sources (the kernel file and the device
     helpers and shared declarations it includes)."""
     h = hashlib.sha256()
-    for name in ("bte_step.cu", "bte_device.cuh", "bte_internal.h"):
+    for name in ("bte_pair.cu", "bte_device.cuh", "bte_internal.h"):
         with open(os.path.join(ROOT, "paper_1401_6047_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
 
 
+def single_route(p, elem: int):
+    """(kernel, steps per batch of kept rows) that the library chooses for a
+    single instance whose launch shape is left to it: "grid_kernel" (on chip,
+    one block per SM), "pair_kernel" (two steps per launch) or
+    "fused_step_kernel" (one)."""
+    from paper_1401_6047_gb300 import bte
+    N1, M1 = p.n_max + 1, p.m_points
+    row_bytes = 2 * -(-M1 // 32) * 32 * elem
+    _, _, K, _ = bte.time_grid(p)
+    fits = False
+    for V in ((1,) if elem == 8 else (2, 4)):
+        for gr in range(1, min(N1, 152) + 1):
+            R = -(-N1 // gr)
+            W = -(-(-(-M1 // (152 // gr))) // V) * V
+            b = ((4 * (R + 2) + 6) * (W + 2 * V) + 2 * (R + 2)) * elem
+            fits |= -(-b // 16) * 16 + 16 * (W + 2 + R) + 8 * (-(-W // V) + R) <= 232448
+    if fits:
+        arr = -(-N1 * bte.launch_shape(p)["pitch"] * elem // 256) * 256
+        return "grid_kernel", max(min(min(max(4 * arr, 2 << 20), 16 << 20) // row_bytes, 4096, K), 1)
+    if elem == 4:
+        return "pair_kernel", max(min((16 << 20) // row_bytes, 4096, K + 3) // 4 * 4, 4)
+    return "fused_step_kernel", 0
+
+
 def ncu_traffic(config_key: str):
-    """DRAM bytes per launch of the fused step kernel from the committed ncu
+    """DRAM bytes per launch of the two-step kernel from the committed ncu
     summary, or None when the summary is missing or the kernel source changed
     since it was taken."""
     try:
@@ -285,9 +309,8 @@ def run_ours(args):
     if args.on_chip:
         mode = "on-chip"
     if mode == "auto":
-        # one launch per step (graph replay, PDL): measured faster than the
-        # persistent mode also where L2 holds the state (401x4001: 17.4 vs
-        # 20.9 us per step; the Table 1 run: 14.1 vs 16.1)
+        # the form the library chooses (faster than the persistent mode also
+        # where L2 holds the state)
         mode = "streamed"
     resident = {"streamed": 0, "on-chip": 1, "persistent": 2, "on-chip-clusters": 3}[mode]
     on_chip = resident in (1, 3)
@@ -308,6 +331,20 @@ def run_ours(args):
         launches_per_solve = 3 + 2 * (-(-K // 8192)) + 1
     else:
         launches_per_solve = 3 + K + (K // graph_len) + (1 if K % graph_len else 0) + 1
+    kernel = {"on-chip": "resident_kernel", "persistent": "fused_step_kernel, persistent",
+              "on-chip-clusters": "wide_kernel", "streamed": "fused_step_kernel"}[mode]
+    if not (args.tile_m or args.chunk_n or args.graph_steps or args.vec) and resident in (0, 3):
+        route, batch = single_route(p, elem)
+        if route == "grid_kernel":
+            # set-up as above; per batch the on-chip launch, the sums of its
+            # rows and a counter update; finalize
+            kernel, on_chip = route, True
+            launches_per_solve = 3 + 3 * (-(-K // batch)) + 1
+        elif route == "pair_kernel" and resident == 0:
+            # one launch per two steps, per batch the sums and a counter
+            # update; an odd last step is one launch and a counter update
+            kernel = route
+            launches_per_solve = 3 + K // 2 + 2 * (-(-(K // 2 * 2) // batch)) + 2 * (K % 2) + 1
 
     # L2 flush buffer (larger than the 129 MB L2), written between timed steps
     flush = torch.empty(256 * 1024 * 1024 // 4, dtype=torch.float32, device=dev)
@@ -366,14 +403,15 @@ def run_ours(args):
         run_total = sum(run_ms)
     value = world * cells * K * args.steps / (total_ms * 1e-3)
 
-    # dominant kernel: the fused step; average duration of one launch over the
-    # timed region (run span / steps; includes inter-launch gaps).  On chip:
-    # one launch per solve, reported per leap-frog step for comparison
-    avg_launch_s = run_total * 1e-3 / (args.steps * K)
+    # dominant kernel: average duration of one launch over the timed region
+    # (run span / launches; includes inter-launch gaps): one or two steps, the
+    # state read and written once.  On chip: reported per leap-frog step for
+    # comparison
+    avg_launch_s = run_total * 1e-3 / (args.steps * K) * (2 if kernel == "pair_kernel" else 1)
     alg_bytes = 8 * elem * cells
     hbm_peak, peak_kind = measured_peaks()
     achieved = alg_bytes / avg_launch_s / 1e9
-    traffic = None if resident else ncu_traffic(f"{args.config}_{args.precision}")
+    traffic = None if kernel != "pair_kernel" else ncu_traffic(f"{args.config}_{args.precision}")
     if state_bytes <= L2_BYTES * 3 // 4 and not on_chip:
         # the state stays in L2 between steps: L2 bandwidth is the roof
         bound, peak = "l2", measure_l2_gbs(dev)
@@ -381,6 +419,15 @@ def run_ours(args):
     else:
         bound, peak = "hbm", hbm_peak
         peak_source = peak_kind + " hbm_gbs"
+
+    rate_unit = "GB/s"
+    if kernel == "grid_kernel":
+        # no memory traffic per step: the arithmetic is the roof (operations of
+        # a cell-update as the kernel performs them)
+        ops, rate_unit = (42, "T FP64 operations/s") if elem == 8 else (52, "T FP32 lane-ops/s")
+        bound, achieved = "alu", cells / avg_launch_s * ops / 1e12
+        peak, peak_source = (0.60, "measured FP64 rate") if elem == 8 else (
+            40.27392, "152 SMs x 128 FP32 lanes x 2070 MHz (one lane operation per lane and clock; FMA counted once)")
 
     result_obs = o
 
@@ -439,19 +486,21 @@ def run_ours(args):
                                                     "launch per 8192 steps",
                                 "persistent": "persistent: one cooperative launch per 8192 steps, "
                                               "grid barrier between steps, state in L2",
-                                "streamed": "streamed: one fused step kernel launch per step, "
-                                            "replayed from CUDA graphs"}[mode],
+                                "streamed": {"grid_kernel": "on chip, one block per SM: the grid in the "
+                                                            "SMs' shared memory together, edges "
+                                                            "exchanged through global memory",
+                                             "pair_kernel": "two steps per launch, replayed from CUDA "
+                                                            "graphs"}.get(
+                                    kernel, "streamed: one fused step kernel launch per step, "
+                                            "replayed from CUDA graphs")}[mode],
                        "absorption": result_obs.absorption, "v_dc": result_obs.v_dc_avg,
                        "norm_max_abs_err": result_obs.norm_max_abs_err,
                        "fp32_vs_fp64": fp32_error(args, result_obs)},
-            "roofline": {"bound": bound, "achieved": achieved, "peak": peak, "unit": "GB/s",
+            "roofline": {"bound": bound, "achieved": achieved, "peak": peak, "unit": rate_unit,
                          "frac": achieved / peak, "traffic": traffic,
                          "peak_source": peak_source,
-                         "hbm_frac": achieved / hbm_peak,
-                         "kernel": {"on-chip": "resident_kernel (per step)",
-                                    "on-chip-clusters": "wide_kernel (per step)",
-                                    "persistent": "fused_step_kernel, persistent (per step)",
-                                    "streamed": "fused_step_kernel"}[mode],
+                         "hbm_frac": alg_bytes / avg_launch_s / 1e9 / hbm_peak,
+                         "kernel": kernel + (" (per step)" if on_chip or mode == "persistent" else ""),
                          "alg_bytes_per_launch": alg_bytes,
                          "avg_launch_us": avg_launch_s * 1e6},
             "cpu_baseline": cpu,

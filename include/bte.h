@@ -141,7 +141,7 @@ typedef struct {
                             and reduction order as mode 0: bit-identical.
                             On a GB300 it is slower than mode 0 on the
                             grids measured (401 x 4001 FP32: 20.9 against
-                            17.4 us per step).
+                            7.2 us per step).
                             3: on chip over several clusters -- the grid
                             cut into G column blocks (one cluster of C CTAs
                             each, C as for 1) whose CTAs keep their part of

@@ -15,8 +15,8 @@
  * What bounds it: one launch per step moves the state through L2 twice and
  * walks its rows behind a block barrier each (401 x 4001 FP32: 17.4 us per
  * step); here a step moves only the blocks' edges, and what remains is the
- * arithmetic of the update (166 warp instructions per 128 cells of a
- * half-step, of which the issue slots are 44 % busy at 401 x 4001) and one
+ * arithmetic of the update (147 warp instructions per 128 cells of a
+ * half-step; the issue slots are 40 % busy at 401 x 4001) and one
  * exchange of edges per half-step, about 0.5 us through L2.
  *
  * Measured (GB300, us per step, one launch per step / here): 31 x 201 FP64

@@ -230,7 +230,7 @@ constexpr int kPairMinRows = 8, kPairMaxRows = 192;
  * or 28 (V = 2) per warp where the warps fill the issue slots; a pass over
  * the boundary 650 to 750.  FP64: each quarter of an SM takes about 1500
  * cycles for a warp's cells, however many of its lanes hold one, and 900 for
- * the part of a boundary cell that waits.
+ * the part of a boundary cell that waits (550 with two lanes per cell).
  * Measured on a GB300 (us per step, this choice / best of a sweep of 14 row
  * splits, both widths, 64 to 512 threads and 0 to 128 polling ones): 31 x 201
  * FP64 2.6 / 2.6, FP32 2.1 / 2.0; 65 x 1000 FP64 8.2 / 7.9, FP32 2.3 / 2.3;
