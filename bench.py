@@ -492,7 +492,8 @@ def run_ours(args):
                                              "pair_kernel": "two steps per launch, replayed from CUDA "
                                                             "graphs"}.get(
                                     kernel, "streamed: one fused step kernel launch per step, "
-                                            "replayed from CUDA graphs")}[mode],
+                                            "replayed from CUDA graphs")}[
+                                    "streamed" if kernel == "grid_kernel" else mode],
                        "absorption": result_obs.absorption, "v_dc": result_obs.v_dc_avg,
                        "norm_max_abs_err": result_obs.norm_max_abs_err,
                        "fp32_vs_fp64": fp32_error(args, result_obs)},

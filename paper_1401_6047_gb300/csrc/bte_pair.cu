@@ -28,7 +28,7 @@
  *
  * What bounds it now: 385 warp instructions per row of 128 columns and two
  * steps (about 320 are the update, the differences and the traffic), issued
- * in 43 % of the slots with three warps per quarter of an SM (160 registers);
+ * in 49 % of the slots with three warps per quarter of an SM (160 registers);
  * DRAM is at 56 %.  A row of a chunk's interior takes the fast form of the
  * iteration, with no test of its own; the rows at a chunk's ends take the
  * general one, which costs twice as much.
