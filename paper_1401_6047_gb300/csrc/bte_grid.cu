@@ -69,6 +69,11 @@ namespace {
 
 using namespace dev;
 
+/* groups of 32 lanes' columns that one CTA of the row sums takes: the whole
+ * row where it has no more than kFoldGroups (16384 FP32 columns), else
+ * kFoldTileGroups per CTA */
+constexpr int kFoldGroups = 128, kFoldTileGroups = 64;
+
 template <typename T, int V>
 __device__ __forceinline__ void ldv(const T* p, T (&x)[V]) {
     if constexpr (sizeof(T) * V == 16 && sizeof(T) == 4) {
@@ -569,26 +574,32 @@ __global__ void __launch_bounds__(kGridThreads, 1) grid_kernel(GridArgs<T> A) {
     }
 }
 
+/* sum of group gq (32 V columns from gq * 32 V) of a row, in every lane */
+template <typename T, int V>
+__device__ __forceinline__ double group_sum(const T* r, int gq, int M, int lane) {
+    const long long m = ((long long)gq * 32 + lane) * V;
+    double v = 0.0;
+#pragma unroll
+    for (int e = 0; e < V; ++e)
+        if (m + e <= M) v += (double)r[m + e];
+    return warp_sum(v);
+}
+
 /* Drift velocity and norm of steps base+1 .. base+K from the rows kept by
  * grid_kernel (CTA i: step base+1+i), added in the order of the one launch
  * per step kernel: lane l of a warp takes V consecutive columns in turn, the
  * warp's lanes a shuffle tree, then the warps of a tile_m tile, then the
- * tiles.  Warps here take the 32 V-column groups round robin. */
+ * tiles.  Warps here take the 32 V-column groups round robin; at most
+ * kFoldGroups groups (wider rows: the two kernels below). */
 template <typename T, int V>
 __global__ void fold_rows_kernel(const T* rows, int mpad, int M, int tile_m, double vscale, double nscale,
                                  const long long* base, double* trace_v, double* trace_n) {
-    extern __shared__ double part[]; /* [2][groups] */
+    __shared__ double part[2 * kFoldGroups];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     const int per_tile = tile_m / (32 * V), ntx = (M + tile_m) / tile_m, ng = ntx * per_tile;
     for (int q = warp; q < 2 * ng; q += nwarp) {
         const int which = q >= ng, gq = which ? q - ng : q;
-        const T* r = rows + ((size_t)blockIdx.x * 2 + which) * mpad;
-        const int m = (gq * 32 + lane) * V;
-        double v = 0.0;
-#pragma unroll
-        for (int e = 0; e < V; ++e)
-            if (m + e <= M) v += (double)r[m + e];
-        v = warp_sum(v);
+        const double v = group_sum<T, V>(rows + ((size_t)blockIdx.x * 2 + which) * mpad, gq, M, lane);
         if (lane == 0) part[q] = v;
     }
     __syncthreads();
@@ -604,6 +615,52 @@ __global__ void fold_rows_kernel(const T* rows, int mpad, int M, int tile_m, dou
         if (threadIdx.x == 0) trace_n[slot] = nscale * sum;
         else trace_v[slot] = vscale * sum;
     }
+}
+
+/* The same for rows of any width: the sums of the tiles, kFoldTileGroups
+ * groups per CTA (blockIdx.y: step), then the tiles of a step in order (one
+ * warp per row, 32 tiles loaded at a time).  A row that one CTA walks takes
+ * as long as the row is wide, however few steps there are to share the SMs
+ * (us per step with one CTA per step / so: 2 x 60001 FP32 44 / 15, 2 x 160001
+ * FP32 106 / 20, FP64 173 / 49; two steps per launch, 8 x 350000: 247 / 29). */
+template <typename T, int V>
+__global__ void __launch_bounds__(256) fold_tiles_kernel(const T* rows, int mpad, int M, int tile_m, double* tsum) {
+    __shared__ double part[2 * kFoldTileGroups];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    const int per_tile = tile_m / (32 * V), ntx = (M + tile_m) / tile_m;
+    const int tpb = kFoldTileGroups / per_tile, t0 = (int)blockIdx.x * tpb, nt = min(tpb, ntx - t0);
+    const int ng = nt * per_tile;
+    for (int q = warp; q < 2 * ng; q += nwarp) {
+        const int which = q >= ng, gq = which ? q - ng : q;
+        const double v =
+            group_sum<T, V>(rows + ((size_t)blockIdx.y * 2 + which) * mpad, t0 * per_tile + gq, M, lane);
+        if (lane == 0) part[q] = v;
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < 2 * nt; q += blockDim.x) {
+        const int which = q >= nt, t = which ? q - nt : q;
+        const double* p = part + which * ng + t * per_tile;
+        double st = 0.0;
+        for (int w = 0; w < per_tile; ++w) st += p[w];
+        tsum[((size_t)blockIdx.y * 2 + which) * ntx + t0 + t] = st;
+    }
+}
+
+__global__ void __launch_bounds__(64) fold_tail_kernel(const double* tsum, int ntx, double vscale, double nscale,
+                                                       const long long* base, double* trace_v, double* trace_n) {
+    const int lane = threadIdx.x & 31, which = threadIdx.x >> 5;
+    const double* p = tsum + ((size_t)blockIdx.x * 2 + which) * ntx;
+    double sum = 0.0, next = lane < ntx ? p[lane] : 0.0;
+    for (int t = 0; t < ntx; t += 32) {
+        const double v = next;
+        next = t + 32 + lane < ntx ? p[t + 32 + lane] : 0.0;
+        const int n = min(32, ntx - t);
+        for (int i = 0; i < n; ++i) sum += __shfl_sync(0xffffffffu, v, i);
+    }
+    if (lane != 0) return;
+    const long long slot = *base + 1 + blockIdx.x;
+    if (which == 0) trace_n[slot] = nscale * sum;
+    else trace_v[slot] = vscale * sum;
 }
 
 template <typename T>
@@ -652,16 +709,24 @@ int launch_grid(const GridArgs<T>& a, int vec, int threads, size_t smem, void* s
     return (int)cudaLaunchKernelExC(&cfg, fn, args);
 }
 
+size_t fold_scratch_bytes(int M, int tile_m, int vec, int K) {
+    const size_t ntx = ((size_t)M + tile_m) / tile_m;
+    return ntx * (tile_m / (32 * vec)) > (size_t)kFoldGroups ? (size_t)K * 2 * ntx * sizeof(double) : 0;
+}
+
 template <typename T>
 int launch_fold_rows(const T* rows, int mpad, int M, int tile_m, int vec, int K, double vscale, double nscale,
-                     const long long* base, double* trace_v, double* trace_n, void* stream) {
-    const int ng = (M + tile_m) / tile_m * (tile_m / (32 * vec));
-    const size_t smem = 2 * (size_t)ng * sizeof(double);
+                     const long long* base, double* trace_v, double* trace_n, double* tsum, void* stream) {
+    constexpr int V = sizeof(T) == 4 ? 4 : 2;
     cudaStream_t st = (cudaStream_t)stream;
-    if constexpr (sizeof(T) == 4)
-        fold_rows_kernel<float, 4><<<K, 256, smem, st>>>(rows, mpad, M, tile_m, vscale, nscale, base, trace_v, trace_n);
-    else
-        fold_rows_kernel<double, 2><<<K, 256, smem, st>>>(rows, mpad, M, tile_m, vscale, nscale, base, trace_v, trace_n);
+    if (vec != V || tile_m % (32 * V) || tile_m / (32 * V) > kFoldTileGroups) return (int)cudaErrorInvalidValue;
+    if (fold_scratch_bytes(M, tile_m, vec, K) == 0) {
+        fold_rows_kernel<T, V><<<K, 256, 0, st>>>(rows, mpad, M, tile_m, vscale, nscale, base, trace_v, trace_n);
+    } else {
+        const int ntx = (int)(((long long)M + tile_m) / tile_m), tpb = kFoldTileGroups / (tile_m / (32 * V));
+        fold_tiles_kernel<T, V><<<dim3((ntx + tpb - 1) / tpb, K), 256, 0, st>>>(rows, mpad, M, tile_m, tsum);
+        fold_tail_kernel<<<K, 64, 0, st>>>(tsum, ntx, vscale, nscale, base, trace_v, trace_n);
+    }
     return (int)cudaGetLastError();
 }
 
@@ -670,7 +735,7 @@ int launch_fold_rows(const T* rows, int mpad, int M, int tile_m, int vec, int K,
     template int grid_configure<T>(int, size_t, int, int*);                                              \
     template int launch_grid<T>(const GridArgs<T>&, int, int, size_t, void*);                            \
     template int launch_fold_rows<T>(const T*, int, int, int, int, int, double, double, const long long*, \
-                                     double*, double*, void*);
+                                     double*, double*, double*, void*);
 BTE_GRID_INSTANTIATE(float)
 BTE_GRID_INSTANTIATE(double)
 

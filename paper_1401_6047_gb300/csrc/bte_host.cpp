@@ -198,7 +198,7 @@ struct Layout {
     int blkGR, blkGC, blkR, blkW, blkV, blk_threads, blk_help;
     size_t blk_smem, blk_words; /* shared memory per CTA; bytes of exchange words */
     int blk_steps, blk_mpad;    /* steps per launch at most; pitch of the kept rows */
-    size_t off_blkx, off_blkq, off_blkrows;
+    size_t off_blkx, off_blkq, off_blkrows, off_fold; /* off_fold: scratch of the row sums */
     /* two steps per launch (FP32 grids that do not fit on chip): the kept
      * rows of blk_steps steps (a multiple of 4) at off_blkrows */
     bool pair;
@@ -487,6 +487,8 @@ int plan(const bte_params* p, const bte_tuning* t, const TimeGrid& tg, Layout& L
         L.off_blkrows = o;
         o += align_up((size_t)L.blk_steps * row_bytes, 256);
     }
+    L.off_fold = o;
+    if (L.blkGR || L.pair) o += align_up(bte::fold_scratch_bytes(M1 - 1, L.tile_m, L.vec, L.blk_steps), 256);
     L.total = o;
     return BTE_OK;
 }
@@ -942,7 +944,7 @@ int enqueue_blocks(bte_handle* h, long long n) {
         int rc = bte::launch_grid<T>(g, L.blkV, L.blk_threads, L.blk_smem, h->stream);
         if (!rc)
             rc = bte::launch_fold_rows<T>(g.rows, g.mpad, g.M, L.tile_m, L.vec, c, sa.vscale, sa.nscale, g.base,
-                                          sa.trace_v, sa.trace_n, h->stream);
+                                          sa.trace_v, sa.trace_n, h->ptr<double>(L.off_fold), h->stream);
         if (!rc) rc = bte::launch_advance_base(h->ptr<long long>(L.off_base), c, h->stream);
         if (rc) return fail(BTE_ECUDA, "on-chip step kernel: %s", cudaGetErrorString((cudaError_t)rc));
         h->k += c;
@@ -995,7 +997,7 @@ int queue_pairs(bte_handle* h, int launches, int set, cudaStream_t st) {
     for (int i = 0; i < launches && !rc; ++i) rc = bte::launch_pair(a, i, set, i > 0, st);
     if (!rc)
         rc = bte::launch_fold_rows<float>(a.kept, a.mpad, a.M, h->L.tile_m, h->L.vec, 2 * launches, sa.vscale,
-                                          sa.nscale, a.base, sa.trace_v, sa.trace_n, st);
+                                          sa.nscale, a.base, sa.trace_v, sa.trace_n, h->ptr<double>(h->L.off_fold), st);
     if (!rc) rc = bte::launch_advance_base(h->ptr<long long>(h->L.off_base), 2 * launches, st);
     return rc;
 }

@@ -320,7 +320,9 @@ int launch_grid(const GridArgs<T>& a, int vec, int threads, size_t smem, void* s
 template <typename T>
 int launch_fold_rows(const T* rows, int mpad, int M, int tile_m, int vec, int K, double vscale,
                      double nscale, const long long* base, double* trace_v, double* trace_n,
-                     void* stream);
+                     double* tsum, void* stream);
+/* bytes at tsum that the sums of K steps' rows need (0: none) */
+size_t fold_scratch_bytes(int M, int tile_m, int vec, int K);
 /* Two-step kernel: warps that fit an SM with chunks of `rows` rows (sets the
  * kernel's attributes), and launch i of a run of them. */
 int pair_configure(int rows, int* warps_per_sm, bool set_limit = true);

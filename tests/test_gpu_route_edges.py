@@ -1,0 +1,50 @@
+"""The kernels that the library chooses by the grid's size, where the choice
+or its bookkeeping can go wrong: very wide rows, grids near the on-chip limit,
+a constant drive, captured calls, several handles at once."""
+import threading
+
+import numpy as np
+import pytest
+
+from paper_1401_6047_gb300 import bte
+from paper_1401_6047_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _params(n_max, m_points, prec=W.FP32_MIXED, omega=2.2, periods=1.5, **kw):
+    L = max(9.0, 0.01 * m_points)
+    if omega == 0.0:
+        kw.update(t_max=2.0)
+    return W.Params(E_dc=1.4, E_omega=0.7, omega=omega, B=2.6, mu=1.7, n_max=n_max, m_points=m_points,
+                    phiy_min=-L, phiy_max=L, dt=2e-3, periods=periods * omega / 2.2, avg_window=0.05, precision=prec,
+                    B_omega=0.3, B_phase=0.4, **kw)
+
+
+def _state(s):
+    return (*s.get_state(0), *s.get_state(1))
+
+
+def _run(p, steps, **kw):
+    st = W.random_state(p, seed=p.n_max)
+    with bte.Solver(p, **kw) as s:
+        s.set_state(0, st[0], st[1])
+        s.set_state(1, st[2], st[3])
+        for k in steps:
+            s.step(k)
+        return (*_state(s), *s.trace())
+
+
+def _equal(got, want):
+    return all(np.array_equal(x, y) for x, y in zip(got, want))
+
+
+# rows of more columns than one CTA of the row sums takes (16384 FP32, 8192
+# FP64), one past a whole number of its pieces, and more than 393216 columns,
+# whose sums once asked for more shared memory than a launch may
+@pytest.mark.parametrize("shape,prec", [((19, 400001), W.FP32_MIXED), ((20, 98305), W.FP32_MIXED),
+                                        ((2, 16385), W.FP32_MIXED), ((1, 60001), W.FP32_MIXED),
+                                        ((9, 8193), W.FP64), ((3, 50001), W.FP64)])
+def test_wide_rows_equal_one_launch_per_step(shape, prec):
+    p = _params(*shape, prec)
+    assert _equal(_run(p, (4, 5, 18)), _run(p, (4, 5, 18), graph_steps=16))
