@@ -956,7 +956,7 @@ int enqueue_blocks(bte_handle* h, long long n) {
 /* Two steps per launch: graphs of blk_steps steps (an even number of
  * launches, so the ping-pong set is the same after each; captured on first
  * use), then launches for the pairs left, each run of them followed by the
- * sums of the rows it kept.  Leaves an odd step to the caller. */
+ * sums of the rows it kept.  Leaves the steps that go singly to the caller. */
 bte::PairArgs pair_args(const bte_handle* h) {
     const bte::StepArgs<float> sa = step_args<float>(h);
     bte::PairArgs a{};
@@ -1002,50 +1002,63 @@ int queue_pairs(bte_handle* h, int launches, int set, cudaStream_t st) {
     return rc;
 }
 
-int enqueue_pairs(bte_handle* h, long long& n) {
+/* whether the caller is capturing the handle's stream into a graph */
+bool capturing(const bte_handle* h) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess) cudaGetLastError();
+    return st == cudaStreamCaptureStatusActive;
+}
+
+/* Every pair flips the ping-pong set, so a captured call takes as many pairs
+ * as leave an even number of flips with the single steps after them: its
+ * replays then start from the set that the one before them ended on.  It
+ * launches no graph of the handle's own, which a capture does not take. */
+int enqueue_pairs(bte_handle* h, long long& n, bool capture) {
     const int most = h->L.blk_steps / 2;
-    while (n >= 2 * most) {
-        const int set = h->set;
-        if (!h->graph[set]) {
-            cudaGraph_t g = nullptr;
-            const int bc = begin_capture(h);
-            if (bc) return bc;
-            const int rc = queue_pairs(h, most, set, h->cap_stream);
-            cudaError_t e = cudaStreamEndCapture(h->cap_stream, &g);
-            if (!rc && e == cudaSuccess) e = cudaGraphInstantiate(&h->graph[set], g, 0);
-            if (g) cudaGraphDestroy(g);
-            if (rc || e != cudaSuccess) {
-                h->graph[set] = nullptr;
-                return fail(BTE_ECUDA, "graph of step pairs: %s",
-                            cudaGetErrorString(e != cudaSuccess ? e : (cudaError_t)rc));
+    long long pairs = n / 2;
+    if (capture && ((n - pairs) & 1)) --pairs;
+    while (pairs > 0) {
+        const int c = (int)std::min<long long>(pairs, most), set = h->set;
+        if (c == most && !capture) {
+            if (!h->graph[set]) {
+                cudaGraph_t g = nullptr;
+                const int bc = begin_capture(h);
+                if (bc) return bc;
+                const int rc = queue_pairs(h, most, set, h->cap_stream);
+                cudaError_t e = cudaStreamEndCapture(h->cap_stream, &g);
+                if (!rc && e == cudaSuccess) e = cudaGraphInstantiate(&h->graph[set], g, 0);
+                if (g) cudaGraphDestroy(g);
+                if (rc || e != cudaSuccess) {
+                    h->graph[set] = nullptr;
+                    return fail(BTE_ECUDA, "graph of step pairs: %s",
+                                cudaGetErrorString(e != cudaSuccess ? e : (cudaError_t)rc));
+                }
             }
+            CU(cudaGraphLaunch(h->graph[set], h->stream));
+        } else {
+            const int rc = queue_pairs(h, c, set, h->stream);
+            if (rc) return fail(BTE_ECUDA, "two-step kernel: %s", cudaGetErrorString((cudaError_t)rc));
         }
-        CU(cudaGraphLaunch(h->graph[set], h->stream));
-        h->k += 2 * most;
-        n -= 2 * most;
-    }
-    if (n >= 2) {
-        const int launches = (int)(n / 2);
-        const int rc = queue_pairs(h, launches, h->set, h->stream);
-        if (rc) return fail(BTE_ECUDA, "two-step kernel: %s", cudaGetErrorString((cudaError_t)rc));
-        h->k += 2 * launches;
-        h->set ^= launches & 1;
-        n -= 2 * launches;
+        h->k += 2 * c;
+        h->set ^= c & 1;
+        pairs -= c;
+        n -= 2 * c;
     }
     return BTE_OK;
 }
 
 template <typename T>
 int enqueue_steps(bte_handle* h, long long n) {
+    const bool capture = capturing(h);
     if (h->pair && n >= 2) {
-        const int rc = enqueue_pairs(h, n);
+        const int rc = enqueue_pairs(h, n, capture);
         if (rc || n == 0) return rc;
     }
     if (h->blk && n >= kBlkMinSteps) return enqueue_blocks<T>(h, n);
     if (h->L.resC) return n > 0 ? enqueue_resident<T>(h, n) : BTE_OK;
     if (h->L.wideG) return n > 0 ? enqueue_wide<T>(h, n) : BTE_OK;
     if (h->L.persist) return enqueue_persist<T>(h, n);
-    while (h->graph_len >= 2 && n >= h->graph_len) {
+    while (!capture && h->graph_len >= 2 && n >= h->graph_len) {
         const int set = h->set;
         if (!h->graph[set]) {
             int rc = capture_graph<T>(h, set);

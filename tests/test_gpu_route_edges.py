@@ -48,3 +48,29 @@ def _equal(got, want):
 def test_wide_rows_equal_one_launch_per_step(shape, prec):
     p = _params(*shape, prec)
     assert _equal(_run(p, (4, 5, 18)), _run(p, (4, 5, 18), graph_steps=16))
+
+
+# two steps per launch: an odd number of pairs, of steps, and more steps than
+# the handle keeps rows for (16 at 120001 columns); on chip: in place; one
+# launch per step, shorter and longer than the handle's own graphs
+@pytest.mark.parametrize("shape,n,kw", [((999, 2520), 2, {}), ((999, 2520), 3, {}), ((999, 2520), 5, {}),
+                                        ((999, 2520), 6, {}), ((999, 2520), 8, {}), ((19, 120001), 16, {}),
+                                        ((19, 120001), 42, {}), ((30, 201), 7, {}),
+                                        ((30, 201), 40, dict(graph_steps=16))])
+def test_captured_calls_replay(shape, n, kw):
+    torch = pytest.importorskip("torch")
+    p = _params(*shape)
+    with bte.Solver(p, **kw) as ref:
+        ref.step(4 + 3 * n)
+        want = _state(ref)
+    stream = torch.cuda.Stream()
+    with bte.Solver(p, stream=stream.cuda_stream, **kw) as s:
+        s.step(4)
+        s.observables(check=False)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            s.step(n)
+        for _ in range(3):
+            g.replay()
+        torch.cuda.synchronize()
+        assert _equal(_state(s), want)
