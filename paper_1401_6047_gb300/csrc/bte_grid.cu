@@ -684,17 +684,13 @@ size_t grid_smem_bytes(int R, int W, int vec) {
 template <typename T>
 int grid_configure(int vec, size_t smem, int threads, int* blocks_per_sm) {
     const void* fn = grid_fn<T>(vec);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
     if (e != cudaSuccess) return (int)e;
     return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, threads, smem);
 }
 
 template <typename T>
 int launch_grid(const GridArgs<T>& a, int vec, int threads, size_t smem, void* stream) {
-    /* the attribute is per function: another handle may have set less */
-    const void* fn = grid_fn<T>(vec);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return (int)e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(a.GR * a.GC);
     cfg.blockDim = dim3(threads);
@@ -706,7 +702,7 @@ int launch_grid(const GridArgs<T>& a, int vec, int threads, size_t smem, void* s
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     void* args[1] = {const_cast<GridArgs<T>*>(&a)};
-    return (int)cudaLaunchKernelExC(&cfg, fn, args);
+    return (int)cudaLaunchKernelExC(&cfg, grid_fn<T>(vec), args);
 }
 
 size_t fold_scratch_bytes(int M, int tile_m, int vec, int K) {

@@ -210,7 +210,7 @@ struct Layout {
  * one per cent), and the fewest steps of a call for which the launch, the
  * load of the blocks and the fold are worth it. */
 constexpr int kBlkCtas = 152;
-constexpr size_t kBlkSmemMax = 232448;
+constexpr size_t kBlkSmemMax = bte::kSmemMax;
 constexpr size_t kBlkRowBytesMin = 2u << 20, kBlkRowBytesMax = 16u << 20;
 constexpr int kBlkMaxSteps = 4096;
 constexpr int kBlkMinSteps = 4;
@@ -301,7 +301,7 @@ constexpr long long kPersistMaxSteps = 8192;
  * step with 7 clusters against 7.1-8.6 with 4; FP32 3.4-3.5 with 2 against
  * 3.5-3.9 with 4) -- with at most 128 CTAs in all, and at create time no
  * more clusters than fit the GPU at once */
-constexpr size_t kWideSmemMax = 232448;
+constexpr size_t kWideSmemMax = bte::kSmemMax;
 constexpr int kWideMaxClusters = 32;
 constexpr int kWideAutoCtas = 128;
 constexpr int kWideMaxCells = bte::kWideMaxThreads - 32; /* a block's cells: one thread each, plus a warp */
@@ -809,11 +809,7 @@ int enqueue_resident(bte_handle* h, long long n) {
     ra.queue = reinterpret_cast<unsigned*>(res + 452);
     ra.C = L.resC;
     ra.red_off = L.res_arrays;
-    /* the kernel's shared-memory attribute is per function: another handle or
-     * a batched run may have set it since this handle was created */
-    int clusters = 0;
-    int rc = bte::resident_max_clusters<T>(L.resC, L.res_smem, kResThreads, &clusters);
-    if (!rc) rc = bte::launch_resident<T>(ra, 1, kResThreads, L.res_smem, h->stream);
+    int rc = bte::launch_resident<T>(ra, 1, kResThreads, L.res_smem, h->stream);
     if (!rc) rc = bte::launch_advance_base(h->ptr<long long>(L.off_base), n, h->stream);
     if (rc) return fail(BTE_ECUDA, "on-chip step kernel: %s", cudaGetErrorString((cudaError_t)rc));
     h->k += n;
@@ -2063,11 +2059,9 @@ int bte_create_ex(const bte_params* p, void* stream, const bte_tuning* tune, voi
         int wps = 0, dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        /* the kernel's shared-memory limit covers every chunk it may be
-         * launched with; a short chunk's occupancy decides the split */
+        /* a short chunk's occupancy decides the split */
         const int N1 = h->p.n_max + 1;
-        rc = bte::pair_configure(kPairMaxRows, &wps);
-        if (!rc) rc = bte::pair_configure(kPairMinRows, &wps, false);
+        rc = bte::pair_configure(kPairMinRows, &wps);
         if (rc) return bail(fail(BTE_ECUDA, "two-step kernel configure: %s", cudaGetErrorString((cudaError_t)rc)));
         h->pair_ntile = (h->p.m_points + bte::kPairCols - 1) / bte::kPairCols;
         int chunks = std::max(1, std::min(wps * sms / h->pair_ntile, N1 / kPairMinRows));

@@ -38,6 +38,12 @@ struct Cols {
 template <typename T>
 constexpr int kDriveRows = sizeof(T) == 8 ? 5 : 3;
 
+/* Shared memory that one block may ask for.  A kernel's limit is a property of
+ * the function, shared by every handle and host thread, so every place that
+ * sets one sets this: with a handle's own size there, a handle made later (or
+ * by another thread) with a smaller block made the first one's launches fail. */
+constexpr int kSmemMax = 232448;
+
 /* Ping-pong state above this many bytes does not stay in L2 (129 MB on a
  * GB300) from one step to the next: the step kernel then alternates the
  * direction of its row walks, so that each step starts with the rows the
@@ -325,7 +331,7 @@ int launch_fold_rows(const T* rows, int mpad, int M, int tile_m, int vec, int K,
 size_t fold_scratch_bytes(int M, int tile_m, int vec, int K);
 /* Two-step kernel: warps that fit an SM with chunks of `rows` rows (sets the
  * kernel's attributes), and launch i of a run of them. */
-int pair_configure(int rows, int* warps_per_sm, bool set_limit = true);
+int pair_configure(int rows, int* warps_per_sm);
 int launch_pair(const PairArgs& a, int i, int parity, bool pdl, void* stream);
 /* Sets the calling thread's bte_last_error() message; returns code. */
 int report_error(int code, const char* msg);

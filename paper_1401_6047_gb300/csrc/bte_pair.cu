@@ -375,17 +375,14 @@ __global__ void __launch_bounds__(kPairWarps * 32, 3) pair_kernel(PairArgs A, in
 
 }  // namespace
 
-int pair_configure(int rows, int* warps_per_sm, bool set_limit) {
-    const size_t smem = (size_t)kPairWarps * warp_bytes(rows);
+int pair_configure(int rows, int* warps_per_sm) {
     for (const void* fn : {reinterpret_cast<const void*>(&pair_kernel<false>), reinterpret_cast<const void*>(&pair_kernel<true>)}) {
-        if (!set_limit) break;
-        const cudaError_t e =
-            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
         if (e != cudaSuccess) return (int)e;
     }
     int blocks = 0;
     const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, pair_kernel<false>, kPairWarps * 32,
-                                                                        smem);
+                                                                        (size_t)kPairWarps * warp_bytes(rows));
     *warps_per_sm = blocks * kPairWarps;
     return (int)e;
 }

@@ -494,7 +494,7 @@ size_t resident_smem_bytes(int N, int M, int C, size_t* arrays_bytes) {
 template <typename T>
 int resident_max_clusters(int C, size_t smem, int threads, int* clusters) {
     cudaError_t e = cudaFuncSetAttribute(resident_kernel<T>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
     if (e == cudaSuccess && C > 8)
         e = cudaFuncSetAttribute(resident_kernel<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return (int)e;

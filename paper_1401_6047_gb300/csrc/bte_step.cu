@@ -822,11 +822,11 @@ static int configure(int tile_m, int chunk_n, int vec, int* blocks_per_sm) {
     const size_t bytes = step_smem_bytes<T>(tile_m, chunk_n, vec);
     const void* fn = step_fn<T, BATCH, PERSIST, false>(vec);
     cudaError_t e =
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
     if (e != cudaSuccess) return (int)e;
     if (!PERSIST) {
         e = cudaFuncSetAttribute(step_fn<T, BATCH, PERSIST, true>(vec),
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
         if (e != cudaSuccess) return (int)e;
     }
     int nb = 0;

@@ -369,7 +369,7 @@ size_t wide_smem_bytes(int rows_per, int Wc) {
 template <typename T>
 int wide_max_clusters(int C, size_t smem, int threads, int* clusters) {
     auto fn = wide_kernel<T>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
     if (e == cudaSuccess && C > 8)
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return (int)e;

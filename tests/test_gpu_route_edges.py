@@ -74,3 +74,42 @@ def test_captured_calls_replay(shape, n, kw):
             g.replay()
         torch.cuda.synchronize()
         assert _equal(_state(s), want)
+
+
+# pairs of launch shapes whose shared memory differs: the first handle's calls
+# after the second handle is made
+@pytest.mark.parametrize("first,second", [(((400, 2001), dict(tile_m=768, chunk_n=64)), ((30, 201), dict(tile_m=32, chunk_n=8))),
+                                          (((400, 4001), {}), ((8, 37), {})),
+                                          (((60, 501), dict(resident=1)), ((30, 201), dict(resident=1))),
+                                          (((60, 201), dict(resident=3, wide_cols=100)), ((30, 201), dict(resident=3, wide_cols=20)))])
+def test_a_later_handle_leaves_an_earlier_one_running(first, second):
+    with bte.Solver(_params(*first[0]), **first[1]) as a:
+        with bte.Solver(_params(*second[0]), **second[1]) as b:
+            for s in (b, a, b, a):
+                s.step(3)
+                s.step(8)
+                assert s.observables(check=False).status == bte.OK
+
+
+def test_handles_on_several_threads():
+    """Each thread makes and steps its own handles; the launches of one are
+    not refused for what another thread's handle needs."""
+    errors = []
+
+    def work(shape):
+        try:
+            for _ in range(6):
+                with bte.Solver(_params(*shape, periods=20.0)) as s:
+                    for _ in range(40):
+                        s.step(8)
+                        s.step(2)
+                    s.observables()
+        except bte.BteError as e:
+            errors.append(f"{shape}: {e}")
+
+    threads = [threading.Thread(target=work, args=(sh,)) for sh in ((119, 4000), (8, 37), (60, 1000), (30, 201))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors
