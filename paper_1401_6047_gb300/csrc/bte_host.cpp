@@ -458,19 +458,21 @@ int plan(const bte_params* p, const bte_tuning* t, const TimeGrid& tg, Layout& L
     L.blkGR = 0;
     L.pair = false;
     const bool shaped = t && (t->tile_m || t->chunk_n || t->graph_steps || t->vec || t->walk);
-    /* FP32 in mode 3 keeps that mode's arithmetic, one column at a time; the
-     * words' region serves both, so that it is as large in every mode */
+    /* FP32 in mode 3 keeps that mode's arithmetic, one column at a time; a
+     * grid that fits only in the other form has none here.  The words' region
+     * serves both, so that it is as large in every mode */
     const bool mode3 = t && t->resident == 3;
-    if (!shaped && pick_blocks(N1, M1, L.elem, !mode3, L)) {
-        const size_t other = (size_t)8 * ((size_t)L.blkGR * M1 + (size_t)L.blkGC * N1) * 4 * L.elem;
-        pick_blocks(N1, M1, L.elem, mode3, L);
+    /* 2 buffers x 2 grids x 2 sides, 16 bytes per FP32 cell, 32 per FP64 */
+    auto words = [&](const Layout& B) { return (size_t)8 * ((size_t)B.blkGR * M1 + (size_t)B.blkGC * N1) * 4 * B.elem; };
+    if (!shaped && pick_blocks(N1, M1, L.elem, mode3, L)) {
+        Layout other = L;
+        L.blk_words = words(L);
+        if (pick_blocks(N1, M1, L.elem, !mode3, other)) L.blk_words = std::max(L.blk_words, words(other));
         L.blk_mpad = (int)align_up(M1, 32);
         const size_t row_bytes = 2 * (size_t)L.blk_mpad * L.elem;
         const size_t keep = std::min(std::max(4 * arr, kBlkRowBytesMin), kBlkRowBytesMax);
         const long long steps = std::min<long long>(keep / row_bytes, kBlkMaxSteps);
         L.blk_steps = (int)std::max<long long>(std::min(steps, tg.K), 1);
-        /* 2 buffers x 2 grids x 2 sides, 16 bytes per FP32 cell, 32 per FP64 */
-        L.blk_words = std::max(other, (size_t)8 * ((size_t)L.blkGR * M1 + (size_t)L.blkGC * N1) * 4 * L.elem);
         L.off_blkx = o;
         o += align_up(L.blk_words, 256);
         L.off_blkq = o; /* cleared together with the words */

@@ -50,6 +50,16 @@ def test_wide_rows_equal_one_launch_per_step(shape, prec):
     assert _equal(_run(p, (4, 5, 18)), _run(p, (4, 5, 18), graph_steps=16))
 
 
+# FP32 grids that fit on chip in one form of the arithmetic only: with one
+# column per thread (its bits are those of mode 3, so these take two steps per
+# launch), and with two or four
+@pytest.mark.parametrize("shape", [(400, 5000), (700, 2880), (137, 14600), (30, 60700)])
+def test_grids_at_the_on_chip_limit_equal_one_launch_per_step(shape):
+    p = _params(*shape)
+    steps = (5, 2, 1, 33)
+    assert _equal(_run(p, steps), _run(p, steps, graph_steps=16))
+
+
 # two steps per launch: an odd number of pairs, of steps, and more steps than
 # the handle keeps rows for (16 at 120001 columns); on chip: in place; one
 # launch per step, shorter and longer than the handle's own graphs
