@@ -141,12 +141,16 @@ __global__ void __launch_bounds__(kPairWarps * 32, 3) pair_kernel(PairArgs A, in
                 *const oWb = A.b_w[cur ^ 1];
 
     /* drive of the two steps; the rotation factors at the end of a half-step
-     * and the start of the grid's next one are the same table entry, except
-     * where the table starts over */
+     * and the start of the grid's next one come from the same table entry,
+     * except where the table starts over: there from its first entry and the
+     * one after its last, which are the same bits for most drives and always
+     * for a constant one (a table of period 1, which starts over every step:
+     * 2049 x 8193 81 us per step in the general form of the iteration) */
     const int kk = (int)(kb % A.P), k1 = kk + 1 == A.P ? 0 : kk + 1;
     const Half<float> Dw = half_drive<float>(A.e_whole, A.dstride, kk), Df = half_drive<float>(A.e_frac, A.dstride, kk);
     const Half<float> Ew = half_drive<float>(A.e_whole, A.dstride, k1), Ef = half_drive<float>(A.e_frac, A.dstride, k1);
-    const bool wrap = k1 == 0;
+    const auto differ = [](float x, float y) { return __float_as_uint(x) != __float_as_uint(y); };
+    const bool wrap = differ(Ew.E0, Dw.E1) || differ(Ew.B0, Dw.B1) || differ(Ef.E0, Df.E1) || differ(Ef.B0, Df.B1);
     const CnK<float> K = cn_constants<float>(A.h, A.nu, A.xi);
     float g[4], w0[4], w1[4], w2[4];
     {
@@ -264,7 +268,7 @@ __global__ void __launch_bounds__(kPairWarps * 32, 3) pair_kernel(PairArgs A, in
     /* iteration q: `od` holds the differences of the rows two back of each
      * source, `nw` takes those of the rows it makes.  FAST: every row it
      * touches exists and is none of rows 0 and 1, every output is this
-     * chunk's, and the table does not start over between the two steps. */
+     * chunk's, and the two steps share their rotation factors. */
     auto iteration = [&](int q, const Rows& od, Rows& nw, auto fast) {
         constexpr bool F = decltype(fast)::value;
         const int j = row_of(q);

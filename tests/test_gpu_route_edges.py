@@ -60,6 +60,15 @@ def test_grids_at_the_on_chip_limit_equal_one_launch_per_step(shape):
     assert _equal(_run(p, steps), _run(p, steps, graph_steps=16))
 
 
+# drives whose table starts over with the entry it ended on (a constant one,
+# from 0 and not) and without, inside a pair and between two
+@pytest.mark.parametrize("omega,B_phase", [(0.0, 0.4), (30.0, 0.0), (31.0, 0.4), (1500.0, 0.4), (3141.0, 0.4)])
+def test_two_steps_per_launch_under_every_drive(omega, B_phase):
+    p = _params(699, 3000, omega=omega).replace(B_phase=B_phase)
+    steps = (5, 2, 41, 70)
+    assert _equal(_run(p, steps), _run(p, steps, graph_steps=16))
+
+
 # two steps per launch: an odd number of pairs, of steps, and more steps than
 # the handle keeps rows for (16 at 120001 columns); on chip: in place; one
 # launch per step, shorter and longer than the handle's own graphs
