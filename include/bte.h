@@ -159,9 +159,11 @@ typedef struct {
                             block has more than 480 cells or does not fit
                             232,448 bytes, or the G clusters do not fit the
                             GPU at once (small grids).  With wide_cols = 0
-                            and no other field set, calls of four steps or
-                            more run in the faster form of mode 0's small
-                            grids instead.
+                            and no other field set, grids of more than one
+                            cluster run in the faster form of mode 0's
+                            small grids instead, their rows added in mode
+                            0's order.  How a run is cut into calls does
+                            not change its bits.
                             0: with every field of this struct zero, a
                             grid that fits the shared memory of the SMs
                             together runs there in calls of four steps or

@@ -514,7 +514,7 @@ struct bte_handle {
     int grid_persist; /* CTAs of a persistent (multi-step) launch, all co-resident */
     bool pair;     /* steps go in pairs, one launch each */
     int pair_ntile, pair_nchunk, pair_rows;
-    bool blk;      /* calls of kBlkMinSteps steps or more run on chip, one block per SM */
+    bool blk;      /* calls of kBlkMinSteps steps or more (mode 3: all) run on chip, one block per SM */
     int set;       /* ping-pong set holding the current state (flips per launch) */
     cudaGraphExec_t graph[2]; /* one graph per starting set */
     double r1;     /* I_1/I_0 */
@@ -1052,7 +1052,10 @@ int enqueue_steps(bte_handle* h, long long n) {
         const int rc = enqueue_pairs(h, n, capture);
         if (rc || n == 0) return rc;
     }
-    if (h->blk && n >= kBlkMinSteps) return enqueue_blocks<T>(h, n);
+    /* mode 3 takes this form for calls of any length: the kernel over clusters
+     * adds the rows in another order, and a run's samples do not depend on how
+     * it is cut into calls */
+    if (h->blk && (n >= kBlkMinSteps || (h->L.wideG && n > 0))) return enqueue_blocks<T>(h, n);
     if (h->L.resC) return n > 0 ? enqueue_resident<T>(h, n) : BTE_OK;
     if (h->L.wideG) return n > 0 ? enqueue_wide<T>(h, n) : BTE_OK;
     if (h->L.persist) return enqueue_persist<T>(h, n);

@@ -132,3 +132,13 @@ def test_handles_on_several_threads():
     for t in threads:
         t.join()
     assert not errors
+
+
+# mode 3 on several clusters and on one, its shape given and not; mode 0
+@pytest.mark.parametrize("shape,kw", [((30, 201), dict(resident=3)), ((47, 256), dict(resident=3)),
+                                      ((16, 96), dict(resident=3)), ((30, 201), dict(resident=3, wide_cols=101)),
+                                      ((30, 201), {}), ((999, 2520), {})])
+@pytest.mark.parametrize("prec", [W.FP64, W.FP32_MIXED])
+def test_cutting_a_run_into_calls_keeps_its_bits(shape, kw, prec):
+    p = _params(*shape, prec)
+    assert _equal(_run(p, (3, 1, 40, 2, 11), **kw), _run(p, (57,), **kw))
