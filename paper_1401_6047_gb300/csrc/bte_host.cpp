@@ -1140,6 +1140,7 @@ int get_grid(bte_handle* h, int grid, double* a, double* b) {
     const Layout& L = h->L;
     const int set = h->set;
     const size_t N1 = h->p.n_max + 1, M1 = h->p.m_points, n = N1 * M1;
+    if (a == b) a = nullptr; /* one array for both: it ends with b */
     double* const dst[2] = {a, b};
     for (int which = 0; which < 2; ++which) {
         if (!dst[which]) continue;

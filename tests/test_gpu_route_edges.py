@@ -142,3 +142,15 @@ def test_handles_on_several_threads():
 def test_cutting_a_run_into_calls_keeps_its_bits(shape, kw, prec):
     p = _params(*shape, prec)
     assert _equal(_run(p, (3, 1, 40, 2, 11), **kw), _run(p, (57,), **kw))
+
+
+@pytest.mark.parametrize("prec", [W.FP64, W.FP32_MIXED])
+def test_state_into_one_array_for_both(prec):
+    """The second grid array is copied last, so it is what one array given for
+    both ends with."""
+    with bte.Solver(_params(30, 201, prec)) as s:
+        s.step(10)
+        for grid in (0, 1):
+            x = np.zeros(s.shape)
+            bte._check(bte.lib().bte_get_state(s._h, grid, bte._dp(x), bte._dp(x)))
+            assert np.array_equal(x, s.get_state(grid)[1])
