@@ -344,8 +344,9 @@ typedef struct bte_batch_opts {
  *     skipped by later launches of its batch.
  * With every shape field of the options zero (tile_m, chunk_n, vec,
  * graph_steps, walk, resident, resident_smem), points that fit no cluster run
- * one after another as single instances instead of streamed, and few points
- * get larger clusters than they need.
+ * one after another as single instances instead of streamed where that is
+ * estimated to take less time, and few points get larger clusters than they
+ * need.
  * All give the same per-cell arithmetic; the per-step sums over phi_y are
  * added in different orders.  out[i] receives the
  * final observables of p[i] exactly as bte_observables reports them after

@@ -196,6 +196,7 @@ struct Layout {
     /* on chip, one block per SM (blkGR = 0: the grid does not fit): blkGR x
      * blkGC blocks of blkR rows x blkW columns, blkV columns per thread */
     int blkGR, blkGC, blkR, blkW, blkV, blk_threads, blk_help;
+    double blk_cycles;          /* pick_blocks' estimate of a half-step */
     size_t blk_smem, blk_words; /* shared memory per CTA; bytes of exchange words */
     int blk_steps, blk_mpad;    /* steps per launch at most; pitch of the kept rows */
     size_t off_blkx, off_blkq, off_blkrows, off_fold; /* off_fold: scratch of the row sums */
@@ -276,6 +277,7 @@ bool pick_blocks(int N1, int M1, size_t elem, bool scalar, Layout& L) {
                 const double t = std::max(t_int, t_x) + t_bnd + 0.4 * nq;
                 if (t < best) {
                     best = t;
+                    L.blk_cycles = t;
                     L.blkGR = GR;
                     L.blkGC = GC;
                     L.blkR = R;
@@ -1190,7 +1192,7 @@ namespace {
 
 struct BatchPoint {
     int idx; /* position in the caller's array */
-    int resC; /* CTAs per cluster of the on-chip tier, 0: streamed */
+    int resC; /* CTAs per cluster of the on-chip tier, 0: streamed or alone */
     TimeGrid tg;
     int N1, M1, ntx, nty, pitch, items;
     double dphi;
@@ -1694,6 +1696,118 @@ int report_error(int code, const char* msg) {
 
 namespace {
 
+/* device bytes of a point in a batch: state arrays, the two drive tables, other tables */
+long long batch_bytes(const BatchPoint& b, const BatchCfg& c) {
+    const int elem = c.fp64 ? 8 : 4, drive = c.fp64 ? bte::kDriveRows<double> : bte::kDriveRows<float>;
+    const long long pitch = (long long)align_up((size_t)(128 / elem + b.ntx * c.tile + 32 / elem), 32);
+    return (b.resC > 0 ? 4ll : 8ll) * b.N1 * pitch * elem + 2ll * drive * (b.tg.P + 2) * elem + 4096;
+}
+
+/* one past the last point of the batch that begins at `first`: on-chip points
+ * of every cluster size share a batch */
+size_t batch_end(const std::vector<BatchPoint>& pts, size_t first, const BatchCfg& c) {
+    long long bytes = 0;
+    size_t last = first;
+    const bool res = pts[first].resC > 0;
+    while (last < pts.size() && (pts[last].resC > 0) == res && (res || (int)(last - first) < c.max_batch)) {
+        const long long b = batch_bytes(pts[last], c);
+        if (last > first && bytes + b > c.max_bytes) break;
+        bytes += b;
+        ++last;
+    }
+    return last;
+}
+
+/* Time of a step of one point run as a single instance, in us, or a negative
+ * value when it cannot be.  Measured (GB300) against the estimate: on chip,
+ * FP32 1.5e-3 us per cycle of pick_blocks (10 x 4001 2.6 / 2.8, 138 x 1533 3.4
+ * / 3.5, 401 x 4001 7.9 / 7.5), FP64 2.2 + 1.04e-3 (21 x 2001 7.1 / 6.9, 89 x
+ * 1001 10.2 / 10.0, 201 x 2001 34 / 36); two steps per launch 4 + 3.4e-6 per
+ * cell with twelve more rows (8 x 350000 29 / 28, 2049 x 8193 60 / 61); one
+ * launch per step, FP64: 12 + 1e-4 per cell (401 x 4001 172 / 172). */
+double alone_us(const bte_params& p, const TimeGrid& tg) {
+    Layout L;
+    if (plan(&p, nullptr, tg, L)) return -1.0;
+    if (L.blkGR) return L.elem == 8 ? 2.2 + 1.04e-3 * L.blk_cycles : 1.5e-3 * L.blk_cycles;
+    const double cells = (double)(p.n_max + 1) * p.m_points;
+    return L.elem == 4 ? 4.0 + 3.4e-6 * cells * (p.n_max + 13) / (p.n_max + 1) : 12.0 + 1e-4 * cells;
+}
+
+/* Time of all steps of the streamed points `pts` (longest runs first) in
+ * lock-step batches, in us: a step takes as many waves of tiles as the items
+ * fill the GPU's `slots` CTAs, and a wave as long as its tiles have rows.
+ * Measured (GB300, chunks of 16): FP32 22 us for tiles of 10 rows and 29 for
+ * 16, a fifth more each where there are several waves, which then mix the
+ * tiles of full and of fewer rows (21 x 6001, 32 points: 80 us, 81 with the
+ * mean rows of a tile); FP64 92 and 145, where they do not (21 x 2001, 32
+ * points: 284 us, 290 with full tiles). */
+double wave_us(const BatchCfg& c, double rows) { return c.fp64 ? 3.7 + 8.83 * rows : 10.5 + 1.15 * rows; }
+double several_waves_us(const BatchPoint& b, const BatchCfg& c) {
+    return c.fp64 ? wave_us(c, std::min(b.N1, c.chunk)) : 1.2 * wave_us(c, (double)b.N1 / b.nty);
+}
+double lock_step_us(const std::vector<BatchPoint>& pts, const BatchCfg& c, int slots) {
+    double total = 0.0;
+    for (size_t first = 0; first < pts.size();) {
+        const size_t last = batch_end(pts, first, c);
+        double items = 0.0, weight = 0.0, longest = 0.0;
+        for (size_t i = first; i < last; ++i) {
+            const BatchPoint& b = pts[i];
+            const double n = (double)b.ntx * b.nty;
+            items += n;
+            weight += n * several_waves_us(b, c);
+            longest = std::max(longest, wave_us(c, std::min(b.N1, c.chunk)));
+            const long long steps = b.tg.K - (i + 1 < last ? pts[i + 1].tg.K : 0);
+            const double waves = std::ceil(items / slots);
+            total += steps * (waves <= 1.0 ? longest : waves * weight / items);
+        }
+        first = last;
+    }
+    return total;
+}
+
+/* Of the points that fit no cluster (pts[from ..], longest runs first), moves
+ * those that run as single instances to the end and returns the first of them.
+ * One point has the whole GPU to itself there, but a small or narrow one
+ * cannot use it: the others wait meanwhile.  Taken is the least estimate of
+ * all alone, all in lock-step, and alone only the points whose own time is
+ * less than their share of a full wave.  Measured (GB300, us per step of the
+ * whole batch, alone / lock-step): FP32 138 x 1533, 8 points 27 / 29, 64
+ * points 214 / 207; 201 x 2001, 64 points 245 / 385; 10 x 4001, 8 points 21 /
+ * 22, 64 points 168 / 45; 31 x 4001, 32 points 103 / 72; FP64 89 x 1001, 8
+ * points 82 / 148, 64 points 655 / 769; 10 x 2001, 64 points 306 / 184. */
+size_t split_alone(const bte_params* p, std::vector<BatchPoint>& pts, size_t from, const BatchCfg& c, int slots) {
+    const size_t n = pts.size() - from;
+    if (n == 0) return from;
+    std::vector<double> us(n);
+    std::vector<char> take[3]; /* 1: alone */
+    for (auto& t : take) t.assign(n, 0);
+    for (size_t i = 0; i < n; ++i) {
+        const BatchPoint& b = pts[from + i];
+        us[i] = alone_us(p[b.idx], b.tg);
+        take[0][i] = us[i] >= 0.0;
+        take[1][i] = us[i] >= 0.0 && us[i] < (double)b.ntx * b.nty / slots * several_waves_us(b, c);
+    }
+    int best = 0;
+    double best_us = 1e300;
+    for (int q = 0; q < 3; ++q) {
+        std::vector<BatchPoint> lock;
+        double t = 0.0;
+        for (size_t i = 0; i < n; ++i)
+            if (take[q][i]) t += us[i] * (double)pts[from + i].tg.K;
+            else lock.push_back(pts[from + i]);
+        t += lock_step_us(lock, c, slots);
+        if (t < best_us) {
+            best_us = t;
+            best = q;
+        }
+    }
+    std::vector<BatchPoint> lock, alone;
+    for (size_t i = 0; i < n; ++i) (take[best][i] ? alone : lock).push_back(pts[from + i]);
+    std::copy(lock.begin(), lock.end(), pts.begin() + from);
+    std::copy(alone.begin(), alone.end(), pts.begin() + from + lock.size());
+    return from + lock.size();
+}
+
 /* pts[from ..] one after another, each as a single instance over one
  * workspace as large as the largest of them needs */
 int run_alone(const bte_params* p, const std::vector<BatchPoint>& pts, size_t from, cudaStream_t st, bte_obs* out) {
@@ -1744,8 +1858,6 @@ int bte_batch_run(const bte_params* p, int32_t n, bte_obs* out, const bte_batch_
     }
     const bool fp64 = cfg.fp64;
     const int vec = cfg.vec, tile = cfg.tile, chunk = cfg.chunk, graph_len = cfg.graph_len;
-    const int max_batch = cfg.max_batch;
-    const long long max_bytes = cfg.max_bytes;
     /* by tier (on-chip cluster size, then streamed), longest runs first, so a
      * streamed batch's members need similar step counts */
     auto by_tier = [](const BatchPoint& x, const BatchPoint& y) {
@@ -1762,23 +1874,31 @@ int bte_batch_run(const bte_params* p, int32_t n, bte_obs* out, const bte_batch_
     }
     int worst = BTE_OK;
     size_t first = 0;
-    /* shapes left to the library: points that fit no cluster (sorted last) run
-     * one after another as single instances, which take the whole GPU for one
-     * point (lock-step launches over the tiles of seven FP64 points of 62 to 97
-     * thousand cells: 150 us per step together; one block per SM: 8 to 10 us
-     * for each) */
+    /* shapes left to the library: of the points that fit no cluster (sorted
+     * last) those that are faster so run one after another as single instances
+     * (see split_alone) */
     const bool shaped = opts && (opts->tile_m || opts->chunk_n || opts->vec || opts->graph_steps || opts->walk ||
                                  opts->resident || opts->resident_smem);
     if (!shaped) {
-        size_t from = pts.size();
-        while (from > 0 && !pts[from - 1].resC) --from;
+        size_t res = pts.size();
+        while (res > 0 && !pts[res - 1].resC) --res;
+        int bps = 0, dev = 0, sms = 0;
+        if (res < pts.size() &&
+            (cudaGetDevice(&dev) != cudaSuccess ||
+             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+             (fp64 ? bte::step_kernel_configure_batch<double>(tile, chunk, vec, &bps)
+                   : bte::step_kernel_configure_batch<float>(tile, chunk, vec, &bps)))) {
+            if (own) cudaStreamDestroy(st);
+            return fail(BTE_ECUDA, "batch kernel configure failed");
+        }
+        const size_t from = split_alone(p, pts, res, cfg, std::max(bps * sms, 1));
         worst = run_alone(p, pts, from, st, out);
         if (worst == BTE_ECUDA || worst == BTE_ENOMEM) {
             if (own) cudaStreamDestroy(st);
             return worst;
         }
         pts.resize(from);
-        widen_clusters(pts, from, fp64);
+        widen_clusters(pts, res, fp64);
         std::sort(pts.begin(), pts.end(), by_tier);
     }
     cudaStream_t cap = nullptr;
@@ -1786,23 +1906,9 @@ int bte_batch_run(const bte_params* p, int32_t n, bte_obs* out, const bte_batch_
         if (own) cudaStreamDestroy(st);
         return fail(BTE_ECUDA, "cudaStreamCreate failed");
     }
-    const int elem = fp64 ? 8 : 4;
     while (first < pts.size()) {
-        size_t last = first;
-        long long bytes = 0;
-        /* on-chip points of every cluster size share a batch */
-        const int resC = pts[first].resC;
-        while (last < pts.size() && (pts[last].resC > 0) == (resC > 0) &&
-               (resC > 0 || (int)(last - first) < max_batch)) {
-            const BatchPoint& b = pts[last];
-            const long long pitch = (long long)align_up((size_t)(128 / elem + b.ntx * tile + 32 / elem), 32);
-            /* state arrays, the two drive tables, other tables */
-            const long long sb = (resC > 0 ? 4ll : 8ll) * b.N1 * pitch * elem + 2ll * (elem == 8 ? bte::kDriveRows<double> : bte::kDriveRows<float>) * (b.tg.P + 2) * elem + 4096;
-            if (last > first && bytes + sb > max_bytes) break;
-            bytes += sb;
-            ++last;
-        }
-        const bool res = resC > 0;
+        const size_t last = batch_end(pts, first, cfg);
+        const bool res = pts[first].resC > 0;
         const int walk = opts ? opts->walk : 0;
         const int rc = fp64 ? run_batch<double>(p, pts, first, last, tile, chunk, vec, graph_len, res, walk, st, cap, out)
                             : run_batch<float>(p, pts, first, last, tile, chunk, vec, graph_len, res, walk, st, cap, out);

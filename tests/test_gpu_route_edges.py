@@ -2,6 +2,7 @@
 or its bookkeeping can go wrong: very wide rows, grids near the on-chip limit,
 a constant drive, captured calls, several handles at once."""
 import threading
+import time
 
 import numpy as np
 import pytest
@@ -154,3 +155,27 @@ def test_state_into_one_array_for_both(prec):
             x = np.zeros(s.shape)
             bte._check(bte.lib().bte_get_state(s._h, grid, bte._dp(x), bte._dp(x)))
             assert np.array_equal(x, s.get_state(grid)[1])
+
+
+def _seconds(pts, **kw):
+    best = 1e9
+    for _ in range(3):
+        t = time.perf_counter()
+        bte.batch_run(pts, **kw)
+        best = min(best, time.perf_counter() - t)
+    return best
+
+
+# points that fit no cluster: many that leave most of the GPU idle alone (3.7
+# and 1.7 times the lock-step time one after another), few and large ones that
+# do not, and both
+@pytest.mark.parametrize("points,prec", [([(9, 4001, 64)], W.FP32_MIXED), ([(9, 2001, 64)], W.FP64),
+                                         ([(200, 2001, 6)], W.FP32_MIXED), ([(400, 4001, 3), (9, 4001, 48)], W.FP32_MIXED)])
+def test_batches_that_fit_no_cluster_are_no_slower_than_lock_step(points, prec):
+    pts = [_params(n, m, prec).replace(periods=0.5, avg_window=0.1) for n, m, count in points for _ in range(count)]
+    assert not bte.batch_plan(pts).any()
+    assert _seconds(pts) < 1.3 * _seconds(pts, resident=1)
+    for o, r in zip(bte.batch_run(pts), bte.batch_run(pts, resident=1)):
+        assert o.status == r.status == bte.OK
+        for x, y in zip((o.v_dr, o.norm, o.v_dc_avg, o.absorption), (r.v_dr, r.norm, r.v_dc_avg, r.absorption)):
+            assert abs(x - y) <= 1e-10 * abs(y)  # the same cells, added in another order
