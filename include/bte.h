@@ -369,8 +369,9 @@ BTE_API int bte_batch_plan(const bte_params* p, int32_t n, const bte_batch_opts*
  * steps), shortens their runs so that the longest has about `steps` time
  * steps (relative run lengths kept), and times bte_batch_run on them for 12
  * candidate option sets (each run once untimed, then timed): on-chip tier
- * with 232,448 / 160,000 / 113,664 bytes of shared memory per CTA, then the
- * streamed tier alone with tile_m = {32, 64, 128} x vec and chunk_n = {8, 16,
+ * with 232,448 / 160,000 / 113,664 bytes of shared memory per CTA (in place of
+ * the first resident_smem = 0, where that runs some of the points on another
+ * route), then the streamed tier alone with tile_m = {32, 64, 128} x vec and chunk_n = {8, 16,
  * 32}.  *best receives the fastest (fields not tuned copied from *base,
  * which may be NULL); seconds (HOST, 12 values, may be NULL) the time of each
  * candidate in that order (1e300 where a candidate does not apply).

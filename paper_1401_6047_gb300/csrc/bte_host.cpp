@@ -1589,12 +1589,13 @@ int run_batch(const bte_params* p, std::vector<BatchPoint>& pts, size_t first, s
  * the CTAs, until it cannot (16, or fewer than two rows each) or 96 CTAs (six
  * clusters of 16) are taken.  The results do not depend on the cluster's size.
  * Time of a step in us, from measured runs: FP64 5 + 0.014 per cell of a CTA,
- * FP32 3.5 + 0.00075. */
-void widen_clusters(std::vector<BatchPoint>& pts, size_t n, bool fp64) {
+ * FP32 3.5 + 0.00075.  Whether any was. */
+bool widen_clusters(std::vector<BatchPoint>& pts, size_t n, bool fp64) {
     auto time = [&](const BatchPoint& b) {
         return (double)b.tg.K * (fp64 ? 5.0 + 1.4e-2 * b.N1 * b.M1 / b.resC : 3.5 + 7.5e-4 * b.N1 * b.M1 / b.resC);
     };
     int ctas = 0;
+    bool any = false;
     for (size_t i = 0; i < n && ctas <= 96; ++i) ctas += pts[i].resC;
     while (n > 0) {
         BatchPoint* b = &pts[0];
@@ -1604,7 +1605,9 @@ void widen_clusters(std::vector<BatchPoint>& pts, size_t n, bool fp64) {
         if (C > 16 || (b->N1 + C - 1) / C < 2 || ctas + b->resC > 96) break;
         ctas += b->resC;
         b->resC = C;
+        any = true;
     }
+    return any;
 }
 
 struct BatchCfg {
@@ -1765,6 +1768,25 @@ double lock_step_us(const std::vector<BatchPoint>& pts, const BatchCfg& c, int s
     return total;
 }
 
+/* by tier (on-chip cluster size, then streamed), longest runs first, so a
+ * streamed batch's members need similar step counts */
+bool by_tier(const BatchPoint& x, const BatchPoint& y) {
+    if (x.resC != y.resC) return x.resC > y.resC;
+    return x.tg.K != y.tg.K ? x.tg.K > y.tg.K : x.idx < y.idx;
+}
+
+/* CTAs of the lock-step kernel that the GPU holds at once */
+int lock_step_slots(const BatchCfg& c, int* slots) {
+    int bps = 0, dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        (c.fp64 ? bte::step_kernel_configure_batch<double>(c.tile, c.chunk, c.vec, &bps)
+                : bte::step_kernel_configure_batch<float>(c.tile, c.chunk, c.vec, &bps)))
+        return fail(BTE_ECUDA, "batch kernel configure failed");
+    *slots = std::max(bps * sms, 1);
+    return BTE_OK;
+}
+
 /* Of the points that fit no cluster (pts[from ..], longest runs first), moves
  * those that run as single instances to the end and returns the first of them.
  * One point has the whole GPU to itself there, but a small or narrow one
@@ -1806,6 +1828,23 @@ size_t split_alone(const bte_params* p, std::vector<BatchPoint>& pts, size_t fro
     std::copy(lock.begin(), lock.end(), pts.begin() + from);
     std::copy(alone.begin(), alone.end(), pts.begin() + from + lock.size());
     return from + lock.size();
+}
+
+/* whether the options leave the routes of the points to the library */
+bool batch_shaped(const bte_batch_opts* o) {
+    return o && (o->tile_m || o->chunk_n || o->vec || o->graph_steps || o->walk || o->resident || o->resident_smem);
+}
+
+/* splits sorted points into those on chip ([0, res)), in lock-step ([res,
+ * from)) and alone */
+int split_batch(const bte_params* p, std::vector<BatchPoint>& pts, const BatchCfg& c, size_t* res, size_t* from) {
+    *res = *from = pts.size();
+    while (*res > 0 && !pts[*res - 1].resC) --*res;
+    if (*res == pts.size()) return BTE_OK;
+    int slots = 0;
+    const int rc = lock_step_slots(c, &slots);
+    if (!rc) *from = split_alone(p, pts, *res, c, slots);
+    return rc;
 }
 
 /* pts[from ..] one after another, each as a single instance over one
@@ -1858,12 +1897,6 @@ int bte_batch_run(const bte_params* p, int32_t n, bte_obs* out, const bte_batch_
     }
     const bool fp64 = cfg.fp64;
     const int vec = cfg.vec, tile = cfg.tile, chunk = cfg.chunk, graph_len = cfg.graph_len;
-    /* by tier (on-chip cluster size, then streamed), longest runs first, so a
-     * streamed batch's members need similar step counts */
-    auto by_tier = [](const BatchPoint& x, const BatchPoint& y) {
-        if (x.resC != y.resC) return x.resC > y.resC;
-        return x.tg.K != y.tg.K ? x.tg.K > y.tg.K : x.idx < y.idx;
-    };
     std::sort(pts.begin(), pts.end(), by_tier);
     cudaStream_t st = opts && opts->stream ? (cudaStream_t)opts->stream : nullptr;
     bool own = false;
@@ -1877,21 +1910,13 @@ int bte_batch_run(const bte_params* p, int32_t n, bte_obs* out, const bte_batch_
     /* shapes left to the library: of the points that fit no cluster (sorted
      * last) those that are faster so run one after another as single instances
      * (see split_alone) */
-    const bool shaped = opts && (opts->tile_m || opts->chunk_n || opts->vec || opts->graph_steps || opts->walk ||
-                                 opts->resident || opts->resident_smem);
-    if (!shaped) {
-        size_t res = pts.size();
-        while (res > 0 && !pts[res - 1].resC) --res;
-        int bps = 0, dev = 0, sms = 0;
-        if (res < pts.size() &&
-            (cudaGetDevice(&dev) != cudaSuccess ||
-             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-             (fp64 ? bte::step_kernel_configure_batch<double>(tile, chunk, vec, &bps)
-                   : bte::step_kernel_configure_batch<float>(tile, chunk, vec, &bps)))) {
+    if (!batch_shaped(opts)) {
+        size_t res = 0, from = 0;
+        const int rc = split_batch(p, pts, cfg, &res, &from);
+        if (rc) {
             if (own) cudaStreamDestroy(st);
-            return fail(BTE_ECUDA, "batch kernel configure failed");
+            return rc;
         }
-        const size_t from = split_alone(p, pts, res, cfg, std::max(bps * sms, 1));
         worst = run_alone(p, pts, from, st, out);
         if (worst == BTE_ECUDA || worst == BTE_ENOMEM) {
             if (own) cudaStreamDestroy(st);
@@ -1981,11 +2006,27 @@ int bte_batch_tune(const bte_params* p, int32_t n, const bte_batch_opts* base, i
         }
         sp[j] = q;
     }
-    /* candidates: on-chip budgets, then streamed shapes */
+    /* candidates: on-chip budgets, then streamed shapes.  The whole budget is
+     * left to the library where it would run some of these points alone or in
+     * larger clusters; else it is named, so that a sample of them, few enough
+     * for either, is not run so */
     const bool fp64 = p[0].precision == BTE_FP64;
+    bool routed = false;
+    bte_batch_opts whole = b0;
+    whole.resident = whole.resident_smem = 0;
+    if (!batch_shaped(&whole)) {
+        std::vector<BatchPoint> pts;
+        BatchCfg cfg;
+        int rc = batch_prepare(p, n, &whole, pts, cfg);
+        size_t res = 0, from = 0;
+        std::sort(pts.begin(), pts.end(), by_tier);
+        if (!rc) rc = split_batch(p, pts, cfg, &res, &from);
+        if (rc) return rc;
+        routed = from < pts.size() || widen_clusters(pts, res, fp64);
+    }
     const int v = b0.vec ? b0.vec : (fp64 ? 2 : 4);
     std::vector<bte_batch_opts> cand;
-    for (int smem : {232448, 160000, 113664}) {
+    for (int smem : {routed ? 0 : 232448, 160000, 113664}) {
         bte_batch_opts o = b0;
         o.resident = 0;
         o.resident_smem = smem;

@@ -179,3 +179,12 @@ def test_batches_that_fit_no_cluster_are_no_slower_than_lock_step(points, prec):
         assert o.status == r.status == bte.OK
         for x, y in zip((o.v_dr, o.norm, o.v_dc_avg, o.absorption), (r.v_dr, r.norm, r.v_dc_avg, r.absorption)):
             assert abs(x - y) <= 1e-10 * abs(y)  # the same cells, added in another order
+
+
+def test_tuned_options_are_no_slower_than_none():
+    """Points that run fastest one after another, which only options that leave
+    the shape to the library do."""
+    pts = [_params(88, 1001, W.FP64).replace(periods=0.3, avg_window=0.1) for _ in range(6)]
+    best, secs = bte.batch_tune(pts, sample=6, steps=400)
+    assert secs.argmin() == 0 and best["resident"] == 0
+    assert _seconds(pts, **best) < 1.3 * _seconds(pts)
