@@ -172,7 +172,7 @@ int backward(bte_sur* h, const float* x, const float* y, const int* idx, long lo
         dh.err = h->err;
         KL(bte::sur::launch_gemm(dh, bte::sur::EPI_BWD, h->M, h->stream));
     }
-    /* weight gradients dZ^T H_prev of both */
+    /* weight gradients dZ^T H_prev of both, and the sums over the samples */
     bte::sur::WgradArgs gw{};
     gw.dZ[0] = h->DZ2;
     gw.dZ[1] = h->DZ3;
@@ -187,7 +187,6 @@ int backward(bte_sur* h, const float* x, const float* y, const int* idx, long lo
     gw.oW[0] = h->off.W2;
     gw.oW[1] = h->off.W3;
     gw.err = h->err;
-    KL(bte::sur::launch_wgrad(gw, h->M, h->stream));
     r = bte::sur::RedArgs{};
     r.DZ1 = h->DZ1;
     r.DZ2 = h->DZ2;
@@ -205,7 +204,7 @@ int backward(bte_sur* h, const float* x, const float* y, const int* idx, long lo
     r.pstride = h->pstride;
     r.off = h->off;
     r.sc = h->sc;
-    KL(bte::sur::launch_reduce_partial(r, h->M, h->stream));
+    KL(bte::sur::launch_grad(gw, r, h->M, h->stream));
     return BTE_OK;
 }
 

@@ -186,10 +186,10 @@ struct EnsArgs {
 };
 
 int launch_gemm(const GemmArgs& a, int epi, int members, void* stream);
-int launch_wgrad(const WgradArgs& a, int members, void* stream);
+/* weight gradients and the partial sums of the other gradients */
+int launch_grad(const WgradArgs& w, const RedArgs& r, int members, void* stream);
 int launch_l1(const L1Args& a, int members, void* stream);
 int launch_head(const HeadArgs& a, int members, void* stream);
-int launch_reduce_partial(const RedArgs& a, int members, void* stream);
 int launch_reduce_final(const RedArgs& a, int members, void* stream); /* into grad */
 int launch_adam(const AdamArgs& a, void* stream);
 int launch_refresh_bf16(const AdamArgs& a, void* stream);

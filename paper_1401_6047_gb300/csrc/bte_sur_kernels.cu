@@ -6,7 +6,7 @@
  * tensor memory) in two GEMM kernels: one for the products along the hidden
  * units (forward, and back through a layer), whose epilogue fuses the bias,
  * the SiLU activation and its derivative, and one for the weight gradients
- * (along the batch).  The thin layers (5 inputs, 2 outputs) are FP32 FMA
+ * (along the batch) beside the reductions over it.  The thin layers (5 inputs, 2 outputs) are FP32 FMA
  * kernels; batch reductions are two-pass and deterministic; Adam keeps FP32
  * master weights and refreshes the BF16 operand copies in the same pass.
  *
@@ -228,14 +228,14 @@ __global__ void __launch_bounds__(kGThreads) gemm_tc_kernel(GemmArgs a) {
 }
 
 /* Weight gradients dW = dZ^T H of both hidden layers (see WgradArgs): 128 x
- * 128 outputs per CTA, blockIdx.z = 2 member + layer, K the batch.  Both
+ * 128 outputs per CTA, K the batch.  Both
  * operands are stored [sample][unit], so they go to shared memory as they
  * are and the tensor cores take them MN-major; stages of 64 samples, three
  * in flight while one is multiplied.  The tile is square because the loads
  * bound it (34 MB through L2 for 8 members x 1024, 25 us; 128 x 32 tiles,
  * which fill more SMs, move 84 MB: 29 us), and K stays whole to keep the
  * order of the sum.  Every wait is bounded, as above. */
-__global__ void __launch_bounds__(kGThreads) wgrad_tc_kernel(WgradArgs a) {
+__device__ __forceinline__ void weight_gradients(const WgradArgs& a, int tile) {
     extern __shared__ unsigned char gsm_raw[];
     unsigned char* gsm = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(gsm_raw) + 1023) & ~(uintptr_t)1023);
@@ -243,10 +243,11 @@ __global__ void __launch_bounds__(kGThreads) wgrad_tc_kernel(WgradArgs a) {
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kGStages);
     const uint32_t bar0 = dev::smem_u32(bars);
 
-    const int layer = blockIdx.z & 1, mem = blockIdx.z >> 1;
-    const __nv_bfloat16* A = a.dZ[layer] + mem * a.sAct;
-    const __nv_bfloat16* B = a.H[layer] + mem * a.sAct;
-    const int m0 = blockIdx.y * GM, n0 = blockIdx.x * GN;
+    const int across = a.H0 / GN, per = across * (a.H0 / GM); /* tiles of one layer of one member */
+    const int layer = tile / per & 1, mem = tile / per >> 1;
+    const __nv_bfloat16* A = (layer ? a.dZ[1] : a.dZ[0]) + mem * a.sAct;
+    const __nv_bfloat16* B = (layer ? a.H[1] : a.H[0]) + mem * a.sAct;
+    const int m0 = tile % per / across * GM, n0 = tile % across * GN;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
         for (int st = 0; st < kGStages; ++st) dev::mbar_init(bar0 + 8 * st, 1);
@@ -254,7 +255,7 @@ __global__ void __launch_bounds__(kGThreads) wgrad_tc_kernel(WgradArgs a) {
     }
     const uint32_t tmem = tmem_begin<GN>(tmem_slot, warp);
     pdl_wait();
-    pdl_trigger(); /* reduce_partial_kernel reads nothing of this one's */
+    pdl_trigger();
 
     const int nk = a.K / GK;
     auto load = [&](int kt) { /* one group per stage, empty past the end */
@@ -290,7 +291,7 @@ __global__ void __launch_bounds__(kGThreads) wgrad_tc_kernel(WgradArgs a) {
     tc::tc_fence_after();
     if (ok) {
         const int sub = warp & 3, half = warp >> 2;
-        float* o = a.grad + mem * a.pstride + a.oW[layer] + (long long)(m0 + sub * 32 + lane) * a.ld + n0;
+        float* o = a.grad + mem * a.pstride + (layer ? a.oW[1] : a.oW[0]) + (long long)(m0 + sub * 32 + lane) * a.ld + n0;
 #pragma unroll 1
         for (int cb = 0; cb < GN / 2; cb += 32) {
             const int cl = half * (GN / 2) + cb;
@@ -449,16 +450,12 @@ __global__ void head_kernel(HeadArgs a) {
 /* values per 128-sample block: b1, W1 (5 per unit), b2, b3, W4 (2 per unit), b4 */
 __host__ __device__ inline int red_count(int H) { return H * (1 + kIn + 1 + 1 + kOut) + kOut; }
 
-/* Partial sums over 128 samples (blockIdx.x) of one member (blockIdx.y).
- * blockIdx.z = 4 part + quarter of the hidden units; part 0: b1 and W1 (from
- * DZ1 and the inputs), 1: b2, 2: b3, 3: W4 and b4 (from H3 and DY).  One
- * hidden unit per thread, the samples added in order, 32 loads in flight (one
- * CTA per 128 samples that did all four arrays: 107 us for 8 members x 1024,
- * one load of each array in flight; so: 10 us).  Launched beside the weight
- * gradients (programmatic dependent launch: that kernel starts after the
- * activations' gradients are complete, and this one reads only those); it
- * ends after them, so what follows it in the stream follows both. */
-constexpr int kRedThreads = 64, kRedFly = 32;
+/* Partial sums over 128 samples of one member; `part` 0: b1 and W1 (from DZ1
+ * and the inputs), 1: b2, 2: b3, 3: W4 and b4 (from H3 and DY).  One hidden
+ * unit per thread, the samples added in order, 32 loads in flight (one CTA per
+ * 128 samples that did all four arrays: 107 us for 8 members x 1024, one load
+ * of each array in flight; so: 10 us). */
+constexpr int kRedFly = 32;
 template <class F>
 __device__ __forceinline__ void over_samples(const __nv_bfloat16* p, int H, F f) {
     for (int r0 = 0; r0 < 128; r0 += kRedFly) {
@@ -469,16 +466,17 @@ __device__ __forceinline__ void over_samples(const __nv_bfloat16* p, int H, F f)
         for (int q = 0; q < kRedFly; ++q) f(r0 + q, __bfloat162float(v[q]));
     }
 }
-__global__ void __launch_bounds__(kRedThreads) reduce_partial_kernel(RedArgs a) {
-    const int mem = blockIdx.y, chunk = blockIdx.x, part = blockIdx.z >> 2;
-    const int r0 = chunk * 128, o = (blockIdx.z & 3) * kRedThreads + threadIdx.x;
+__device__ __forceinline__ void reduce_partial(const RedArgs& a, int chunk, int mem, int part) {
+    const int r0 = chunk * 128, o = threadIdx.x;
     __shared__ float sx[128][kIn];
     const int H = a.H, nred = red_count(H);
     float* out = a.partial + ((long long)mem * (a.Bp / 128) + chunk) * nred;
     const long long e = ((long long)mem * a.Bp + r0) * H + o;
+    pdl_wait();
+    pdl_trigger();
     if (part == 0) {
         const int* idx = a.idx ? a.idx + (long long)mem * a.Bp : nullptr;
-        for (int r = threadIdx.x; r < 128; r += kRedThreads) {
+        for (int r = threadIdx.x; r < 128; r += blockDim.x) {
             float xh[kIn];
             load_xh(a.x, idx, a.row0, r0 + r, a.nvalid, a.sc, xh);
 #pragma unroll
@@ -499,7 +497,7 @@ __global__ void __launch_bounds__(kRedThreads) reduce_partial_kernel(RedArgs a) 
         over_samples((part == 1 ? a.DZ2 : a.DZ3) + e, H, [&](int, float d) { gb += d; });
         out[H * (kIn + part) + o] = gb;
     } else {
-        for (int r = threadIdx.x; r < 128; r += kRedThreads) {
+        for (int r = threadIdx.x; r < 128; r += blockDim.x) {
             const long long yo = ((long long)mem * a.Bp + r0 + r) * kOut;
             sx[r][0] = a.DY[yo];
             sx[r][1] = a.DY[yo + 1];
@@ -518,7 +516,22 @@ __global__ void __launch_bounds__(kRedThreads) reduce_partial_kernel(RedArgs a) 
             out[H * (3 + kIn + kOut) + o] = s;
         }
     }
-    pdl_wait();
+}
+
+/* The gradients of a step in one launch: CTAs of weight-gradient tiles first,
+ * then those of the reductions (member, 128 samples, part), which run on the
+ * SMs that the tiles leave and are over before them.  Both read what the
+ * backward products wrote, so every CTA waits for the launch before it (a step
+ * of 8 members on 1024 points: 94 us with the reductions in a launch of their
+ * own, 92 so). */
+__global__ void __launch_bounds__(kGThreads) grad_kernel(WgradArgs w, RedArgs r, int tiles) {
+    const int b = (int)blockIdx.x - tiles;
+    if (b < 0) {
+        weight_gradients(w, blockIdx.x);
+    } else {
+        const int chunks = r.Bp / 128;
+        reduce_partial(r, b / 4 % chunks, b / (4 * chunks), b % 4);
+    }
 }
 
 /* value q of a member's packed reductions: its sum over the 128-sample
@@ -640,8 +653,8 @@ int reduce_count(int H) { return red_count(H); }
 
 /* A launch that may begin while the one before it drains: the kernel reads
  * and writes nothing of it before its griddepcontrol.wait. */
-template <class K, class A>
-static int launch_pdl(K* kernel, dim3 grid, int threads, size_t smem, void* stream, const A& args) {
+template <class... P, class... A>
+static int launch_pdl(void (*kernel)(P...), dim3 grid, int threads, size_t smem, void* stream, const A&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
@@ -652,7 +665,7 @@ static int launch_pdl(K* kernel, dim3 grid, int threads, size_t smem, void* stre
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return ok_or(cudaLaunchKernelEx(&cfg, kernel, args));
+    return ok_or(cudaLaunchKernelEx(&cfg, kernel, P(args)...));
 }
 
 template <int EPI>
@@ -671,12 +684,13 @@ int launch_gemm(const GemmArgs& a, int epi, int members, void* stream) {
     return (int)cudaErrorInvalidValue;
 }
 
-int launch_wgrad(const WgradArgs& a, int members, void* stream) {
-    if (a.H0 % GM || a.K % GK || a.K <= 0) return (int)cudaErrorInvalidValue;
+int launch_grad(const WgradArgs& w, const RedArgs& r, int members, void* stream) {
+    if (w.H0 % GM || w.K % GK || w.K <= 0 || r.H != kGThreads || r.Bp % 128) return (int)cudaErrorInvalidValue;
     const cudaError_t e =
-        cudaFuncSetAttribute(wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGSmem);
+        cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGSmem);
     if (e != cudaSuccess) return (int)e;
-    return launch_pdl(wgrad_tc_kernel, dim3(a.H0 / GN, a.H0 / GM, 2 * members), kGThreads, kGSmem, stream, a);
+    const int tiles = 2 * members * (w.H0 / GN) * (w.H0 / GM);
+    return launch_pdl(grad_kernel, dim3(tiles + 4 * members * (r.Bp / 128)), kGThreads, kGSmem, stream, w, r, tiles);
 }
 
 int launch_l1(const L1Args& a, int members, void* stream) {
@@ -685,10 +699,6 @@ int launch_l1(const L1Args& a, int members, void* stream) {
 
 int launch_head(const HeadArgs& a, int members, void* stream) {
     return launch_pdl(head_kernel, dim3(a.Bp / 8, members), 256, 0, stream, a);
-}
-
-int launch_reduce_partial(const RedArgs& a, int members, void* stream) {
-    return launch_pdl(reduce_partial_kernel, dim3(a.Bp / 128, members, 16), kRedThreads, 0, stream, a);
 }
 
 int launch_reduce_final(const RedArgs& a, int members, void* stream) {
