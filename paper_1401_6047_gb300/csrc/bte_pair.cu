@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(kPairWarps * 32, 3) pair_kernel(PairArgs A, in
     const uint32_t ring = mine + lane * 16, rot_f = ring + kRing * kRowBytes;
     const uint32_t hrow = mine + kRing * kRowBytes + 3 * 512;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const long long kb = *A.base + 2 * launch_i; /* only the counter kernel moves base */
+    const long long kb = __ldcg(A.base) + 2 * launch_i; /* see step_counter in bte_step.cu */
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
     const int item = (int)blockIdx.x * kPairWarps + warp;

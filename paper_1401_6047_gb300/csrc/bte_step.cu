@@ -155,6 +155,12 @@ __device__ __forceinline__ void diffs(const T (&own)[V], T left, T right, T (&d)
     d[V - 1] = right - own[V - 2];
 }
 
+/* The step counter, which a launch reads before its wait.  Only the counter
+ * kernel moves it, which is complete before the first launch of a run begins;
+ * the later ones of the run begin while the one before them is under way and
+ * so read it from L2, where that kernel's write is, not from an L1 line that
+ * an earlier run may have left. */
+__device__ __forceinline__ long long step_counter(const long long* base) { return __ldcg(base); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -340,7 +346,7 @@ __global__ void __launch_bounds__(MaxBlock<T, V>::value)
     /* new-row buffers: entries outside the tile's columns +-1 stay zero */
     for (int q = tid; q < 4 * WN; q += blockDim.x) sN[q] = (T)0;
     /* only the counter kernel moves base */
-    const long long kbase0 = *(BATCH ? Bt.base : A.base) + launch_i;
+    const long long kbase0 = step_counter(BATCH ? Bt.base : A.base) + launch_i;
     const int cur0 = (parity + launch_i) & 1;
     __syncthreads();
 

@@ -2,7 +2,8 @@
 (programmatic dependent launch): what a kernel reads was written by that
 launch or an earlier one, and is guaranteed to be visible only after the
 kernel's own wait.  Checked on the source of the surrogate's kernels: no load
-helper stands before the wait."""
+helper stands before the wait; and of the step kernels: the step counter,
+which they read before it, comes from L2."""
 import os
 import re
 
@@ -43,3 +44,10 @@ def test_no_load_before_the_wait(kernel):
 
 def test_every_dependent_launch_is_covered():
     assert {"gemm_tc_kernel", "grad_kernel", "l1_kernel", "head_kernel", "adam_kernel"} == set(_launched())
+
+
+@pytest.mark.parametrize("name", ["bte_step.cu", "bte_pair.cu"])
+def test_step_counter_read_before_the_wait_comes_from_l2(name):
+    text = re.sub(r"/\*.*?\*/", "", open(os.path.join(os.path.dirname(SRC), name)).read(), flags=re.S)
+    assert not re.search(r"\*\s*\(?\s*(BATCH \? )?(A|Bt)\.base", text)
+    assert re.search(r"__ldcg\((A\.)?base\)", text)
