@@ -123,10 +123,13 @@ __device__ __forceinline__ double recip<double>(double x) {
 }
 
 /* Arithmetic with exactly one rounding per operation and no contraction
- * left to the compiler (the _rn intrinsics are never fused or reordered).
- * Every kernel that applies the per-cell update -- streamed, persistent,
- * on-chip, start-up -- goes through these, so they all perform the same
- * sequence of roundings and agree bit for bit. */
+ * left to the compiler (the scalar _rn intrinsics are never fused or
+ * reordered).  Every kernel that applies the per-cell update goes through
+ * these, or in FP32 with two or four columns per thread through cn_row's
+ * paired operations; kernels of the same form perform the same sequence of
+ * roundings and agree bit for bit.  The two FP32 forms differ by one rounding
+ * (see cn_row): the one-column form is that of bte_wide.cu, of mode 3 and of
+ * the start-up half step. */
 template <typename T>
 struct Rn;
 template <>
@@ -269,10 +272,15 @@ __device__ __forceinline__ void cn_cell(T a, T b, T X, T Y, T cc, T hr, T g, T t
 /* The update of V consecutive columns of one row (V = 2 or 4): the stencil
  * terms from the other grid's differences in rows n+1 (next) and n-1 (prev),
  * the rotations n w0, n w1 (w = rot_factor at the half-step's start and end;
- * FP64: w0 the sum of the two) and cn_cell.  FP32 runs two columns per instruction with Blackwell's paired
- * FP32 operations (__ffma2_rn, __fadd2_rn, __fmul2_rn), which round each
- * component exactly as the scalar _rn form: the same bits as cn_cell on
- * each column, in half the issue slots.  FP64 runs cn_cell per column. */
+ * FP64: w0 the sum of the two) and cn_cell.  FP32 runs two columns per
+ * instruction with Blackwell's paired FP32 operations (__ffma2_rn, __fadd2_rn,
+ * __fmul2_rn), in half the issue slots: cn_cell's operations, but for the last
+ * ones, a + t / D and b + u / D as one multiply-add each, where cn_cell rounds
+ * the product first.  (Unlike the scalar intrinsics, a paired sum of a paired
+ * product is fused by the compiler where the product has no other use, always
+ * so in 4 million random cases; written out, nothing is left to it.  th + th1,
+ * whose products are used again, it leaves alone: with either of them fused the
+ * results differ.)  FP64 runs cn_cell per column. */
 __device__ __forceinline__ float2 pair(float x, float y) { return make_float2(x, y); }
 __device__ __forceinline__ float2 neg2(float2 v) { return make_float2(-v.x, -v.y); }
 
@@ -307,8 +315,8 @@ __device__ __forceinline__ void cn_row(const T (&a)[V], const T (&b)[V], const T
             float2 u = __ffma2_rn(th1, src, __fmul2_rn(nu, Sb));
             u = __ffma2_rn(A, cb, u);
             u = __ffma2_rn(neg2(Bv), ca, u);
-            const float2 na = __fadd2_rn(A, __fmul2_rn(t, inv));
-            const float2 nb = __fadd2_rn(Bv, __fmul2_rn(u, inv));
+            const float2 na = __ffma2_rn(t, inv, A);
+            const float2 nb = __ffma2_rn(u, inv, Bv);
             an[e] = na.x;
             an[e + 1] = na.y;
             bn[e] = nb.x;

@@ -43,10 +43,9 @@
  * after reading it (blocks read each other's edges in both directions, the
  * corners included), so no reader can find it gone.
  *
- * FP32 cells are updated in column pairs (cn_row), whose products and sums
- * the compiler joins into other multiply-adds than the one-column form's;
- * grid_kernel<float, 1> has the latter's bits, those of bte_wide.cu, for the
- * mode that gives them.
+ * FP32 cells are updated in column pairs (cn_row), whose last sums are
+ * multiply-adds where the one-column form rounds twice; grid_kernel<float, 1>
+ * has the latter's bits, those of bte_wide.cu, for the mode that gives them.
  *
  * Every wait is bounded by %globaltimer.  A wait that gives up sets the
  * launch's quit word, at which every other waiting CTA gives up too, and the
