@@ -1090,8 +1090,9 @@ int enqueue_steps(bte_handle* h, long long n) {
  * enough work, else f(0, 1). */
 template <class F>
 void in_parts(size_t bytes, F f) {
-    const int parts = (int)std::min<size_t>(std::min<size_t>(8, std::max(1u, std::thread::hardware_concurrency())),
-                                            bytes >> 22);
+    /* asked for once: the question costs microseconds, a small grid's copy 30 */
+    static const size_t cpus = std::min<size_t>(8, std::max(1u, std::thread::hardware_concurrency()));
+    const int parts = (int)std::min(cpus, bytes >> 22);
     if (parts < 2) {
         f(0, 1);
         return;
@@ -1135,6 +1136,11 @@ void widen(double* x, size_t n) {
     }
 }
 
+/* cells from which the two arrays of an FP32 grid are widened side by side (a
+ * thread costs about 20 us; both arrays in us, one after the other / so: 201 x
+ * 2001 273 / 200, 401 x 4001 1129 / 708) */
+constexpr size_t kWidenBoth = 200000;
+
 /* Both arrays of one grid: FP64 straight into the caller's arrays, FP32 into
  * their second halves and widened there. */
 template <typename T>
@@ -1158,9 +1164,18 @@ int get_grid(bte_handle* h, int grid, double* a, double* b) {
                              h->stream));
     }
     CU(cudaStreamSynchronize(h->stream));
-    if (sizeof(T) == 4)
-        for (double* d : dst)
-            if (d) widen(d, n);
+    if (sizeof(T) == 4) {
+        std::thread other; /* the second array beside the first */
+        if (a && b && n >= kWidenBoth) {
+            try {
+                other = std::thread(widen, b, n);
+            } catch (...) { /* no thread to be had */
+            }
+        }
+        if (a) widen(a, n);
+        if (other.joinable()) other.join();
+        else if (b) widen(b, n);
+    }
     return BTE_OK;
 }
 

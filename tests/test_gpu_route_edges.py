@@ -188,3 +188,24 @@ def test_tuned_options_are_no_slower_than_none():
     best, secs = bte.batch_tune(pts, sample=6, steps=400)
     assert secs.argmin() == 0 and best["resident"] == 0
     assert _seconds(pts, **best) < 1.3 * _seconds(pts)
+
+
+# few cells and many, an odd number of them, the two arrays of an FP32 grid
+# widened one after the other and side by side, in one stretch and in several
+@pytest.mark.parametrize("shape", [(1, 3), (2, 21), (30, 201), (398, 501), (399, 501), (1000, 2101)])
+@pytest.mark.parametrize("prec", [W.FP64, W.FP32_MIXED])
+def test_state_comes_back_as_it_was_set(shape, prec):
+    p = _params(*shape, prec)
+    st = W.random_state(p, seed=5)
+    if prec == W.FP32_MIXED:
+        st = [x.astype(np.float32).astype(np.float64) for x in st]
+    with bte.Solver(p) as s:
+        s.set_state(0, st[0], st[1])
+        s.set_state(1, st[2], st[3])
+        assert _equal(_state(s), st)
+        for which in (0, 1):  # one array of a grid alone
+            x = np.zeros(s.shape)
+            args = [None, None]
+            args[which] = bte._dp(x)
+            bte._check(bte.lib().bte_get_state(s._h, 1, *args))
+            assert np.array_equal(x, st[2 + which])
