@@ -176,10 +176,8 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs<T> A) 
     const int C = A.C;
     double* acc = reinterpret_cast<double*>(smem + A.red_off); /* [6] window sums, [4] rotation */
     int* s_next = reinterpret_cast<int*>(acc + 10);
-    /* the last warp of every CTA holds no cell; rank 0's adds the row sums */
-    const int tid = threadIdx.x, nthr = (int)blockDim.x - 32;
-    const int lane = tid & 31;
-    const bool comp = tid < nthr, observer = rank == 0 && !comp;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const bool observer = rank == 0 && tid >= (int)blockDim.x - 32; /* adds the row sums */
 
     for (;;) {
         if (rank == 0 && tid == 0) *s_next = (int)atomicAdd(A.queue, 1u);
@@ -257,16 +255,34 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs<T> A) 
          * thread runs the same number of iterations (the differences use
          * warp shuffles); iterations past row R-2 read clamped rows and store
          * nothing. */
+        const int nint = R > 2 ? R - 2 : 0;
+        /* boundary rows 0 and R-1 (one row when R == 1) */
+        const int nbnd = R >= 2 ? 2 : R;
+        /* The last warp holds no cell, so that no cell waits for the row sums
+         * -- unless the column groups just fill all the threads: without that
+         * warp's 32 a point of 241 to 256 groups has one row block where it had
+         * two, one of 481 to 512 walks its rows twice.  Compared are the rows
+         * that a thread walks in a half-step, in FP64 (where a row of the CTA
+         * takes some 13000 cycles) with the passes over the boundary rows; in
+         * FP32 a row takes about 1100 cycles and the sums cost rank 0 2800 per
+         * step.  Measured (40 points, ms, all threads / without the last warp):
+         * FP64 61 x 501 110 / 167, 101 x 170 75 / 84, FP32 61 x 1001 16.1 / 18.4,
+         * 101 x 641 16.0 / 17.4, 61 x 2001 33.2 / 36.5; 41 x 2001, one row more
+         * to walk, 30.2 / 29.6. */
+        auto walk = [&](int n) {
+            const int c = min(ncg, n), split = n / c;
+            return (ncg + c - 1) / c * ((nint + split - 1) / split) + (sizeof(T) == 8 ? (nbnd * ncg + n - 1) / n : 0);
+        };
+        const int nall = (int)blockDim.x;
+        const int nthr = walk(nall) + (rank == 0 && sizeof(T) == 4 ? 1 : 0) < walk(nall - 32) ? nall : nall - 32;
+        const bool comp = tid < nthr;
         const int cpp = min(ncg, nthr);
         const int rsplit = nthr / cpp;
         const int gl = tid % cpp, rp = tid / cpp;
         const bool t_on = rp < rsplit;
         const int npass = (ncg + cpp - 1) / cpp;
-        const int nint = R > 2 ? R - 2 : 0;
         const int nrow = (nint + rsplit - 1) / rsplit;
         const int lo = 1 + rp * nrow;
-        /* boundary rows 0 and R-1 (one row when R == 1) */
-        const int nbnd = R >= 2 ? 2 : R;
 
         /* one half-step on the rows of this CTA: own grid (o) updated in place
          * from the other grid (x) */
@@ -350,7 +366,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs<T> A) 
             }
         };
 
-        /* The observer adds the new whole grid's rows 0 (a) and 1 (b) while
+        /* The observer, a warp, adds the new whole grid's rows 0 (a) and 1 (b) while
          * the fractional half-step, which leaves them unchanged, runs, and
          * folds them into the window sums: some 50 FP64 operations in a row,
          * each about 64 cycles of a quarter of an SM, that no other warp
@@ -447,8 +463,8 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(ResArgs<T> A) 
             __syncthreads();
             cluster_arrive();
             /* ---- fractional grid: z_f^{k+3/2} = T(z_f^{k+1/2}; S(z_w^{k+1})) ---- */
+            if (observer) observe(k + 1);
             if (comp) half_interior(2, 0, Df);
-            else if (observer) observe(k + 1);
             cluster_wait();
             if (comp) half_boundary(2, 0, Df);
             __syncthreads();

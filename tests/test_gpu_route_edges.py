@@ -209,3 +209,24 @@ def test_state_comes_back_as_it_was_set(shape, prec):
             args[which] = bte._dp(x)
             bte._check(bte.lib().bte_get_state(s._h, 1, *args))
             assert np.array_equal(x, st[2 + which])
+
+
+# points on chip whose column groups (2 columns in FP64, 4 in FP32) need the
+# last warp's threads for another row block or to be walked once: on, just
+# below and just above each edge, with few rows per CTA and many
+@pytest.mark.parametrize("groups", [96, 97, 160, 161, 170, 171, 240, 241, 256, 257, 480, 481, 512, 513])
+@pytest.mark.parametrize("n_max", [4, 24])
+@pytest.mark.parametrize("prec", [W.FP64, W.FP32_MIXED])
+def test_on_chip_points_at_the_edges_of_the_thread_split(groups, n_max, prec):
+    """Against lock-step launches; FP32 states are equal, their sums added in
+    FP32 pairs (1e-7 of the norm, 2e-6 of the drift)."""
+    V = 2 if prec == W.FP64 else 4
+    pts = [_params(n_max, groups * V - k, prec).replace(periods=0.06, avg_window=0.05) for k in (0, 1)]
+    fits = bte.batch_plan(pts).all()
+    if not fits:
+        pytest.skip("does not fit a cluster")
+    for o, r in zip(bte.batch_run(pts, resident_smem=232448), bte.batch_run(pts, resident=1)):
+        assert o.status == r.status == bte.OK
+        for k in ("v_dr", "norm", "v_dc_avg", "absorption"):
+            x, y = getattr(o, k), getattr(r, k)
+            assert abs(x - y) <= (1e-12 * max(abs(y), 1e-3) if prec == W.FP64 else 1e-7 if k == "norm" else 2e-6)
