@@ -20,8 +20,8 @@
  * exchange of edges per half-step, about 0.5 us through L2.
  *
  * Measured (GB300, us per step, one launch per step / here): 31 x 201 FP64
- * 23.0 / 2.6, FP32 9.3 / 2.1; 65 x 1000 FP64 45 / 7.9; 138 x 1533 FP32 14.4 /
- * 3.3; 120 x 4000 FP32 13.9 / 3.9; 401 x 4001 FP32 17.0 / 7.2.  (With the
+ * 22.7 / 2.6, FP32 9.6 / 2.0; 65 x 1000 FP64 43 / 8.1; 138 x 1533 FP32 14.5 /
+ * 3.2; 120 x 4000 FP32 13.9 / 3.8; 401 x 4001 FP32 17.0 / 7.2.  (With the
  * compute threads polling: 3.9, 2.5, 9.4, 3.6, 4.5 and 7.5.)
  *
  * A half-step of a CTA (its last 128 threads only poll, keep rows 0 and 1 and
@@ -52,7 +52,8 @@
  * error word that the host reports as BTE_ETIMEOUT.
  *
  * Rows 0 (a) and 1 (b) of each new whole grid are copied to a buffer, and
- * fold_rows_kernel adds them afterwards in exactly the order of the one
+ * fold_rows_kernel (wide rows: fold_tiles_kernel and fold_tail_kernel) adds
+ * them afterwards in exactly the order of the one
  * launch per step kernel (V columns per lane, a 32-lane tree, the warps of a
  * tile in order, tiles in order), so the drift velocity and norm (Eqs.
  * v_dr_generic, norm_in_phi) of a step are the same bits whichever kernel

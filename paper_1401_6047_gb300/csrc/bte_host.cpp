@@ -234,8 +234,8 @@ constexpr int kPairMinRows = 8, kPairMaxRows = 192;
  * the part of a boundary cell that waits (550 with two lanes per cell).
  * Measured on a GB300 (us per step, this choice / best of a sweep of 14 row
  * splits, both widths, 64 to 512 threads and 0 to 128 polling ones): 31 x 201
- * FP64 2.6 / 2.6, FP32 2.1 / 2.0; 65 x 1000 FP64 8.2 / 7.9, FP32 2.3 / 2.3;
- * 120 x 4000 FP64 39.4 / 39.4, FP32 3.9 / 3.8; 138 x 1533 FP32 3.3 / 3.1;
+ * FP64 2.6 / 2.6, FP32 2.0 / 2.0; 65 x 1000 FP64 8.1 / 7.9, FP32 2.3 / 2.3;
+ * 120 x 4000 FP64 39.4 / 39.4, FP32 3.8 / 3.8; 138 x 1533 FP32 3.2 / 3.1;
  * 401 x 4001 FP32 7.2 / 7.2.  False when no split fits the shared memory. */
 constexpr int kBlkHelp = 128; /* polling threads */
 bool pick_blocks(int N1, int M1, size_t elem, bool scalar, Layout& L) {

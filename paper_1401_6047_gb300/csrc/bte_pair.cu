@@ -34,8 +34,10 @@
  * general one, which costs twice as much.
  *
  * Measured (GB300, us per step, one launch per step / here): 2049 x 8193
- * 93.2 / 58.9; 701 x 5000 27.3 / 16.1; 1024 x 2400 21.6 / 13.5; 1000 x 2503
- * 20.9 / 14.6; 20 x 120001 56.3 / 35.7.
+ * 93.2 / 58.8; 701 x 5000 27.3 / 15.3; 1024 x 2400 21.6 / 11.8; 1000 x 2503
+ * 20.9 / 13.0; 20 x 120001 56.3 / 18.1; few rows, nearly all of whose
+ * iterations are general: 16 x 200000 62 / 20, 8 x 350000 77 / 29, 4 x 390000
+ * 78 / 25.
  *
  * Where the state is larger than L2, launches walk the rows upward and
  * downward in turn, as in bte_step.cu (DOWN, the mirror image).  The cells'
