@@ -1005,7 +1005,10 @@ int queue_pairs(bte_handle* h, int launches, int set, cudaStream_t st) {
 /* whether the caller is capturing the handle's stream into a graph */
 bool capturing(const bte_handle* h) {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess) cudaGetLastError();
+    if (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess) {
+        cudaGetLastError(); /* the legacy stream beside another one's capture: the launches will say so */
+        return false;
+    }
     return st == cudaStreamCaptureStatusActive;
 }
 
