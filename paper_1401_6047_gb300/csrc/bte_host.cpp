@@ -1754,18 +1754,20 @@ double alone_us(const bte_params& p, const TimeGrid& tg) {
     return L.elem == 4 ? 4.0 + 3.4e-6 * cells * (p.n_max + 13) / (p.n_max + 1) : 12.0 + 1e-4 * cells;
 }
 
-/* Time of all steps of the streamed points `pts` (longest runs first) in
- * lock-step batches, in us: a step takes as many waves of tiles as the items
- * fill the GPU's `slots` CTAs, and a wave as long as its tiles have rows.
- * Measured (GB300, chunks of 16): FP32 22 us for tiles of 10 rows and 29 for
- * 16, a fifth more each where there are several waves, which then mix the
- * tiles of full and of fewer rows (21 x 6001, 32 points: 80 us, 81 with the
+/* Time in us of one wave of lock-step tiles of so many rows, and of one of
+ * several.  Measured (GB300, chunks of 16): FP32 22 us for tiles of 10 rows and
+ * 29 for 16, a fifth more each where there are several waves, which then mix
+ * the tiles of full and of fewer rows (21 x 6001, 32 points: 80 us, 81 with the
  * mean rows of a tile); FP64 92 and 145, where they do not (21 x 2001, 32
  * points: 284 us, 290 with full tiles). */
 double wave_us(const BatchCfg& c, double rows) { return c.fp64 ? 3.7 + 8.83 * rows : 10.5 + 1.15 * rows; }
 double several_waves_us(const BatchPoint& b, const BatchCfg& c) {
     return c.fp64 ? wave_us(c, std::min(b.N1, c.chunk)) : 1.2 * wave_us(c, (double)b.N1 / b.nty);
 }
+
+/* Time of all steps of the streamed points `pts` (longest runs first) in
+ * lock-step batches, in us: a step takes as many waves of tiles as the items
+ * fill the GPU's `slots` CTAs. */
 double lock_step_us(const std::vector<BatchPoint>& pts, const BatchCfg& c, int slots) {
     double total = 0.0;
     for (size_t first = 0; first < pts.size();) {
